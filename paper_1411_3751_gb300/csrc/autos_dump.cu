@@ -84,6 +84,51 @@ __global__ void __launch_bounds__(AW * 32) autos_kernel(const uint8_t* __restric
 // offset domain (u = x + 8 + 8i) and are mapped back here:
 //   V = Vu - (8 - 8i) s_a - (8 + 8i) conj(s_c) + 128 T_off,   A = Au - 16 (Re s + Im s) + 128 T_off
 // (s = per-input offset sums and T_off = samples accumulated through that path, per cadence).
+
+// float((double)v / (double)n), the definition of CF32_NORM.
+__device__ __forceinline__ float norm_exact(long long v, long long n) {
+  return n > 0 ? __double2float_rn(__ddiv_rn(__ll2double_rn(v), (double)n)) : 0.f;
+}
+
+// The same value without FP64 arithmetic (a GB300 SM does about 2 FP64 operations per clock: with the
+// FP64 division the 109-channel, 512-input normalised dump took 553 us, eight times its HBM time): v
+// and 1 / n as sums of two floats, the product to about 2^-46 relative. If adding +-2^-44 to it does
+// not change the rounded float, that float is the rounded exact quotient (and so the one the double
+// division rounds to, whose error is 2^-53); else, about one value in 2^18, divide as defined.
+__device__ __forceinline__ float norm_fast(long long v, long long n, float rh, float rl) {
+  const float hi = __ll2float_rn(v);
+  const float lo = __ll2float_rn(v - __float2ll_rn(hi));
+  const float p = __fmul_rn(hi, rh);
+  const float e = __fmaf_rn(lo, rh, __fmaf_rn(hi, rl, __fmaf_rn(hi, rh, -p)));
+  const float d = __fmul_rn(fabsf(p), 5.6843418860808015e-14f);  // 2^-44
+  const float q1 = __fadd_rn(p, __fadd_rn(e, d)), q2 = __fadd_rn(p, __fsub_rn(e, d));
+  return q1 == q2 ? q1 : norm_exact(v, n);
+}
+
+// Sample count of a normalised dump: n for every cell with rh + rl = 1 / n, or (cells reset
+// selectively) n - base[...] each.
+struct DumpNorm {
+  long long n;
+  float rh, rl;
+};
+
+DumpNorm dump_norm(long long n) {
+  const double inv = n > 0 ? 1.0 / (double)n : 0.0;
+  DumpNorm d;
+  d.n = n;
+  d.rh = (float)inv;
+  d.rl = (float)(inv - (double)d.rh);
+  return d;
+}
+
+// One value in format FMT (CI64: long long, else float); ns = the cell's own count if HAS_BASE.
+template <bool HAS_BASE>
+__device__ __forceinline__ float as_float(long long v, int fmt, const DumpNorm& dn, long long ns) {
+  if (fmt == CORR_FMT_CF32) return __ll2float_rn(v);
+  if (HAS_BASE) return norm_exact(v, ns);
+  return dn.n > 0 ? norm_fast(v, dn.n, dn.rh, dn.rl) : 0.f;
+}
+
 template <typename T>
 __device__ __forceinline__ void put(void* out, long long k, long long v, int fmt, long long n_samples) {
   if (fmt == CORR_FMT_CI64) {
@@ -91,17 +136,18 @@ __device__ __forceinline__ void put(void* out, long long k, long long v, int fmt
   } else if (fmt == CORR_FMT_CF32) {
     static_cast<float*>(out)[k] = __ll2float_rn(v);
   } else {
-    static_cast<float*>(out)[k] = n_samples > 0 ? __double2float_rn(__ddiv_rn(__ll2double_rn(v), (double)n_samples)) : 0.f;
+    static_cast<float*>(out)[k] = norm_exact(v, n_samples);
   }
 }
 
-// station pair index b -> (a, c) with b = a (a + 1) / 2 + c, a >= c
+// station pair index b -> (a, c) with b = a (a + 1) / 2 + c, a >= c; b < 2^31 - 2^15 (a <= 65534), so
+// that (a + 1) (a + 2) < 2^32
 __device__ __forceinline__ void pair_of(int b, int& sa, int& sc) {
-  int a = (int)((sqrtf(8.0f * (float)b + 1.0f) - 1.0f) * 0.5f);
-  while ((long long)a * (a + 1) / 2 > b) --a;
-  while ((long long)(a + 1) * (a + 2) / 2 <= b) ++a;
-  sa = a;
-  sc = b - (int)((long long)a * (a + 1) / 2);
+  unsigned a = (unsigned)((sqrtf(8.0f * (float)b + 1.0f) - 1.0f) * 0.5f);
+  while (a * (a + 1) / 2 > (unsigned)b) --a;
+  while ((a + 1) * (a + 2) / 2 <= (unsigned)b) ++a;
+  sa = (int)a;
+  sc = b - (int)(a * (a + 1) / 2);
 }
 
 // Corrected value of cross cell `cell` (= f * B_s * P + b * P + pidx) from its raw int64 sums.
@@ -131,31 +177,124 @@ __device__ __forceinline__ long long auto_value(const long long* __restrict__ ac
   return v;
 }
 
-// Cross dump of cells [cell0, cell0 + n_cells) (a cell = one (re, im) pair), output indexed from 0.
-__global__ void dump_cross_kernel(const long long* __restrict__ acc, long long cell0, long long n_cells,
-                                  void* __restrict__ out, int fmt, long long n_samples, Shape2 g) {
-  const long long cpc = g.Bs * g.P;  // cells per channel
-  const int lp = g.P == 4 ? 2 : 0;
-  for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < n_cells; k += (long long)gridDim.x * blockDim.x) {
-    const long long cell = cell0 + k;
-    const long long f = cell / cpc;
-    const int r = (int)(cell - f * cpc);
-    const int b = r >> lp, pidx = r & (g.P - 1);
-    long long re, im;
-    cross_value(acc, cell, f, b, pidx, g, re, im);
-    const long long ns = g.base ? n_samples - g.base[b] : n_samples;
-    put<void>(out, 2 * k, re, fmt, ns);
-    put<void>(out, 2 * k + 1, im, fmt, ns);
+// NPOL neighbouring cells (16 bytes each) as one access: at NPOL = 2 the 256-bit forms, a whole 32-byte
+// sector a thread. (Two 16-byte stores a thread write half sectors, which the L2 has to merge: the
+// 200-input, 300-channel float dump took 205 us so, latency-bound at 0.9 TB/s.)
+template <int NPOL>
+__device__ __forceinline__ void load_cells(const longlong2* p, longlong2 (&v)[NPOL]) {
+  if constexpr (NPOL == 2)
+    asm volatile("ld.global.v4.b64 {%0, %1, %2, %3}, [%4];"
+                 : "=l"(v[0].x), "=l"(v[0].y), "=l"(v[1].x), "=l"(v[1].y)
+                 : "l"(p)
+                 : "memory");
+  else
+    v[0] = *p;
+}
+template <int NPOL>
+__device__ __forceinline__ void store_cells(longlong2* p, const longlong2 (&v)[NPOL]) {
+  if constexpr (NPOL == 2)
+    asm volatile("st.global.v4.b64 [%0], {%1, %2, %3, %4};" ::"l"(p), "l"(v[0].x), "l"(v[0].y), "l"(v[1].x), "l"(v[1].y)
+                 : "memory");
+  else
+    *p = v[0];
+}
+
+// Cross dump. A thread takes a unit = the NPOL products of one station pair and a-polarisation, i.e.
+// NPOL neighbouring cells (one s_a and NPOL neighbouring s_c serve them; NPOL = 2: 32 bytes in, 32 or
+// 16 out). blockIdx.y is the channel f0 + blockIdx.y, whose units are divided over gridDim.x blocks;
+// [u0, u1) are the units dumped, numbered over all channels, the output indexed from u0 (vec: a unit's
+// values leave in one store, the output is aligned to that). With ZERO the
+// dumped cells restart from zero in the same pass (a separate memset wrote them once more and cost
+// its launch), and if zero_soff the block, alone on its channel, zeroes the channel's offset sums too.
+constexpr int DUMP_NT = 256;
+
+template <int NPOL, bool ZERO, bool HAS_BASE>
+__global__ void __launch_bounds__(DUMP_NT) dump_cross_kernel(long long* __restrict__ acc, long long u0, long long u1,
+                                                             long long f0, void* __restrict__ out, int fmt, DumpNorm dn,
+                                                             bool vec, Shape2 g, long long* zero_soff) {
+  const long long f = f0 + blockIdx.y;
+  const long long upc = g.Bs * NPOL;  // units per channel
+  const long long first = f * upc;
+  const unsigned r_begin = (unsigned)(u0 > first ? u0 - first : 0);
+  const unsigned r_end = (unsigned)(u1 - first < upc ? u1 - first : upc);
+  const bool corr = g.soff != nullptr && g.t_off != 0;
+  const longlong2* s = reinterpret_cast<const longlong2*>(g.soff) + f * g.N;
+  for (unsigned r = r_begin + blockIdx.x * DUMP_NT + threadIdx.x; r < r_end; r += gridDim.x * DUMP_NT) {
+    const int b = (int)(NPOL == 2 ? r >> 1 : r);
+    longlong2* cell = reinterpret_cast<longlong2*>(acc) + (first + r) * NPOL;
+    longlong2 v[NPOL];
+    load_cells<NPOL>(cell, v);
+    if (corr) {
+      int sa, sc;
+      pair_of(b, sa, sc);
+      const longlong2 s_a = s[NPOL * sa + (NPOL == 2 ? (int)(r & 1) : 0)];
+#pragma unroll
+      for (int q = 0; q < NPOL; ++q) {
+        const longlong2 s_c = s[NPOL * sc + q];
+        v[q].x += 128 * g.t_off - 8 * (s_a.x + s_a.y + s_c.x + s_c.y);
+        v[q].y -= 8 * (s_a.y - s_a.x + s_c.x - s_c.y);
+      }
+    }
+    const long long o = (first + r - u0) * NPOL;
+    if (fmt == CORR_FMT_CI64) {
+      if (vec) {
+        store_cells<NPOL>(static_cast<longlong2*>(out) + o, v);
+      } else {
+#pragma unroll
+        for (int q = 0; q < NPOL; ++q) {
+          static_cast<long long*>(out)[2 * (o + q)] = v[q].x;
+          static_cast<long long*>(out)[2 * (o + q) + 1] = v[q].y;
+        }
+      }
+    } else {
+      const long long ns = HAS_BASE ? dn.n - g.base[b] : dn.n;
+      float w[2 * NPOL];
+#pragma unroll
+      for (int q = 0; q < NPOL; ++q) {
+        w[2 * q] = as_float<HAS_BASE>(v[q].x, fmt, dn, ns);
+        w[2 * q + 1] = as_float<HAS_BASE>(v[q].y, fmt, dn, ns);
+      }
+      if (!vec) {
+#pragma unroll
+        for (int q = 0; q < 2 * NPOL; ++q) static_cast<float*>(out)[2 * o + q] = w[q];
+      } else if constexpr (NPOL == 2) {
+        *reinterpret_cast<float4*>(static_cast<float*>(out) + 2 * o) = make_float4(w[0], w[1], w[2], w[3]);
+      } else {
+        *reinterpret_cast<float2*>(static_cast<float*>(out) + 2 * o) = make_float2(w[0], w[1]);
+      }
+    }
+    if (ZERO) {
+      // last, when the cells have arrived: zeroes stored behind loads still in flight made the pass
+      // latency-bound (205 us instead of 40 at 200 inputs x 300 channels)
+      longlong2 z[NPOL];
+#pragma unroll
+      for (int q = 0; q < NPOL; ++q) z[q] = make_longlong2(0, 0);
+      store_cells<NPOL>(cell, z);
+    }
+  }
+  if (ZERO && zero_soff) {
+    __syncthreads();  // every thread has read the sums
+    longlong2* z = reinterpret_cast<longlong2*>(zero_soff) + f * g.N;
+    for (int i = threadIdx.x; i < g.N; i += DUMP_NT) z[i] = make_longlong2(0, 0);
   }
 }
 
-// Autos dump of elements [k0, k0 + n).
-__global__ void dump_autos_kernel(const long long* __restrict__ acc, long long k0, long long n, void* __restrict__ out,
-                                  int fmt, long long n_samples, Shape2 g) {
+// Autos dump of elements [k0, k0 + n); with zero_soff (the offset sums of g) the dumped inputs' sums and
+// offset sums restart from zero.
+__global__ void dump_autos_kernel(long long* __restrict__ acc, long long k0, long long n, void* __restrict__ out,
+                                  int fmt, DumpNorm dn, Shape2 g, long long* zero_soff) {
   for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < n; k += (long long)gridDim.x * blockDim.x) {
     const long long v = auto_value(acc, k0 + k, g);
-    const long long ns = g.base ? n_samples - g.base[(k0 + k) % g.N] : n_samples;
-    put<void>(out, k, v, fmt, ns);
+    if (fmt == CORR_FMT_CI64)
+      static_cast<long long*>(out)[k] = v;
+    else if (g.base)
+      static_cast<float*>(out)[k] = as_float<true>(v, fmt, dn, dn.n - g.base[(k0 + k) % g.N]);
+    else
+      static_cast<float*>(out)[k] = as_float<false>(v, fmt, dn, dn.n);
+    if (zero_soff) {
+      acc[k0 + k] = 0;
+      reinterpret_cast<longlong2*>(zero_soff)[k0 + k] = make_longlong2(0, 0);
+    }
   }
 }
 
@@ -254,16 +393,45 @@ cudaError_t launch_set_base(long long* d_base, const int* d_st, int n_st, long l
   return cudaGetLastError();
 }
 
-cudaError_t launch_dump(const long long* d_acc, long long n_elems, void* d_out, int fmt, long long n_samples,
-                        long long k_base, const Shape2& g, cudaStream_t st) {
+cudaError_t launch_dump(long long* d_acc, long long n_elems, void* d_out, int fmt, long long n_samples, long long k_base,
+                        const Shape2& g, long long* zero_soff, bool zero, bool* soff_zeroed, cudaStream_t st) {
+  *soff_zeroed = false;
   if (n_elems == 0) return cudaSuccess;
-  const long long n_units = g.autos ? n_elems : n_elems / 2;
-  long long blocks = (n_units + 255) / 256;
-  if (blocks > (long long)sm_count() * 32) blocks = (long long)sm_count() * 32;
-  if (g.autos)
-    dump_autos_kernel<<<(unsigned)blocks, 256, 0, st>>>(d_acc, k_base, n_elems, d_out, fmt, n_samples, g);
-  else
-    dump_cross_kernel<<<(unsigned)blocks, 256, 0, st>>>(d_acc, k_base / 2, n_elems / 2, d_out, fmt, n_samples, g);
+  const DumpNorm dn = dump_norm(n_samples);
+  if (g.autos) {
+    long long blocks = (n_elems + 255) / 256;
+    if (blocks > (long long)sm_count() * 32) blocks = (long long)sm_count() * 32;
+    dump_autos_kernel<<<(unsigned)blocks, 256, 0, st>>>(d_acc, k_base, n_elems, d_out, fmt, dn, g, zero ? zero_soff : nullptr);
+    *soff_zeroed = zero;
+    return cudaGetLastError();
+  }
+  const long long upc = g.Bs * g.npol, u0 = k_base / 2 / g.npol, u1 = u0 + n_elems / 2 / g.npol;
+  const long long f0 = u0 / upc, f1 = (u1 - 1) / upc;
+  // blocks per channel: one (which may then zero the channel's offset sums) up to 16 units a thread,
+  // else 4 units a thread
+  const bool whole = upc <= 16 * DUMP_NT;
+  const long long bx = whole ? 1 : (upc + 4 * DUMP_NT - 1) / (4 * DUMP_NT);
+  const dim3 grid((unsigned)bx, (unsigned)(f1 - f0 + 1));
+  const bool zs = zero && whole && u0 == f0 * upc && u1 == (f1 + 1) * upc;
+  long long* z = zs ? zero_soff : nullptr;
+  *soff_zeroed = zs;
+  const bool base = g.base != nullptr;
+  const bool vec = reinterpret_cast<uintptr_t>(d_out) % ((fmt == CORR_FMT_CI64 ? 16 : 8) * g.npol) == 0;
+#define DUMP_CROSS(NP, ZE, BA) dump_cross_kernel<NP, ZE, BA><<<grid, DUMP_NT, 0, st>>>(d_acc, u0, u1, f0, d_out, fmt, dn, vec, g, z)
+  if (g.npol == 2) {
+    if (zero) {
+      if (base) DUMP_CROSS(2, true, true); else DUMP_CROSS(2, true, false);
+    } else {
+      if (base) DUMP_CROSS(2, false, true); else DUMP_CROSS(2, false, false);
+    }
+  } else {
+    if (zero) {
+      if (base) DUMP_CROSS(1, true, true); else DUMP_CROSS(1, true, false);
+    } else {
+      if (base) DUMP_CROSS(1, false, true); else DUMP_CROSS(1, false, false);
+    }
+  }
+#undef DUMP_CROSS
   return cudaGetLastError();
 }
 

@@ -575,6 +575,30 @@ int accumulate_batch_chunks(corr_ctx* c, const uint8_t* const* blocks, int n, cu
   return CORR_OK;
 }
 
+// Restart the selected integrations: zero the per-cell counts and, where not yet done, the sums (`cells`)
+// and the offset sums (`offsets`).
+int restart(corr_ctx* c, int what, bool cells, bool offsets, cudaStream_t st) {
+  if (what & CORR_WHAT_CROSS) {
+    cudaError_t e = cudaSuccess;
+    if (cells) e = cudaMemsetAsync(c->d_cross, 0, (size_t)c->L.cross_elems * 8, st);
+    if (e == cudaSuccess && offsets) e = cudaMemsetAsync(c->d_soff, 0, (size_t)c->L.autos_elems * 16, st);
+    if (e == cudaSuccess && c->d_cross_base) e = cudaMemsetAsync(c->d_cross_base, 0, (size_t)c->L.s.Bs * 8, st);
+    if (e != cudaSuccess) return cuda_fail(e, "corr_reset");
+    c->n_cross = 0;
+    c->n_off = 0;
+  }
+  if (what & CORR_WHAT_AUTO) {
+    cudaError_t e = cudaSuccess;
+    if (cells) e = cudaMemsetAsync(c->d_autos, 0, (size_t)c->L.autos_elems * 8, st);
+    if (e == cudaSuccess && offsets) e = cudaMemsetAsync(c->d_soff_auto, 0, (size_t)c->L.autos_elems * 16, st);
+    if (e == cudaSuccess && c->d_auto_base) e = cudaMemsetAsync(c->d_auto_base, 0, (size_t)c->L.s.N * 8, st);
+    if (e != cudaSuccess) return cuda_fail(e, "corr_reset");
+    c->n_auto = 0;
+    c->n_off_auto = 0;
+  }
+  return CORR_OK;
+}
+
 }  // namespace host
 }  // namespace corr
 
@@ -1004,24 +1028,7 @@ int corr_accumulate_autos(corr_ctx* c, const void* d_samples, void* stream) {
 int corr_reset(corr_ctx* c, int what, void* stream) {
   if (!c) return fail(CORR_ERR_ARG, "corr_reset: NULL context");
   if (what < 1 || what > 3) return fail(CORR_ERR_ARG, "corr_reset: what must be CROSS, AUTO or both");
-  cudaStream_t st = (cudaStream_t)stream;
-  if (what & CORR_WHAT_CROSS) {
-    cudaError_t e = cudaMemsetAsync(c->d_cross, 0, (size_t)c->L.cross_elems * 8, st);
-    if (e == cudaSuccess) e = cudaMemsetAsync(c->d_soff, 0, (size_t)c->L.autos_elems * 16, st);
-    if (e == cudaSuccess && c->d_cross_base) e = cudaMemsetAsync(c->d_cross_base, 0, (size_t)c->L.s.Bs * 8, st);
-    if (e != cudaSuccess) return cuda_fail(e, "corr_reset");
-    c->n_cross = 0;
-    c->n_off = 0;
-  }
-  if (what & CORR_WHAT_AUTO) {
-    cudaError_t e = cudaMemsetAsync(c->d_autos, 0, (size_t)c->L.autos_elems * 8, st);
-    if (e == cudaSuccess) e = cudaMemsetAsync(c->d_soff_auto, 0, (size_t)c->L.autos_elems * 16, st);
-    if (e == cudaSuccess && c->d_auto_base) e = cudaMemsetAsync(c->d_auto_base, 0, (size_t)c->L.s.N * 8, st);
-    if (e != cudaSuccess) return cuda_fail(e, "corr_reset");
-    c->n_auto = 0;
-    c->n_off_auto = 0;
-  }
-  return CORR_OK;
+  return restart(c, what, true, true, (cudaStream_t)stream);
 }
 
 int corr_dump(corr_ctx* c, void* out, int is_device_ptr, int what, int fmt, int reset, void* stream) {
@@ -1031,7 +1038,8 @@ int corr_dump(corr_ctx* c, void* out, int is_device_ptr, int what, int fmt, int 
   if (fmt != CORR_FMT_CI64 && fmt != CORR_FMT_CF32 && fmt != CORR_FMT_CF32_NORM)
     return fail(CORR_ERR_ARG, "corr_dump: unknown format");
   cudaStream_t st = (cudaStream_t)stream;
-  const long long* acc = what == CORR_WHAT_CROSS ? c->d_cross : c->d_autos;
+  long long* acc = what == CORR_WHAT_CROSS ? c->d_cross : c->d_autos;
+  long long* soff = what == CORR_WHAT_CROSS ? c->d_soff : c->d_soff_auto;
   const long long n = what == CORR_WHAT_CROSS ? c->L.cross_elems : c->L.autos_elems;
   const long long ns = what == CORR_WHAT_CROSS ? c->n_cross : c->n_auto;
   const size_t esz = fmt == CORR_FMT_CI64 ? 8 : 4;
@@ -1040,14 +1048,17 @@ int corr_dump(corr_ctx* c, void* out, int is_device_ptr, int what, int fmt, int 
   g.npol = c->L.s.npol;
   g.P = c->L.s.P;
   g.Bs = c->L.s.Bs;
-  g.soff = what == CORR_WHAT_CROSS ? c->d_soff : c->d_soff_auto;
+  g.soff = soff;
   g.t_off = what == CORR_WHAT_CROSS ? c->n_off : c->n_off_auto;
   g.autos = what == CORR_WHAT_AUTO ? 1 : 0;
   g.base = what == CORR_WHAT_CROSS ? c->d_cross_base : c->d_auto_base;
   cudaError_t e;
+  // a device dump with reset zeroes the cells as it dumps them, and the offset sums where it can; a host
+  // dump (whose copies may still fail) is restarted after its last chunk
+  bool soff_zeroed = false;
   if (is_device_ptr) {
     const bool tb = timer_begin(c, CORR_KERNEL_DUMP, st);
-    e = launch_dump(acc, n, out, fmt, ns, 0, g, st);
+    e = launch_dump(acc, n, out, fmt, ns, 0, g, soff, reset != 0, &soff_zeroed, st);
     timer_end(c, CORR_KERNEL_DUMP, st, tb);
     if (e != cudaSuccess) return cuda_fail(e, "corr_dump: launch");
   } else {
@@ -1056,7 +1067,7 @@ int corr_dump(corr_ctx* c, void* out, int is_device_ptr, int what, int fmt, int 
     for (long long k = 0; k < n; k += per) {
       const long long m = (n - k) < per ? (n - k) : per;
       const bool tb = timer_begin(c, CORR_KERNEL_DUMP, st);
-      e = launch_dump(acc, m, c->d_stage[buf], fmt, ns, k, g, st);
+      e = launch_dump(acc, m, c->d_stage[buf], fmt, ns, k, g, soff, false, &soff_zeroed, st);
       timer_end(c, CORR_KERNEL_DUMP, st, tb);
       if (e != cudaSuccess) return cuda_fail(e, "corr_dump: launch");
       e = cudaMemcpyAsync(static_cast<uint8_t*>(out) + (size_t)k * esz, c->d_stage[buf], (size_t)m * esz,
@@ -1065,7 +1076,7 @@ int corr_dump(corr_ctx* c, void* out, int is_device_ptr, int what, int fmt, int 
       buf ^= 1;
     }
   }
-  if (reset) return corr_reset(c, what, stream);
+  if (reset) return restart(c, what, !is_device_ptr, !soff_zeroed, st);
   return CORR_OK;
 }
 

@@ -189,8 +189,10 @@ unsigned long long context_id();
 // Raise a kernel's dynamic shared-memory limit to `bytes` in the current context, once per (kernel,
 // context); thread-safe.
 cudaError_t set_smem_limit(const void* func, int bytes);
-cudaError_t launch_dump(const long long* d_acc, long long n_elems, void* d_out, int fmt, long long n_samples,
-                        long long k_base, const Shape2& g, cudaStream_t st);
+// `zero`: the dumped cells restart from zero in the same pass, and, where the kernel can do that too
+// (*soff_zeroed), so do the offset sums zero_soff of the dumped channels.
+cudaError_t launch_dump(long long* d_acc, long long n_elems, void* d_out, int fmt, long long n_samples, long long k_base,
+                        const Shape2& g, long long* zero_soff, bool zero, bool* soff_zeroed, cudaStream_t st);
 
 // Thread-local message returned by corr_last_error().
 void set_last_error(const std::string& msg);

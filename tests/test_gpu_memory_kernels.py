@@ -29,6 +29,44 @@ def _at_offset(torch, shape, dtype, skip):
     return torch.full((n + skip,), 7, dtype=dtype, device="cuda")[skip:].view(shape)
 
 
+# channels of one block, of several blocks and of a block and a bit; both polarisation counts
+@pytest.mark.parametrize("N,C,T,npol", [(2, 5, 77, 2), (1, 3, 50, 1), (64, 7, 301, 2), (91, 3, 301, 1), (130, 2, 999, 2),
+                                        (260, 2, 129, 2)])
+@pytest.mark.parametrize("skip", [0, 1])
+def test_dump_restarts_and_alignments(env, N, C, T, npol, skip):
+    corr, synth, torch = env
+    host = synth.generate_host(synth.Spec(kind="saturate", seed=N + T, seg_len=64, m8_segment=1), 2 * T, C, N)
+    x = [torch.from_numpy(host[i * T:(i + 1) * T].copy()).cuda() for i in range(2)]
+    with corr.Correlator(N, C, T, npol) as xc:
+        for what, k in ((corr.CORR_WHAT_CROSS, 0), (corr.CORR_WHAT_AUTO, 1)):
+            for fmt, f in ((corr.CORR_FMT_CI64, oracle.FMT_CI64), (corr.CORR_FMT_CF32, oracle.FMT_CF32),
+                           (corr.CORR_FMT_CF32_NORM, oracle.FMT_CF32_NORM)):
+                dtype = torch.int64 if fmt == corr.CORR_FMT_CI64 else torch.float32
+                for block in (0, 1):  # each dump restarts: the second holds the second block alone
+                    xc.accumulate(x[block])
+                    out = _at_offset(torch, xc.out_shape(what), dtype, skip)
+                    xc.dump(what, fmt, reset=True, out=out)
+                    want = oracle.correlate(host[block * T:(block + 1) * T], npol)[k]
+                    assert np.array_equal(out.cpu().numpy(), oracle.to_format(want, f, T)), (what, fmt, block)
+                    assert xc.samples(what) == 0
+                xc.reset()
+        xc.sync()
+
+
+def test_normalised_dump_is_the_nearest_float(env):
+    """70 million quotients of sums by an odd count, all near 2^24 distinct numerators: the FP64-free
+    division and its fallback near ties against the double division."""
+    corr, synth, torch = env
+    N, C, T = 512, 64, 8001
+    x = synth.generate_device(synth.Spec(kind="gauss_tone", seed=8), T, C, N)
+    with corr.Correlator(N, C, T, 2) as xc:
+        xc.accumulate(x)
+        v = xc.dump(corr.CORR_WHAT_CROSS)
+        q = xc.dump(corr.CORR_WHAT_CROSS, corr.CORR_FMT_CF32_NORM)
+        assert torch.equal(q, (v.double() / float(T)).float())
+        xc.sync()
+
+
 # granules of 16, 8, 4, 2 and 1 bytes; empty parts; runs longer than a piece; more columns than a block
 @pytest.mark.parametrize("T,C,n_local,chan_b,in_b", [
     (3, 300, 32, [0, 109, 109, 300], [0, 16, 48]), (2, 40, 24, [0, 0, 40], [0, 8, 24, 24]), (5, 7, 12, [0, 3, 7], [0, 4, 20]),
