@@ -4,78 +4,104 @@
 namespace corr {
 namespace {
 
-__device__ __forceinline__ int nib(unsigned v) { return ((int)(v & 0xF) ^ 8) - 8; }
+// Autocorrelations A[f][n] += sum_t |x_{f,n}(t)|^2 (Sec. 2.6: total power of selected inputs at a high
+// cadence). HBM-bound: the samples are read once. A row t is M = C N neighbouring bytes; a thread keeps
+// 16 of them (16 cells) and walks down t with eight 16-byte loads in flight, the 8 warps of a block
+// taking every eighth row of the same 512 bytes; the warps' int32 sums meet in shared memory and are
+// added to the int64 sums by one thread a cell. gridDim.y splits t where the columns alone leave SMs
+// idle (the sums then meet in 64-bit atomics, exact in any order).
+// 512 inputs x 2400 channels x 240 samples: 358 us with one byte a load, 62 us so.
+//
+// A square of a 4-bit component x = m - 8 s (s the sign bit, m the low three) is m^2 or (8 - m)^2: a byte
+// permute with the nibbles as selectors looks four of them up at once, the selectors' top bit making
+// the other sign's entries zero (the permute then repeats the entry's top bit, clear in every entry).
+constexpr int AU_NT = 256, AU_W = AU_NT / 32, AU_U = 8;
 
-__device__ __forceinline__ int power_of(unsigned b) {
-  const int re = nib(b >> 4), im = nib(b);
-  return re * re + im * im;
+// squares of the four components in the low 16 bits of w (wx = w ^ 0x88888888), one byte each
+__device__ __forceinline__ uint32_t squares4(uint32_t w, uint32_t wx) {
+  uint32_t p, q;  // prmt's default mode; the intrinsic leaves the selectors' top bits undocumented
+  asm("prmt.b32 %0, %1, %2, %3;" : "=r"(p) : "r"(0x09040100u), "r"(0x31241910u), "r"(w));
+  asm("prmt.b32 %0, %1, %2, %3;" : "=r"(q) : "r"(0x19243140u), "r"(0x01040910u), "r"(wx));
+  return p | q;
 }
 
-// Autocorrelations A[f][n] += sum_t |x_{f,n}(t)|^2 (Sec. 2.6: total power of selected inputs at a
-// high cadence), and optionally the offset sums s[f][n] += sum_t (x + 8 + 8i) needed to map the
-// tensor path's offset-domain products back to V (see the fused X-engine). One block of 4 warps per
-// (channel, group of 32 inputs). Lane l of a warp reads the 4 inputs 4 (l % 8) .. +3 at time offset
-// l / 8, so each warp covers 32 inputs x 4 samples per step and each sample byte is read once.
-// Per-thread int32 partials are reduced over the four time lanes with warp shuffles, then over the
-// 4 warps through shared memory, and added to int64.
-constexpr int AW = 4;
+// acc[0..3] += |x|^2 of the four samples of w
+__device__ __forceinline__ void add_power4(int (&acc)[16], int k, uint32_t w) {
+  const uint32_t wx = w ^ 0x88888888u;
+  const uint32_t lo = squares4(w, wx), hi = squares4(w >> 16, wx >> 16);
+  acc[4 * k + 0] = (int)__dp4a(lo, 0x00000101u, (unsigned)acc[4 * k + 0]);
+  acc[4 * k + 1] = (int)__dp4a(lo, 0x01010000u, (unsigned)acc[4 * k + 1]);
+  acc[4 * k + 2] = (int)__dp4a(hi, 0x00000101u, (unsigned)acc[4 * k + 2]);
+  acc[4 * k + 3] = (int)__dp4a(hi, 0x01010000u, (unsigned)acc[4 * k + 3]);
+}
 
-__global__ void __launch_bounds__(AW * 32) autos_kernel(const uint8_t* __restrict__ in, int N, int C, int T,
-                                                        long long* __restrict__ autos, long long* __restrict__ soff) {
-  const int f = blockIdx.y;
-  const int n0 = blockIdx.x * 32;
+// VEC: 16-byte loads (rows and buffer multiples of 16 bytes); else 16 bytes at any address: the five
+// aligned words around them, shifted together, or byte by byte where those words would leave the
+// buffer [in, end).
+template <bool VEC>
+__device__ __forceinline__ uint4 autos_load(const uint8_t* p, int nv, const uint8_t* in, const uint8_t* end) {
+  if (VEC) return __ldg(reinterpret_cast<const uint4*>(p));
+  const uint32_t sh = (uint32_t)(reinterpret_cast<uintptr_t>(p) & 3);
+  const uint8_t* q = p - sh;
+  uint32_t x[5] = {0u, 0u, 0u, 0u, 0u};
+  if (nv == 16 && q >= in && q + 20 <= end) {
+#pragma unroll
+    for (int k = 0; k < 5; ++k) x[k] = __ldg(reinterpret_cast<const uint32_t*>(q) + k);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) x[k] = __funnelshift_r(x[k], x[k + 1], 8 * sh);
+  } else {
+    for (int k = 0; k < nv; ++k) x[k >> 2] |= (uint32_t)p[k] << (8 * (k & 3));
+  }
+  return make_uint4(x[0], x[1], x[2], x[3]);
+}
+
+template <bool VEC>
+__global__ void __launch_bounds__(AU_NT) autos_kernel(const uint8_t* __restrict__ in, long long M, int T, int rows,
+                                                      long long* __restrict__ autos) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int sub = lane & 7, toff = lane >> 3;  // inputs n0 + 4 sub .. +3, time offset 0..3
-  int acc[4] = {0, 0, 0, 0}, sr[4] = {0, 0, 0, 0}, si[4] = {0, 0, 0, 0};
-  long long acc64[4] = {0, 0, 0, 0}, sr64[4] = {0, 0, 0, 0}, si64[4] = {0, 0, 0, 0};
-  int since = 0;
-  for (int t = warp * 4 + toff; t < T; t += AW * 4) {
-    const uint8_t* row = in + ((size_t)t * C + f) * N + n0 + 4 * sub;
+  const long long col = blockIdx.x * 512LL + 16 * lane;
+  const int nv = M - col >= 16 ? 16 : (M > col ? (int)(M - col) : 0);
+  const int t_end = (int)min((long long)T, (blockIdx.y + 1LL) * rows);
+  const uint8_t* end = in + (size_t)T * M;
+  int acc[16];
 #pragma unroll
-    for (int q = 0; q < 4; ++q)
-      if (n0 + 4 * sub + q < N) {
-        const unsigned b = row[q];
-        acc[q] += power_of(b);
-        sr[q] += (int)((b >> 4) ^ 8u);   // Re + 8
-        si[q] += (int)((b & 15u) ^ 8u);  // Im + 8
-      }
-    if (++since == (1 << 20)) {  // int32 partials stay below 128 * 2^20
+  for (int k = 0; k < 16; ++k) acc[k] = 0;
+  if (nv > 0) {
+    // long: the last steps of a row count near 2^31 would overflow an int
+    for (long long t0 = (long long)blockIdx.y * rows + warp; t0 < t_end; t0 += AU_W * AU_U) {
+      uint4 w[AU_U];
 #pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        acc64[q] += acc[q];
-        sr64[q] += sr[q];
-        si64[q] += si[q];
-        acc[q] = sr[q] = si[q] = 0;
+      for (int u = 0; u < AU_U; ++u) {
+        const long long t = t0 + AU_W * u;
+        w[u] = t < t_end ? autos_load<VEC>(in + (size_t)t * M + col, nv, in, end) : make_uint4(0u, 0u, 0u, 0u);
       }
-      since = 0;
+#pragma unroll
+      for (int u = 0; u < AU_U; ++u) {
+        add_power4(acc, 0, w[u].x);
+        add_power4(acc, 1, w[u].y);
+        add_power4(acc, 2, w[u].z);
+        add_power4(acc, 3, w[u].w);
+      }
     }
   }
-  __shared__ long long part[3][AW][32];
+  __shared__ __align__(16) int part[AU_W][512];
 #pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    long long v[3] = {acc64[q] + acc[q], sr64[q] + sr[q], si64[q] + si[q]};
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-      v[k] += __shfl_xor_sync(0xffffffffu, v[k], 8);
-      v[k] += __shfl_xor_sync(0xffffffffu, v[k], 16);
-      if (toff == 0) part[k][warp][4 * sub + q] = v[k];
-    }
-  }
+  for (int k = 0; k < 4; ++k)
+    *reinterpret_cast<int4*>(&part[warp][16 * lane + 4 * k]) =
+        make_int4(acc[4 * k], acc[4 * k + 1], acc[4 * k + 2], acc[4 * k + 3]);
   __syncthreads();
-  if (threadIdx.x < 32) {
-    const int n = n0 + threadIdx.x;
-    long long sum[3] = {0, 0, 0};
 #pragma unroll
-    for (int w = 0; w < AW; ++w)
+  for (int h = 0; h < 2; ++h) {
+    const int i = threadIdx.x + AU_NT * h;
+    const long long cell = blockIdx.x * 512LL + i;
+    if (cell >= M) break;
+    long long sum = 0;
 #pragma unroll
-      for (int k = 0; k < 3; ++k) sum[k] += part[k][w][threadIdx.x];
-    if (n < N) {
-      autos[(long long)f * N + n] += sum[0];
-      if (soff) {
-        soff[((long long)f * N + n) * 2] += sum[1];
-        soff[((long long)f * N + n) * 2 + 1] += sum[2];
-      }
-    }
+    for (int v = 0; v < AU_W; ++v) sum += part[v][i];
+    if (gridDim.y == 1)
+      autos[cell] += sum;
+    else
+      atomicAdd(reinterpret_cast<unsigned long long*>(autos + cell), (unsigned long long)sum);
   }
 }
 
@@ -365,11 +391,22 @@ __global__ void set_base_kernel(long long* __restrict__ base, const int* __restr
 
 }  // namespace
 
-cudaError_t launch_autos(const Shape& s, const uint8_t* d_in, int T_blk, long long* d_autos, long long* d_soff,
-                         cudaStream_t st) {
+cudaError_t launch_autos(const Shape& s, const uint8_t* d_in, int T_blk, long long* d_autos, cudaStream_t st) {
   if (T_blk == 0) return cudaSuccess;
-  dim3 grid((s.N + 31) / 32, s.C);
-  autos_kernel<<<grid, AW * 32, 0, st>>>(d_in, s.N, s.C, T_blk, d_autos, d_soff);
+  const long long M = (long long)s.C * s.N;
+  const long long gx = (M + 511) / 512;
+  // rows per block: all of them while the columns fill the GPU (four blocks an SM), else at least 64 (8 a
+  // warp, one step of loads); at most 2^20 (8 x 2^17 samples of at most 128 in an int32 sum)
+  const long long want = (4LL * sm_count() + gx - 1) / gx;
+  long long rows = ((long long)T_blk + want - 1) / want;
+  if (rows < 64) rows = 64;
+  if (rows > (1 << 20)) rows = 1 << 20;
+  if (rows > T_blk) rows = T_blk;
+  const dim3 grid((unsigned)gx, (unsigned)((T_blk + rows - 1) / rows));
+  if (M % 16 == 0 && reinterpret_cast<uintptr_t>(d_in) % 16 == 0)
+    autos_kernel<true><<<grid, AU_NT, 0, st>>>(d_in, M, T_blk, (int)rows, d_autos);
+  else
+    autos_kernel<false><<<grid, AU_NT, 0, st>>>(d_in, M, T_blk, (int)rows, d_autos);
   return cudaGetLastError();
 }
 

@@ -110,9 +110,8 @@ inline long long round_up(long long x, long long m) { return (x + m - 1) / m * m
 cudaError_t launch_fp32(const Shape& s, const uint8_t* d_in, int T_blk, int flush_len, const int2* d_tiles,
                         int n_tiles, long long* d_cross, long long* d_autos, cudaStream_t st);
 
-// Autos (+ offset sums when d_soff != nullptr).
-cudaError_t launch_autos(const Shape& s, const uint8_t* d_in, int T_blk, long long* d_autos, long long* d_soff,
-                         cudaStream_t st);
+// Autocorrelations of a block.
+cudaError_t launch_autos(const Shape& s, const uint8_t* d_in, int T_blk, long long* d_autos, cudaStream_t st);
 
 // Fused unpack + tcgen05 X-engine (offset-domain products into d_cross, diagonal into d_autos).
 cudaError_t launch_i8mma(const Shape& s, const uint8_t* d_in, int T_blk, int flush_len, const int2* d_tiles,

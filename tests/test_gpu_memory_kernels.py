@@ -67,6 +67,22 @@ def test_normalised_dump_is_the_nearest_float(env):
         xc.sync()
 
 
+# a few columns, many columns, a last partial column, one sample, a split time range; odd pointers
+@pytest.mark.parametrize("N,C,T", [(1, 1, 1), (2, 3, 5000), (7, 5, 65), (512, 3, 63), (33, 31, 129), (256, 400, 40)])
+@pytest.mark.parametrize("skip", [0, 1, 5])
+def test_total_power_columns(env, N, C, T, skip):
+    corr, synth, torch = env
+    host = synth.generate_host(synth.Spec(kind="saturate", seed=N * 3 + T, seg_len=32, m8_segment=0), T, C, N)
+    x = _at_offset(torch, host.shape, torch.uint8, skip)
+    x.copy_(torch.from_numpy(host))
+    with corr.Correlator(N, C, T, 1) as xc:
+        xc.accumulate_autos(x)
+        xc.accumulate_autos(x)
+        a = xc.dump(corr.CORR_WHAT_AUTO)
+        xc.sync()
+    assert np.array_equal(a.cpu().numpy(), 2 * oracle.autos(host))
+
+
 # granules of 16, 8, 4, 2 and 1 bytes; empty parts; runs longer than a piece; more columns than a block
 @pytest.mark.parametrize("T,C,n_local,chan_b,in_b", [
     (3, 300, 32, [0, 109, 109, 300], [0, 16, 48]), (2, 40, 24, [0, 0, 40], [0, 8, 24, 24]), (5, 7, 12, [0, 3, 7], [0, 4, 20]),
