@@ -63,10 +63,13 @@ typedef enum corr_path {
   CORR_PATH_FP32 = 1,  /* FP32 FMA on CUDA cores (the arithmetic the paper's K20X X-engine used, Sec. 2.5) */
   CORR_PATH_I8MMA = 2, /* warp-level integer MMA (mma.sync s8 x s8 -> s32) on sign-extended nibbles,
                           unpacked in shared memory inside the kernel; the integer tensor path */
-  CORR_PATH_FP8TC = 3, /* tcgen05 kind::f8f6f4 (e4m3 operands, FP32 accumulation in TMEM): an
-                          unpack pass builds the offset operand and the per-input sums in device
-                          scratch, a TMA-fed persistent kernel multiplies and adds the autos from its
-                          diagonal. The default. */
+  CORR_PATH_FP8TC = 3, /* tcgen05 kind::f8f6f4 (e4m3 operands, FP32 accumulation in TMEM). The default. A
+                          TMA-fed persistent kernel builds the offset operand and the per-input sums
+                          on the chip, multiplies and adds the autos from its diagonal, where the
+                          rows allow TMA (16-byte aligned blocks; N a multiple of 16, or an array of
+                          at most 64 inputs whose channels pack into such rows) and neither a tile
+                          plan other than the default nor a build schedule was asked for; else an
+                          unpack pass writes the operand to device scratch for such a kernel. */
   CORR_PATH_FP8TC_FUSED = 4 /* same arithmetic with the unpack done inside the X-engine by converter
                                warps (no scratch; slower on this input layout, kept for comparison) */
 } corr_path;

@@ -202,6 +202,19 @@ int encode_op_tensor_map(CUtensorMap* map, void* d_op, int R, int T_pad, int C, 
 // Raw input in[T][C][N] as a 3-D map, boxes of 64 inputs x 1 channel x 128 samples, no swizzle.
 int encode_input_tensor_map(CUtensorMap* map, const void* d_in, int N, int C, int T, std::string* err);
 
+// A block in[T][C][N] as a 2-D map of T rows of C N bytes, boxes of box_bytes x 128 samples (64-byte swizzle if set).
+int encode_raw_tensor_map(CUtensorMap* map, const void* d_in, long long row_bytes, int T, int box_bytes, bool swizzle,
+                          std::string* err);
+
+// X-engines that build their operand on the chip (xeng_direct.cuh): n blocks of one array, products into
+// cross and autos, offset sums into s1 and s2. launch_xeng_direct: SM pairs, more than 64 inputs;
+// launch_xeng_small: at most 64. xeng_*_supported: the shapes and alignments each takes.
+struct DirectJob;
+cudaError_t launch_xeng_direct(const DirectJob& j, int num_sms, cudaStream_t st);
+bool xeng_direct_supported(const Shape& s, const void* d_in);
+cudaError_t launch_xeng_small(const DirectJob& j, int num_sms, cudaStream_t st);
+bool xeng_small_supported(const Shape& s, const void* d_in);
+
 // The fused path needs 16-byte TMA strides (N % 16 == 0, aligned input) and boxes no larger than the
 // array (N >= 64, T >= 128).
 bool f8_fused_supported(const Shape& s, const void* d_in, int T_blk);
