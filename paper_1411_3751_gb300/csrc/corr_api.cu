@@ -274,32 +274,61 @@ void free_ctx(corr_ctx* c) {
 
 XengArgs xeng_args(const corr_ctx* c, int buf, int T_run, int flush);  // buf: operand buffer d_op (0) or d_op2 (1)
 
-// The tensor path without an operand in HBM (launch_xeng_direct, launch_xeng_small), for blocks it takes. A tile
-// plan or a build schedule that was asked for keeps the two passes.
-bool takes_direct(const corr_ctx* c, const uint8_t* d_in) {
-  if (c->tile_plan != c->plan_default || c->prep_sms > 0) return false;
-  return xeng_small_supported(c->L.s, d_in) || xeng_direct_supported(c->L.s, d_in);
+// How a block takes the tensor path: without an operand in HBM (launch_xeng_direct, launch_xeng_small) from its own
+// rows or from rows repacked to whole 16-byte columns, or in the two passes, which a tile plan or a build
+// schedule that was asked for keeps.
+enum Route { ROUTE_TWO_PASS, ROUTE_DIRECT, ROUTE_REPACK };
+
+int repacked_inputs(const corr_ctx* c) { return (int)round_up(c->L.s.N, 16); }
+
+Route route_of(const corr_ctx* c, const uint8_t* d_in) {
+  if (c->tile_plan != c->plan_default || c->prep_sms > 0) return ROUTE_TWO_PASS;
+  const Shape& s = c->L.s;
+  if (xeng_small_supported(s, s.N, d_in) || xeng_direct_supported(s, s.N, d_in)) return ROUTE_DIRECT;
+  const int Np = repacked_inputs(c);
+  if (c->d_op && (xeng_small_supported(s, Np, c->d_op) || xeng_direct_supported(s, Np, c->d_op))) return ROUTE_REPACK;
+  return ROUTE_TWO_PASS;
 }
 
-// n blocks of T_blk samples through it, in one launch (n at most direct_max_blocks).
-int accumulate_direct(corr_ctx* c, const uint8_t* const* blocks, int n, int T_blk, cudaStream_t st) {
+// n blocks of T_blk samples, all of one of the direct routes, in as many launches as `most` blocks a launch make.
+int accumulate_direct(corr_ctx* c, const uint8_t* const* blocks, int n, int T_blk, int most, Route route, cudaStream_t st) {
   DirectJob j;
   j.s = c->L.s;
-  j.blocks = blocks;
-  j.n = n;
   j.T_blk = T_blk;
+  j.ld = c->L.s.N;
   j.flush_len = flush_for(c, CORR_PATH_FP8TC);
   j.cross = c->d_cross;
   j.autos = c->d_autos;
   j.s1 = c->d_soff;
   j.s2 = c->d_soff_auto;
   j.err = c->d_err;
-  const bool tb = timer_begin(c, CORR_KERNEL_XENG, st);
-  const cudaError_t e = c->L.s.N <= 64 ? launch_xeng_small(j, c->num_sms, st) : launch_xeng_direct(j, c->num_sms, st);
-  timer_end(c, CORR_KERNEL_XENG, st, tb);
-  if (e != cudaSuccess) return cuda_fail(e, "tensor x-engine launch");
-  c->n_off += (long long)T_blk * n;
-  c->n_off_auto += (long long)T_blk * n;
+  int K = std::min(most, direct_max_blocks(T_blk));
+  const uint8_t* packed[xd::MAX_BLOCKS];
+  const long long rows = (long long)T_blk * c->L.s.C;
+  if (route == ROUTE_REPACK) {  // in the operand scratch, which holds twice as many blocks' samples
+    j.ld = repacked_inputs(c);
+    K = (int)std::min<long long>(K, (long long)(c->L.op_buf_bytes / ((size_t)rows * j.ld)));
+    for (int i = 0; i < K; ++i) packed[i] = c->d_op + (size_t)i * rows * j.ld;
+  }
+  for (int b0 = 0; b0 < n; b0 += K) {
+    j.n = std::min(K, n - b0);
+    j.blocks = blocks + b0;
+    if (route == ROUTE_REPACK) {
+      j.blocks = packed;
+      for (int i = 0; i < j.n; ++i) {
+        const bool tb = timer_begin(c, CORR_KERNEL_UNPACK, st);
+        const cudaError_t e = launch_repack(blocks[b0 + i], rows, c->L.s.N, j.ld, c->d_op + (size_t)i * rows * j.ld, st);
+        timer_end(c, CORR_KERNEL_UNPACK, st, tb);
+        if (e != cudaSuccess) return cuda_fail(e, "repack launch");
+      }
+    }
+    const bool tb = timer_begin(c, CORR_KERNEL_XENG, st);
+    const cudaError_t e = c->L.s.N <= 64 ? launch_xeng_small(j, c->num_sms, st) : launch_xeng_direct(j, c->num_sms, st);
+    timer_end(c, CORR_KERNEL_XENG, st, tb);
+    if (e != cudaSuccess) return cuda_fail(e, "tensor x-engine launch");
+    c->n_off += (long long)T_blk * j.n;
+    c->n_off_auto += (long long)T_blk * j.n;
+  }
   return CORR_OK;
 }
 
@@ -319,8 +348,8 @@ int accumulate_device(corr_ctx* c, const uint8_t* d_in, int T_blk, cudaStream_t 
     e = launch_i8mma(c->L.s, d_in, T_blk, flush, c->d_tiles32, c->n_tiles32, c->d_cross, c->d_autos, st);
     timer_end(c, CORR_KERNEL_XENG, st, tb);
     if (e != cudaSuccess) return cuda_fail(e, "int8 mma x-engine launch");
-  } else if (path == CORR_PATH_FP8TC && takes_direct(c, d_in)) {
-    return accumulate_direct(c, &d_in, 1, T_blk, st);
+  } else if (const Route route = path == CORR_PATH_FP8TC ? route_of(c, d_in) : ROUTE_TWO_PASS; route != ROUTE_TWO_PASS) {
+    return accumulate_direct(c, &d_in, 1, T_blk, 1, route, st);
   } else {
     // tensor paths: one pass builds the operand (two-pass path) and the per-input offset sums for
     // both cadences; the X-engine adds the offset-domain products and their diagonal.
@@ -571,19 +600,13 @@ int accumulate_batch_overlap(corr_ctx* c, const uint8_t* const* blocks, int n, c
 // flushes. With prep_sms_for(c) = k > 0 the build of chunk j + 1 runs on k SMs beside the multiply of
 // chunk j (accumulate_batch_overlap); otherwise the chunks run in order on the caller's stream.
 int accumulate_batch_chunks(corr_ctx* c, const uint8_t* const* blocks, int n, cudaStream_t st) {
-  bool direct = true;
-  for (int b = 0; b < n && direct; ++b) direct = takes_direct(c, blocks[b]);
-  if (direct) {
+  const Route route = n > 0 ? route_of(c, blocks[0]) : ROUTE_TWO_PASS;
+  bool same = route != ROUTE_TWO_PASS;
+  for (int b = 1; b < n && same; ++b) same = route_of(c, blocks[b]) == route;
+  if (same)
     // as many blocks per launch as fit it (512 inputs x 128 channels x 16 blocks of 8192 samples: 6.38 ms in one
     // launch, 6.55 in four), or the number that was asked for
-    const int kmax = direct_max_blocks(c->L.s.T);
-    const int K = c->L.K_batch == c->K_default ? kmax : std::min(kmax, c->L.K_batch);
-    for (int b0 = 0; b0 < n; b0 += K) {
-      const int rc = accumulate_direct(c, blocks + b0, std::min(K, n - b0), c->L.s.T, st);
-      if (rc != CORR_OK) return rc;
-    }
-    return CORR_OK;
-  }
+    return accumulate_direct(c, blocks, n, c->L.s.T, c->L.K_batch == c->K_default ? xd::MAX_BLOCKS : c->L.K_batch, route, st);
   // overlapped schedule when there are at least two chunks and the TMA build takes the shape (the wide
   // plan 2 fills both accumulators per item and is not overlapped)
   const int k = prep_sms_for(c);

@@ -208,12 +208,15 @@ int encode_raw_tensor_map(CUtensorMap* map, const void* d_in, long long row_byte
 
 // X-engines that build their operand on the chip (xeng_direct.cuh): n blocks of one array, products into
 // cross and autos, offset sums into s1 and s2. launch_xeng_direct: SM pairs, more than 64 inputs;
-// launch_xeng_small: at most 64. xeng_*_supported: the shapes and alignments each takes.
+// launch_xeng_small: at most 64. xeng_*_supported: the shapes, row lengths ld (inputs a channel as
+// stored) and alignments each takes.
 struct DirectJob;
 cudaError_t launch_xeng_direct(const DirectJob& j, int num_sms, cudaStream_t st);
-bool xeng_direct_supported(const Shape& s, const void* d_in);
+bool xeng_direct_supported(const Shape& s, int ld, const void* d_in);
 cudaError_t launch_xeng_small(const DirectJob& j, int num_sms, cudaStream_t st);
-bool xeng_small_supported(const Shape& s, const void* d_in);
+bool xeng_small_supported(const Shape& s, int ld, const void* d_in);
+// in[rows][N] -> out[rows][Np], Np = N rounded up to a multiple of 16 (repack.cu).
+cudaError_t launch_repack(const uint8_t* d_in, long long rows, int N, int Np, uint8_t* d_out, cudaStream_t st);
 
 // The fused path needs 16-byte TMA strides (N % 16 == 0, aligned input) and boxes no larger than the
 // array (N >= 64, T >= 128).

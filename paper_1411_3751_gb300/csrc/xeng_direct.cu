@@ -144,7 +144,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(D_THREADS, 1)
       uint32_t phase = 0, n_issued = 0;
       for (long long w = pair; w < total && !*abort_flag; w += n_pairs) {
         const Item it(args, w);
-        const int xc = it.f * args.N + it.c0 + 64 * (int)rank, xa = it.f * args.N + it.a0 + 64 * (int)rank;
+        const int xc = it.f * args.ld + it.c0 + 64 * (int)rank, xa = it.f * args.ld + it.a0 + 64 * (int)rank;
         xd::StagePos p(it.k0, args.n_kb);
         for (int k = it.k0; k < it.k1; ++k, p.next(args.n_kb)) {
           if (!ptx::mbar_wait(&raw_empty[slot], phase ^ 1, WAIT_NS)) {
@@ -419,8 +419,8 @@ int direct_max_pairs() {
 
 }  // namespace
 
-bool xeng_direct_supported(const Shape& s, const void* d_in) {
-  return s.N > 64 && s.N % 16 == 0 && reinterpret_cast<uintptr_t>(d_in) % 16 == 0 && (long long)s.N * s.C < (1LL << 31);
+bool xeng_direct_supported(const Shape& s, int ld, const void* d_in) {
+  return s.N > 64 && ld % 16 == 0 && reinterpret_cast<uintptr_t>(d_in) % 16 == 0 && (long long)ld * s.C < (1LL << 31);
 }
 
 int direct_splits(long long items, int slots, int n_k, int overhead) {
@@ -445,7 +445,7 @@ cudaError_t direct_args(const DirectJob& j, int box_bytes, bool swizzle, xd::Arg
   if (j.n > xd::MAX_BLOCKS) return cudaErrorInvalidValue;
   for (int b = 0; b < j.n; ++b) {
     std::string err;
-    if (encode_raw_tensor_map(&a->map[b], j.blocks[b], (long long)j.s.C * j.s.N, j.T_blk, box_bytes, swizzle, &err) != 0) {
+    if (encode_raw_tensor_map(&a->map[b], j.blocks[b], (long long)j.s.C * j.ld, j.T_blk, box_bytes, swizzle, &err) != 0) {
       set_last_error(err);
       return cudaErrorInvalidValue;
     }
@@ -456,6 +456,7 @@ cudaError_t direct_args(const DirectJob& j, int box_bytes, bool swizzle, xd::Arg
   a->s2 = j.s2;
   a->Bs = j.s.Bs;
   a->N = j.s.N;
+  a->ld = j.ld;
   a->C = j.s.C;
   a->npol = j.s.npol;
   a->T = j.T_blk;

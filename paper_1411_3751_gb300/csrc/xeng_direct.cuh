@@ -11,13 +11,14 @@ namespace xd {
 constexpr int MAX_BLOCKS = 16;  // blocks of one launch: one tensor map each
 
 struct Args {
-  CUtensorMap map[MAX_BLOCKS];  // block b as [T][C N] bytes
+  CUtensorMap map[MAX_BLOCKS];  // block b as [T][C ld] bytes
   long long* cross;
   long long* autos;
   long long* s1;  // offset sums [C][N][2], both cadences
   long long* s2;
   long long Bs;
   int N, C, npol, T;
+  int ld;               // inputs a row and channel as stored: N, or more (repacked rows)
   int n_kb, n_k;        // 128-sample stages of a block (the last one may be short) and of all blocks
   int chunk_k;          // stages per in-chip partial sum
   int splits, kps;      // the stages of an item are divided over `splits` items of kps stages
@@ -111,8 +112,8 @@ inline int direct_max_blocks(int T) {
 // One launch's work: `n` blocks of T_blk samples of one array.
 struct DirectJob {
   Shape s;
-  const uint8_t* const* blocks;
-  int n, T_blk, flush_len;
+  const uint8_t* const* blocks;  // [T_blk][C][ld]
+  int n, T_blk, ld, flush_len;
   long long *cross, *autos, *s1, *s2;
   int* err;
 };

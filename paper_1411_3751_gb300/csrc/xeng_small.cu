@@ -272,10 +272,10 @@ __global__ void __launch_bounds__(S_THREADS, 1) xeng_small_kernel(const __grid_c
             re += __shfl_xor_sync(0xffffffffu, re, 16);
             im += __shfl_xor_sync(0xffffffffu, im, 16);
             const int in = 16 * c + 4 * i + b;  // input row of the unit
-            const int ch = in / args.N;
+            const int ch = in / args.ld, n = in - ch * args.ld;
             const long long f = u * args.g + ch;
-            if (pr == i && ch < args.g && u < args.n_units && f < args.C) {
-              const long long idx = (f * args.N + in - ch * args.N) * 2;
+            if (pr == i && ch < args.g && n < args.N && u < args.n_units && f < args.C) {
+              const long long idx = (f * args.N + n) * 2;
               atomicAdd(reinterpret_cast<unsigned long long*>(args.s1 + idx), (unsigned long long)re);
               atomicAdd(reinterpret_cast<unsigned long long*>(args.s1 + idx + 1), (unsigned long long)im);
               atomicAdd(reinterpret_cast<unsigned long long*>(args.s2 + idx), (unsigned long long)re);
@@ -291,9 +291,9 @@ __global__ void __launch_bounds__(S_THREADS, 1) xeng_small_kernel(const __grid_c
     const int lp = args.npol >> 1;
     const int row = 32 * q + lane;
     const int ic = 4 * (row >> 3) + (row & 3);  // c-input of the unit
-    const int ch = ic / args.N, c = ic - ch * args.N;
+    const int ch = ic / args.ld, c = ic - ch * args.ld;
     // the chunks (16 a-inputs) that hold this warp's channels, from the diagonal on
-    const int last = min(64, ((16 * q + 15) / args.N + 1) * args.N);
+    const int last = min(64, ((16 * q + 15) / args.ld + 1) * args.ld);
     const int cc_end = (last + 15) / 16;
     uint32_t use[2] = {0u, 0u};
     int acc = 0;
@@ -321,7 +321,7 @@ __global__ void __launch_bounds__(S_THREADS, 1) xeng_small_kernel(const __grid_c
             uint32_t v[32];
             ptx::tmem_ld_32x32b_x32(tbase + 256 * acc + 128 * h + ((uint32_t)(32 * q) << 16) + 32 * cc, v);
             ptx::tmem_ld_wait();
-            xd::add_chunk<4, ADD, 8>(v, im_lane, live ? c : -1, 16 * cc - ch * args.N, args.N, lp, cross_f, autos_f);
+            xd::add_chunk<4, ADD, 8>(v, im_lane, live ? c : -1, 16 * cc - ch * args.ld, args.N, lp, cross_f, autos_f);
           }
         }
         ptx::tc_fence_before();
@@ -338,19 +338,19 @@ __global__ void __launch_bounds__(S_THREADS, 1) xeng_small_kernel(const __grid_c
   if (warp == 1) ptx::tmem_dealloc(tbase, TMEM_COLS);
 }
 
-// Channels per 64-input unit: as many as fit with a unit of whole 16-byte columns; 0 if none.
-int small_group(int N) {
-  if (N > 64) return 0;
-  for (int g = 64 / N; g >= 1; --g)
-    if (g * N % 16 == 0) return g;
+// Channels (of ld stored inputs) per 64-input unit: as many as fit with a unit of whole 16-byte columns; 0 if none.
+int small_group(int ld) {
+  if (ld > 64) return 0;
+  for (int g = 64 / ld; g >= 1; --g)
+    if (g * ld % 16 == 0) return g;
   return 0;
 }
 
 }  // namespace
 
-bool xeng_small_supported(const Shape& s, const void* d_in) {
-  const long long row = (long long)s.N * s.C;
-  return small_group(s.N) > 0 && row % 16 == 0 && row < (1LL << 31) && reinterpret_cast<uintptr_t>(d_in) % 16 == 0;
+bool xeng_small_supported(const Shape& s, int ld, const void* d_in) {
+  const long long row = (long long)ld * s.C;
+  return s.N <= 64 && small_group(ld) > 0 && row % 16 == 0 && row < (1LL << 31) && reinterpret_cast<uintptr_t>(d_in) % 16 == 0;
 }
 
 cudaError_t launch_xeng_small(const DirectJob& j, int num_sms, cudaStream_t st) {
@@ -360,8 +360,8 @@ cudaError_t launch_xeng_small(const DirectJob& j, int num_sms, cudaStream_t st) 
   xd::Args a;
   if (e == cudaSuccess) e = direct_args(j, 128, false, &a);
   if (e != cudaSuccess) return e;
-  a.g = small_group(j.s.N);
-  a.ub = a.g * j.s.N;
+  a.g = small_group(j.ld);
+  a.ub = a.g * j.ld;
   a.n_units = (j.s.C + a.g - 1) / a.g;
   const long long pairs = (a.n_units + 1) / 2;
   a.splits = direct_splits(pairs, num_sms, a.n_k, 4);

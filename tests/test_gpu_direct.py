@@ -78,7 +78,8 @@ def test_batches_and_flushes(env, N, C, T, blocks, flush):
 
 
 @pytest.mark.parametrize("N,C,T,blocks", [(64, 701, 4096, 2), (32, 2401, 2048, 2), (16, 2500, 4096, 1), (48, 640, 3000, 1),
-                                          (128, 310, 4096, 1), (512, 24, 8192, 2), (208, 160, 2000, 3)])
+                                          (128, 310, 4096, 1), (512, 24, 8192, 2), (208, 160, 2000, 3), (200, 170, 4096, 2),
+                                          (132, 190, 3000, 2), (134, 150, 3000, 2), (40, 700, 4096, 1)])
 def test_several_items_a_cta(env, N, C, T, blocks):
     """More work items than SMs and rings that wrap many times, against the int8 path on the same blocks."""
     corr, synth, torch = env
@@ -94,10 +95,15 @@ def test_several_items_a_cta(env, N, C, T, blocks):
         assert torch.equal(a, b)
 
 
-@pytest.mark.parametrize("N,C,skip", [(64, 2, 1), (64, 2, 8), (32, 3, 4), (128, 2, 8), (20, 3, 0), (40, 2, 0), (7, 3, 0)])
-def test_rows_that_tma_does_not_take(env, N, C, skip):
-    """Unaligned blocks and input counts without 16-byte rows: the two passes, same sums."""
-    _check(env, _host(env[1], N, C, 300), 1, skip=skip)
+# rows TMA does not take, repacked: counts of every alignment (odd and even counts,
+# unaligned blocks, a last column of 1 .. 16 inputs, rows of one and of many columns)
+@pytest.mark.parametrize("N,C,npol,skip", [(72, 2, 2, 0), (200, 3, 2, 0), (136, 1, 1, 8), (68, 3, 2, 0), (100, 2, 2, 4), (260, 1, 2, 12),
+                                           (128, 2, 2, 8), (128, 2, 2, 1), (131, 3, 1, 0), (67, 2, 1, 3), (130, 2, 2, 2),
+                                           (66, 1, 2, 0), (40, 3, 2, 0), (20, 2, 2, 0), (10, 3, 2, 0), (7, 3, 1, 0), (33, 2, 1, 0),
+                                           (1, 3, 1, 0), (64, 2, 2, 1), (32, 3, 2, 4), (16, 5, 2, 8), (5, 1, 1, 7)])
+@pytest.mark.parametrize("T,blocks", [(1, 1), (129, 1), (1000, 2), (300, 18)])
+def test_rows_that_tma_does_not_take(env, N, C, npol, skip, T, blocks):
+    _check(env, _host(env[1], N, C, T, blocks), npol, skip=skip, blocks=blocks)
 
 
 def test_schedules_that_were_asked_for_mix_with_the_default(env):
