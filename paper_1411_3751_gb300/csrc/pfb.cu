@@ -11,9 +11,14 @@
 // One CTA of 256 threads per (input, two spectra). The real DFT is a 4096-point complex FFT of
 // z[j] = y[2j] + i y[2j+1] followed by the split step that separates the even and odd halves:
 //   X[k] = (Z[k] + conj Z[-k]) / 2 - i W^k (Z[k] - conj Z[-k]) / 2,  W = exp(-2 pi i / M).
-// The complex FFT is a Stockham autosort FFT (no bit reversal), three radix-16 passes in shared
-// memory; each thread holds 16 points per pass. Twiddles come from tables computed on the host in
-// double precision.
+// The complex FFT is a Stockham autosort FFT (no bit reversal) of three radix-16 passes. What bounded it
+// was shared memory (four exchanges of 64 KB a spectrum) and load latency, so data leave the registers
+// only twice: the FIR sums are formed by the threads whose first pass takes them, and in the last pass a
+// thread of a spectrum's 128 holds columns u and 256 - u, whose outputs are each other's mirror images
+// k and 4096 - k, so that the split step needs no exchange either. Twiddles come from tables computed on
+// the host in double precision. 512 inputs x 64 spectra, 4 taps: 753 us before, 588 us so
+// (2 CTAs of 8 warps an SM; without the FIR's loads 465, without the output stores 489; with 80 registers and a
+// third CTA 686, with the samples staged through shared memory by 16-byte loads 613).
 #include "corr_internal.cuh"
 
 #include <cmath>
@@ -78,162 +83,190 @@ __device__ __forceinline__ void dft16(float2 (&v)[16]) {
   for (int q = 0; q < 16; ++q) v[q] = t[q];
 }
 
-constexpr int PFB_SPB = 2;                  // spectra per block (share the coefficient loads)
+constexpr int PFB_SPB = 2;                    // spectra per block (share the coefficient and frame loads)
 constexpr int PFB_ZLEN = PFB_H + PFB_H / 16;  // padded complex buffer per spectrum
 
-// 4096-point complex FFT of z (padded layout) in place, Stockham radix 16: spans Ns = 1, 16, 256.
-// The 15 twiddles exp(-2 pi i r k / (16 Ns)) of a thread come from 4 table loads, w^{4a+b} = w^{4a} w^b.
-__device__ __forceinline__ void fft4096(float2* z, int tid) {
-#pragma unroll 1
-  for (int Ns = 1, tw = PFB_H / 16; Ns < PFB_H; Ns *= 16, tw /= 16) {
-    const int k = tid & (Ns - 1);
-    const int e = k * tw;  // < 4096 / 16; the table loads go out before the shared-memory loads
-    float2 w1 = make_float2(1.f, 0.f), w4 = w1, w8 = w1, w12 = w1;
-    if (Ns > 1) {
-      w1 = g_w4096[e];
-      w4 = g_w4096[4 * e];
-      w8 = g_w4096[8 * e];
-      w12 = g_w4096[12 * e];
-    }
-    float2 v[16];
+// v[r] *= w^r for r = 1 .. 15 from w1 = w, w4 = w^4, w8, w12, as w^(4a + b) = w^(4a) w^b, for each of S columns.
+template <int S>
+__device__ __forceinline__ void twiddle16(float2 (&v)[S][16], float2 w1, float2 w4, float2 w8, float2 w12) {
+  const float2 w2 = cmul(w1, w1), w3 = cmul(w2, w1);
 #pragma unroll
-    for (int r = 0; r < 16; ++r) v[r] = z[sidx(tid + r * (PFB_H / 16))];
-    if (Ns > 1) {
-      const float2 w2 = cmul(w1, w1), w3 = cmul(w2, w1);
-      v[1] = cmul(v[1], w1);
-      v[2] = cmul(v[2], w2);
-      v[3] = cmul(v[3], w3);
-      v[4] = cmul(v[4], w4);
-      v[5] = cmul(v[5], cmul(w4, w1));
-      v[6] = cmul(v[6], cmul(w4, w2));
-      v[7] = cmul(v[7], cmul(w4, w3));
-      v[8] = cmul(v[8], w8);
-      v[9] = cmul(v[9], cmul(w8, w1));
-      v[10] = cmul(v[10], cmul(w8, w2));
-      v[11] = cmul(v[11], cmul(w8, w3));
-      v[12] = cmul(v[12], w12);
-      v[13] = cmul(v[13], cmul(w12, w1));
-      v[14] = cmul(v[14], cmul(w12, w2));
-      v[15] = cmul(v[15], cmul(w12, w3));
-    }
-    dft16(v);
-    __syncthreads();
-    const int base = (tid - k) * 16 + k;
+  for (int a = 0; a < 4; ++a) {
+    const float2 wa = a == 1 ? w4 : a == 2 ? w8 : w12;
+    const float2 t1 = a ? cmul(wa, w1) : w1, t2 = a ? cmul(wa, w2) : w2, t3 = a ? cmul(wa, w3) : w3;
 #pragma unroll
-    for (int q = 0; q < 16; ++q) z[sidx(base + q * Ns)] = v[q];
-    __syncthreads();
+    for (int s = 0; s < S; ++s) {
+      if (a) v[s][4 * a] = cmul(v[s][4 * a], wa);
+      v[s][4 * a + 1] = cmul(v[s][4 * a + 1], t1);
+      v[s][4 * a + 2] = cmul(v[s][4 * a + 2], t2);
+      v[s][4 * a + 3] = cmul(v[s][4 * a + 3], t3);
+    }
   }
+}
+__device__ __forceinline__ float2 conjf2(float2 a) { return make_float2(a.x, -a.y); }
+
+// X[k] and X[4096 - k] from a = Z[k], b = Z[4096 - k] and w = W^k, scaled:
+//   E = (a + conj b) / 2, O = (a - conj b) / 2, X[k] = E - i w O, X[4096 - k] = conj(E + i w O).
+__device__ __forceinline__ void split_pair(float2 a, float2 b, float2 w, float2& xk, float2& xm) {
+  const float h = 0.5f * PFB_SCALE;
+  const float2 e = make_float2(h * (a.x + b.x), h * (a.y - b.y));
+  const float2 od = make_float2(h * (a.x - b.x), h * (a.y + b.y));
+  const float2 wo = mul_mi(cmul(w, od));
+  xk = cadd(e, wo);
+  xm = make_float2(e.x - wo.x, wo.y - e.y);
 }
 
-// Split step: X[k] from Z[k] and Z[4096 - k], scaled, written to o[0 .. 4095].
-__device__ __forceinline__ void split_store(const float2* z, float2* __restrict__ o, int tid) {
-  if (tid == 0) {
-    const float2 z0 = z[sidx(0)];
-    o[0] = make_float2((z0.x + z0.y) * PFB_SCALE, 0.f);  // DC; the Nyquist bin (z0.x - z0.y) is not kept
-    const float2 zh = z[sidx(PFB_H / 2)];              // k = 2048: X = conj(Z[2048]) (W^2048 = -i)
-    o[PFB_H / 2] = make_float2(zh.x * PFB_SCALE, -zh.y * PFB_SCALE);
-  }
-  float2 wk[PFB_H / 2 / PFB_NT];  // this thread's split twiddles, loaded together
-#pragma unroll
-  for (int q = 0; q < PFB_H / 2 / PFB_NT; ++q) {
-    const int k = 1 + tid + q * PFB_NT;
-    wk[q] = k < PFB_H / 2 ? g_w8192[k] : make_float2(0.f, 0.f);
-  }
-#pragma unroll
-  for (int q = 0; q < PFB_H / 2 / PFB_NT; ++q) {
-    const int k = 1 + tid + q * PFB_NT;
-    if (k >= PFB_H / 2) break;
-    const float2 a = z[sidx(k)], b = z[sidx(PFB_H - k)];
-    const float2 w = wk[q];
-    const float2 wm = make_float2(-w.x, w.y);  // W^(4096 - k) = -conj(W^k)
-    // k: E = (a + conj b) / 2, O = (a - conj b) / 2, X[k] = E - i W^k O
-    {
-      const float2 e = make_float2(0.5f * (a.x + b.x), 0.5f * (a.y - b.y));
-      const float2 od = make_float2(0.5f * (a.x - b.x), 0.5f * (a.y + b.y));
-      const float2 wo = mul_mi(cmul(w, od));
-      o[k] = make_float2((e.x + wo.x) * PFB_SCALE, (e.y + wo.y) * PFB_SCALE);
-    }
-    // 4096 - k: roles of a and b swap
-    {
-      const float2 e = make_float2(0.5f * (b.x + a.x), 0.5f * (b.y - a.y));
-      const float2 od = make_float2(0.5f * (b.x - a.x), 0.5f * (b.y + a.y));
-      const float2 wo = mul_mi(cmul(wm, od));
-      o[PFB_H - k] = make_float2((e.x + wo.x) * PFB_SCALE, (e.y + wo.y) * PFB_SCALE);
-    }
-  }
+// Two samples of one frame (2-byte aligned) as a word, the second one in the high half.
+__device__ __forceinline__ int load2(const int8_t* __restrict__ p) {
+  return (int)__ldg(reinterpret_cast<const unsigned short*>(p));
 }
+__device__ __forceinline__ int byte0(int w) { return (int)(int8_t)(uint8_t)w; }
+__device__ __forceinline__ int byte1(int w) { return (int)(int8_t)(uint8_t)(w >> 8); }
 
-// 8 samples of one frame at p (8-byte aligned when vec8, else 4-byte aligned), as two words.
-__device__ __forceinline__ int2 load8(const int8_t* __restrict__ p, bool vec8) {
-  if (vec8) return __ldg(reinterpret_cast<const int2*>(p));
-  return make_int2(__ldg(reinterpret_cast<const int*>(p)), __ldg(reinterpret_cast<const int*>(p) + 1));
-}
-__device__ __forceinline__ int sbyte(int2 w, int k) {  // signed byte k (0..7) of w
-  const int v = k < 4 ? w.x : w.y;
-  return (int)(int8_t)(uint8_t)((unsigned)v >> (8 * (k & 3)));
-}
-__device__ __forceinline__ void fir_tap(int (&y)[8], const int4& c0, const int4& c1, int2 xs) {
-  y[0] += c0.x * sbyte(xs, 0);
-  y[1] += c0.y * sbyte(xs, 1);
-  y[2] += c0.z * sbyte(xs, 2);
-  y[3] += c0.w * sbyte(xs, 3);
-  y[4] += c1.x * sbyte(xs, 4);
-  y[5] += c1.y * sbyte(xs, 5);
-  y[6] += c1.z * sbyte(xs, 6);
-  y[7] += c1.w * sbyte(xs, 7);
-}
+// W32^q = exp(-2 pi i q / 32): W^(256 q), the split step's factor between a column's outputs
+__device__ constexpr float2 kW32[16] = {
+    {1.f, -0.f},
+    {0.98078528040323043f, -0.19509032201612825f},
+    {0.92387953251128674f, -0.38268343236508977f},
+    {0.83146961230254524f, -0.55557023301960218f},
+    {0.70710678118654757f, -0.70710678118654752f},
+    {0.55557023301960229f, -0.83146961230254524f},
+    {0.38268343236508984f, -0.92387953251128674f},
+    {0.19509032201612833f, -0.98078528040323043f},
+    {0.f, -1.f},
+    {-0.19509032201612819f, -0.98078528040323043f},
+    {-0.38268343236508973f, -0.92387953251128674f},
+    {-0.55557023301960196f, -0.83146961230254546f},
+    {-0.70710678118654746f, -0.70710678118654757f},
+    {-0.83146961230254535f, -0.55557023301960218f},
+    {-0.92387953251128674f, -0.38268343236508989f},
+    {-0.98078528040323043f, -0.19509032201612861f}};
 
-// One CTA per (input, pair of spectra t0, t0 + 1): the FIR of both spectra shares each coefficient
-// load and each frame load (frames t0 .. t0 + P), then each spectrum is transformed in its own shared
-// buffer. PT > 0 fixes the tap count at compile time (all loads of a step issued together); PT == 0
-// takes it from P.
+// PT > 0 fixes the tap count at compile time; PT == 0 takes it from P.
 template <int PT>
-__global__ void __launch_bounds__(PFB_NT, 3) pfb_kernel(const int8_t* __restrict__ adc, long long stride, int T,
-                                                        int P, bool vec8, const int* __restrict__ h,
-                                                        float2* __restrict__ out) {
+__global__ void __launch_bounds__(PFB_NT, 2) pfb_kernel(const int8_t* __restrict__ adc, long long stride, int T,
+                                                        int P, const int* __restrict__ h, float2* __restrict__ out) {
   extern __shared__ float2 zs[];  // PFB_SPB buffers of PFB_ZLEN
   const int t0 = blockIdx.x * PFB_SPB, n = blockIdx.y, tid = threadIdx.x;
   const int ns = T - t0 < PFB_SPB ? T - t0 : PFB_SPB;
-  const int8_t* x = adc + (size_t)n * stride + (size_t)t0 * PFB_M;
-  // FIR: thread handles samples m = 8 tid + 2048 j .. + 7 (j < 4), for both spectra
-#pragma unroll 1
-  for (int j = 0; j < PFB_M / (8 * PFB_NT); ++j) {
-    const int m = 8 * tid + 8 * PFB_NT * j;
-    int y[PFB_SPB][8];
+  float2 v[PFB_SPB][16];
+  // FIR: the thread's column of the first pass, points tid + 256 r, i.e. samples 2 tid + 512 r and the next,
+  // of both spectra: frames t0 .. t0 + P (the last one only if there is a second spectrum)
+  const int8_t* x = adc + (size_t)n * stride + (size_t)t0 * PFB_M + 2 * tid;
+  const int* hc = h + 2 * tid;
 #pragma unroll
-    for (int s = 0; s < PFB_SPB; ++s)
-#pragma unroll
-      for (int k = 0; k < 8; ++k) y[s][k] = 0;
+  for (int r = 0; r < 16; ++r) {
+    int y[PFB_SPB][2] = {{0, 0}, {0, 0}};
     if (PT > 0) {
-      int2 fr[PT + 1];  // frames t0 .. t0 + PT at m
+      int fr[PT + 1];
+      int2 c[PT > 0 ? PT : 1];
 #pragma unroll
-      for (int q = 0; q <= PT; ++q) fr[q] = q < PT || ns > 1 ? load8(x + (size_t)q * PFB_M + m, vec8) : make_int2(0, 0);
+      for (int q = 0; q <= PT; ++q) fr[q] = q < PT || ns > 1 ? load2(x + (size_t)q * PFB_M + 512 * r) : 0;
 #pragma unroll
-      for (int p = 0; p < PT; ++p) {
-        const int4* hp = reinterpret_cast<const int4*>(h + p * PFB_M + m);
-        const int4 c0 = __ldg(hp), c1 = __ldg(hp + 1);
-        fir_tap(y[0], c0, c1, fr[p]);
-        fir_tap(y[1], c0, c1, fr[p + 1]);
-      }
+      for (int p = 0; p < PT; ++p) c[p] = __ldg(reinterpret_cast<const int2*>(hc + p * PFB_M + 512 * r));
+#pragma unroll
+      for (int p = 0; p < PT; ++p)
+#pragma unroll
+        for (int s = 0; s < PFB_SPB; ++s) {
+          y[s][0] += c[p].x * byte0(fr[p + s]);
+          y[s][1] += c[p].y * byte1(fr[p + s]);
+        }
     } else {
-#pragma unroll 2
+      int f0 = load2(x + 512 * r);
       for (int p = 0; p < P; ++p) {
-        const int4* hp = reinterpret_cast<const int4*>(h + p * PFB_M + m);
-        const int4 c0 = __ldg(hp), c1 = __ldg(hp + 1);
-        fir_tap(y[0], c0, c1, load8(x + (size_t)p * PFB_M + m, vec8));
-        if (ns > 1) fir_tap(y[1], c0, c1, load8(x + (size_t)(p + 1) * PFB_M + m, vec8));
+        const int2 c = __ldg(reinterpret_cast<const int2*>(hc + p * PFB_M + 512 * r));
+        const int f1 = p + 1 < P || ns > 1 ? load2(x + (size_t)(p + 1) * PFB_M + 512 * r) : 0;
+        y[0][0] += c.x * byte0(f0);
+        y[0][1] += c.y * byte1(f0);
+        y[1][0] += c.x * byte0(f1);
+        y[1][1] += c.y * byte1(f1);
+        f0 = f1;
       }
     }
 #pragma unroll
-    for (int s = 0; s < PFB_SPB; ++s)
+    for (int s = 0; s < PFB_SPB; ++s) v[s][r] = make_float2((float)y[s][0], (float)y[s][1]);
+  }
+  // pass 1 (span 1): outputs 16 tid + q
 #pragma unroll
-      for (int q = 0; q < 4; ++q)
-        zs[s * PFB_ZLEN + sidx(m / 2 + q)] = make_float2((float)y[s][2 * q], (float)y[s][2 * q + 1]);
+  for (int s = 0; s < PFB_SPB; ++s) {
+    dft16(v[s]);
+#pragma unroll
+    for (int q = 0; q < 16; ++q) zs[s * PFB_ZLEN + sidx(16 * tid + q)] = v[s][q];
   }
   __syncthreads();
-  for (int s = 0; s < ns; ++s) {
-    fft4096(zs + s * PFB_ZLEN, tid);
-    split_store(zs + s * PFB_ZLEN, out + ((size_t)n * T + t0 + s) * PFB_H, tid);
+  // pass 2 (span 16): points tid + 256 r -> 16 (tid - k) + k + 16 q, k = tid mod 16
+  {
+    const int k = tid & 15, e = 16 * k;
+    const float2 w1 = g_w4096[e], w4 = g_w4096[4 * e], w8 = g_w4096[8 * e], w12 = g_w4096[12 * e];
+#pragma unroll
+    for (int s = 0; s < PFB_SPB; ++s)
+#pragma unroll
+      for (int r = 0; r < 16; ++r) v[s][r] = zs[s * PFB_ZLEN + sidx(tid + 256 * r)];
+    twiddle16<PFB_SPB>(v, w1, w4, w8, w12);
+    __syncthreads();
+    const int base = (tid - k) * 16 + k;
+#pragma unroll
+    for (int s = 0; s < PFB_SPB; ++s) {
+      dft16(v[s]);
+#pragma unroll
+      for (int q = 0; q < 16; ++q) zs[s * PFB_ZLEN + sidx(base + 16 * q)] = v[s][q];
+    }
+  }
+  __syncthreads();
+  // pass 3 (span 256) and split step: threads 128 s .. + 127 take spectrum s, thread u columns u and 256 - u
+  // (thread 0: columns 0 and 128, each its own mirror image)
+  const int s = tid >> 7, u = tid & 127;
+  if (s >= ns) return;
+  const int cb = u ? 256 - u : 128, eb = u ? u : 128;
+  const float2* z = zs + s * PFB_ZLEN;
+  float2 c2[1][16], d2[1][16];
+  float2(&za)[16] = c2[0];
+  float2(&zb)[16] = d2[0];
+  {
+    const float2 w1 = g_w4096[u], w4 = g_w4096[4 * u], w8 = g_w4096[8 * u], w12 = g_w4096[12 * u];
+#pragma unroll
+    for (int r = 0; r < 16; ++r) za[r] = z[sidx(u + 256 * r)];
+    twiddle16<1>(c2, w1, w4, w8, w12);
+    dft16(za);  // za[q] = Z[u + 256 q]
+  }
+  {
+    // column 256 - u: exp(-2 pi i (256 - u) r / 4096) = W16^r conj(w^r); the factor W16^r advances the outputs
+    // by one: zb[q] = Z[cb + 256 ((q + 15) mod 16)] (also with eb = 128 for column 128)
+    const float2 w1 = conjf2(g_w4096[eb]), w4 = conjf2(g_w4096[4 * eb]), w8 = conjf2(g_w4096[8 * eb]),
+                 w12 = conjf2(g_w4096[12 * eb]);
+#pragma unroll
+    for (int r = 0; r < 16; ++r) zb[r] = z[sidx(cb + 256 * r)];
+    twiddle16<1>(d2, w1, w4, w8, w12);
+    dft16(zb);
+  }
+  float2* o = out + ((size_t)n * T + t0 + s) * PFB_H;
+  if (u != 0) {
+    const float2 w = g_w8192[u];
+#pragma unroll
+    for (int q = 0; q < 16; ++q) {  // k = u + 256 q, 4096 - k = 256 - u + 256 (15 - q)
+      float2 xk, xm;
+      split_pair(za[q], zb[(16 - q) & 15], cmul(w, kW32[q]), xk, xm);
+      o[u + 256 * q] = xk;
+      o[PFB_H - u - 256 * q] = xm;
+    }
+  } else {
+    o[0] = make_float2((za[0].x + za[0].y) * PFB_SCALE, 0.f);  // DC; the Nyquist bin (x - y) is not kept
+    o[PFB_H / 2] = make_float2(za[8].x * PFB_SCALE, -za[8].y * PFB_SCALE);  // k = 2048: W^2048 = -i
+#pragma unroll
+    for (int q = 1; q < 8; ++q) {  // k = 256 q, 4096 - k = 256 (16 - q)
+      float2 xk, xm;
+      split_pair(za[q], za[16 - q], kW32[q], xk, xm);
+      o[256 * q] = xk;
+      o[PFB_H - 256 * q] = xm;
+    }
+    const float2 w = g_w8192[128];
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {  // k = 128 + 256 q, 4096 - k = 128 + 256 (15 - q)
+      float2 xk, xm;
+      split_pair(zb[q + 1], zb[(16 - q) & 15], cmul(w, kW32[q]), xk, xm);
+      o[128 + 256 * q] = xk;
+      o[PFB_H - 128 - 256 * q] = xm;
+    }
   }
 }
 
@@ -266,16 +299,15 @@ cudaError_t launch_pfb(const int8_t* d_adc, long long stride, int N, int T, int 
   if (e == cudaSuccess) e = ensure_twiddles(dev);
   if (e != cudaSuccess) return e;
   constexpr int smem = PFB_SPB * PFB_ZLEN * (int)sizeof(float2);
-  const bool vec8 = ((reinterpret_cast<uintptr_t>(d_adc) | (uintptr_t)stride) & 7) == 0;
   const dim3 grid((unsigned)((T + PFB_SPB - 1) / PFB_SPB), (unsigned)N);
   if (P == 4) {
     e = set_smem_limit(reinterpret_cast<const void*>(pfb_kernel<4>), smem);
     if (e != cudaSuccess) return e;
-    pfb_kernel<4><<<grid, PFB_NT, smem, st>>>(d_adc, stride, T, P, vec8, d_h, d_out);
+    pfb_kernel<4><<<grid, PFB_NT, smem, st>>>(d_adc, stride, T, P, d_h, d_out);
   } else {
     e = set_smem_limit(reinterpret_cast<const void*>(pfb_kernel<0>), smem);
     if (e != cudaSuccess) return e;
-    pfb_kernel<0><<<grid, PFB_NT, smem, st>>>(d_adc, stride, T, P, vec8, d_h, d_out);
+    pfb_kernel<0><<<grid, PFB_NT, smem, st>>>(d_adc, stride, T, P, d_h, d_out);
   }
   return cudaGetLastError();
 }
