@@ -281,8 +281,7 @@ enum Route { ROUTE_TWO_PASS, ROUTE_DIRECT, ROUTE_REPACK };
 
 int repacked_inputs(const corr_ctx* c) { return (int)round_up(c->L.s.N, 16); }
 
-Route route_of(const corr_ctx* c, const uint8_t* d_in) {
-  if (c->tile_plan != c->plan_default || c->prep_sms > 0) return ROUTE_TWO_PASS;
+Route direct_route(const corr_ctx* c, const uint8_t* d_in) {
   const Shape& s = c->L.s;
   if (xeng_small_supported(s, s.N, d_in) || xeng_direct_supported(s, s.N, d_in)) return ROUTE_DIRECT;
   const int Np = repacked_inputs(c);
@@ -290,23 +289,33 @@ Route route_of(const corr_ctx* c, const uint8_t* d_in) {
   return ROUTE_TWO_PASS;
 }
 
-// n blocks of T_blk samples, all of one of the direct routes, in as many launches as `most` blocks a launch make.
-int accumulate_direct(corr_ctx* c, const uint8_t* const* blocks, int n, int T_blk, int most, Route route, cudaStream_t st) {
+Route route_of(const corr_ctx* c, const uint8_t* d_in) {
+  return c->tile_plan != c->plan_default || c->prep_sms > 0 ? ROUTE_TWO_PASS : direct_route(c, d_in);
+}
+
+DirectJob direct_job(const corr_ctx* c, int T_blk, Route route) {
   DirectJob j;
   j.s = c->L.s;
+  j.blocks = nullptr;
+  j.n = 0;
   j.T_blk = T_blk;
-  j.ld = c->L.s.N;
+  j.ld = route == ROUTE_REPACK ? repacked_inputs(c) : c->L.s.N;
   j.flush_len = flush_for(c, CORR_PATH_FP8TC);
   j.cross = c->d_cross;
   j.autos = c->d_autos;
   j.s1 = c->d_soff;
   j.s2 = c->d_soff_auto;
   j.err = c->d_err;
+  return j;
+}
+
+// n blocks of T_blk samples, all of one of the direct routes, in as many launches as `most` blocks a launch make.
+int accumulate_direct(corr_ctx* c, const uint8_t* const* blocks, int n, int T_blk, int most, Route route, cudaStream_t st) {
+  DirectJob j = direct_job(c, T_blk, route);
   int K = std::min(most, direct_max_blocks(T_blk));
   const uint8_t* packed[xd::MAX_BLOCKS];
   const long long rows = (long long)T_blk * c->L.s.C;
   if (route == ROUTE_REPACK) {  // in the operand scratch, which holds twice as many blocks' samples
-    j.ld = repacked_inputs(c);
     K = (int)std::min<long long>(K, (long long)(c->L.op_buf_bytes / ((size_t)rows * j.ld)));
     for (int i = 0; i < K; ++i) packed[i] = c->d_op + (size_t)i * rows * j.ld;
   }
@@ -329,6 +338,50 @@ int accumulate_direct(corr_ctx* c, const uint8_t* const* blocks, int n, int T_bl
     c->n_off += (long long)T_blk * j.n;
     c->n_off_auto += (long long)T_blk * j.n;
   }
+  return CORR_OK;
+}
+
+// One block of every array: the operand work first (repacked rows; where an array takes neither direct route the
+// two-pass build), then the X-engines one behind the other. Counts nothing: a captured launch is counted when
+// it is replayed. Timed and its waits reported on the first array, flushed by its period.
+int enqueue_group(corr_ctx* const* ctx, int n, const uint8_t* const* in, cudaStream_t st) {
+  corr_ctx* c0 = ctx[0];
+  const int flush = flush_for(c0, CORR_PATH_FP8TC);
+  bool tb = timer_begin(c0, CORR_KERNEL_UNPACK, st);
+  for (int i = 0; i < n; ++i) {
+    corr_ctx* c = ctx[i];
+    const Shape& s = c->L.s;
+    const Route route = direct_route(c, in[i]);
+    cudaError_t e = cudaSuccess;
+    if (route == ROUTE_REPACK)
+      e = launch_repack(in[i], (long long)s.T * s.C, s.N, repacked_inputs(c), c->d_op, st);
+    else if (route == ROUTE_TWO_PASS)
+      e = launch_f8_prep(s, in[i], s.T, c->L.T_pad, c->L.T_pad * c->L.K_batch, 0, c->L.R_buf, c->d_op, c->d_soff,
+                         c->d_soff_auto, st);
+    if (e != cudaSuccess) return cuda_fail(e, "group operand build");
+  }
+  timer_end(c0, CORR_KERNEL_UNPACK, st, tb);
+  tb = timer_begin(c0, CORR_KERNEL_XENG, st);
+  for (int i = 0; i < n; ++i) {
+    corr_ctx* c = ctx[i];
+    const Route route = direct_route(c, in[i]);
+    cudaError_t e;
+    if (route == ROUTE_TWO_PASS) {
+      XengArgs a = xeng_args(c, 0, c->L.T_pad, flush);
+      a.err = c0->d_err;
+      e = launch_f8_xeng(a, c->num_sms, st);
+    } else {
+      const uint8_t* block = route == ROUTE_REPACK ? c->d_op : in[i];
+      DirectJob j = direct_job(c, c->L.s.T, route);
+      j.blocks = &block;
+      j.n = 1;
+      j.flush_len = flush;
+      j.err = c0->d_err;
+      e = c->L.s.N <= 64 ? launch_xeng_small(j, c->num_sms, st) : launch_xeng_direct(j, c->num_sms, st);
+    }
+    if (e != cudaSuccess) return cuda_fail(e, "group x-engine launch");
+  }
+  timer_end(c0, CORR_KERNEL_XENG, st, tb);
   return CORR_OK;
 }
 

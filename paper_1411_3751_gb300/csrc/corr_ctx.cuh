@@ -113,6 +113,8 @@ int set_batch_blocks(corr_ctx* c, int K);
 int max_batch_blocks(const corr_ctx* c);
 // n device blocks through the two-pass tensor path (batch schedule of the context's settings)
 int accumulate_batch_chunks(corr_ctx* c, const uint8_t* const* blocks, int n, cudaStream_t st);
+// one block in[i] of each of n arrays through the tensor path (no counting; any tile plan)
+int enqueue_group(corr_ctx* const* ctx, int n, const uint8_t* const* in, cudaStream_t st);
 // T_blk samples of a device block [T_blk][C][N] through the context's current path
 int accumulate_device(corr_ctx* c, const uint8_t* d_in, int T_blk, cudaStream_t st);
 

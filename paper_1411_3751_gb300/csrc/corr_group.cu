@@ -1,5 +1,5 @@
 // Groups of sub-arrays of the C ABI (corr_group_*): several contexts of different N and C with one
-// block length, correlated by one persistent tensor-core launch over all their work items.
+// block length, correlated by one call.
 #include <algorithm>
 #include <cstdio>
 #include <cstdlib>
@@ -17,16 +17,9 @@
 using namespace corr;
 using namespace corr::host;
 
-// =============================================================================================
-// Groups of sub-arrays (different N and C, one block length): one persistent tensor-core launch
-// covers the work items of every sub-array; per-array tile plans come from a small autotuner.
-// =============================================================================================
-
 struct corr_group {
   int n;
   corr_ctx* ctx[kMaxGroupArrays];
-  WorkItem* d_items;
-  long long n_items;
   cudaGraphExec_t graph;
   int T;
 };
@@ -65,94 +58,13 @@ void tune_store(const std::tuple<int, int, int, int, int>& k, int plan) {
   std::fclose(fh);
 }
 
-// Group work list: arrays in order of decreasing N (largest tiles first, the short items of small
-// arrays last, where they even out the tail), each channel-major. (Merging the arrays in proportion
-// to their channel counts, so that HBM-bound small-array items run beside tensor-bound large ones,
-// measured the same: 0.638 against 0.641 ms for 32-512 inputs x 2400-109 channels x 4096 samples,
-// whose X-engine time is the MMA issue of the 200-512-input members.)
-int group_build_items(corr_group* g) {
-  std::vector<int> order(g->n);
-  for (int i = 0; i < g->n; ++i) order[i] = i;
-  std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return g->ctx[x]->L.s.N > g->ctx[y]->L.s.N; });
-  std::vector<WorkItem> items;
-  for (int i : order) {
-    corr_ctx* c = g->ctx[i];
-    // group launches run the one-SM mode: a member on plan 2 or 3 joins with plan 0; members of at
-    // most 32 inputs as channel groups
-    if (channel_group(c->L) > 0) {
-      for (int f = 0; f < c->L.s.C; f += channel_group(c->L)) items.push_back(WorkItem{i, f, 0, 0, 128, 0});
-      continue;
-    }
-    const std::vector<F8Tile> t8 = f8_tile_plan(c->L.s.N, c->L.R, c->tile_plan >= 2 ? 0 : c->tile_plan);
-    for (int f = 0; f < c->L.s.C; ++f)
-      for (const F8Tile& t : t8) items.push_back(WorkItem{i, f, t.c0, t.a0, t.nb, 0});
-  }
-  WorkItem* d = nullptr;
-  if (cudaMalloc(&d, items.size() * sizeof(WorkItem)) != cudaSuccess) {
-    cudaGetLastError();
-    return fail(CORR_ERR_OOM, "group work list allocation failed");
-  }
-  cudaError_t e = cudaMemcpy(d, items.data(), items.size() * sizeof(WorkItem), cudaMemcpyHostToDevice);
-  if (e != cudaSuccess) {
-    cudaFree(d);
-    return cuda_fail(e, "group work list upload");
-  }
-  cudaFree(g->d_items);
-  g->d_items = d;
-  g->n_items = (long long)items.size();
-  return CORR_OK;
-}
-
-// One grouped accumulate: one operand-build launch over all arrays, then one persistent X-engine launch.
+// One grouped accumulate.
 int group_enqueue(corr_group* g, const uint8_t* const* in, cudaStream_t st) {
-  corr_ctx* c0 = g->ctx[0];
-  const int T_pad = c0->L.T_pad;
-  XengArgs a;
-  std::memset(&a, 0, sizeof(a));
   for (int i = 0; i < g->n; ++i)
     if (!g->ctx[i]->d_op)
       return fail(CORR_ERR_STATE, "group member " + std::to_string(i) +
                                       " has no operand scratch (its path was set to FP32 or int8; set a tensor path)");
-  // every member's operand build in one launch
-  PrepJobDesc jobs[kMaxGroupArrays];
-  for (int i = 0; i < g->n; ++i) {
-    corr_ctx* c = g->ctx[i];
-    jobs[i].s = c->L.s;
-    jobs[i].in = in[i];
-    jobs[i].T_stride = c->L.T_pad * c->L.K_batch;
-    jobs[i].t_base = 0;
-    jobs[i].R = c->L.R_buf;
-    jobs[i].op = c->d_op;
-    jobs[i].s1 = c->d_soff;
-    jobs[i].s2 = c->d_soff_auto;
-  }
-  {
-    const bool tb = timer_begin(c0, CORR_KERNEL_UNPACK, st);
-    const cudaError_t e = launch_f8_prep_group(jobs, g->n, c0->L.s.T, T_pad, st);
-    timer_end(c0, CORR_KERNEL_UNPACK, st, tb);
-    if (e != cudaSuccess) return cuda_fail(e, "group operand build");
-  }
-  for (int i = 0; i < g->n; ++i) {
-    corr_ctx* c = g->ctx[i];
-    a.a[i].tmap = channel_group(c->L) > 0 ? c->tmap_cp : c->tmap;
-    a.a[i].cgroup = channel_group(c->L);
-    a.a[i].C = c->L.s.C;
-    a.a[i].cross = c->d_cross;
-    a.a[i].autos = c->d_autos;
-    a.a[i].Bs = c->L.s.Bs;
-    a.a[i].N = c->L.s.N;
-    a.a[i].npol = c->L.s.npol;
-  }
-  a.items = g->d_items;
-  a.n_items = g->n_items;
-  a.T_run = T_pad;
-  a.flush_len = flush_for(c0, CORR_PATH_FP8TC);
-  a.err = c0->d_err;
-  const bool tb = timer_begin(c0, CORR_KERNEL_XENG, st);
-  cudaError_t e = launch_f8_xeng(a, c0->num_sms, st);
-  timer_end(c0, CORR_KERNEL_XENG, st, tb);
-  if (e != cudaSuccess) return cuda_fail(e, "group x-engine launch");
-  return CORR_OK;
+  return enqueue_group(g->ctx, g->n, in, st);
 }
 
 void group_count(corr_group* g) {
@@ -189,12 +101,6 @@ corr_group* corr_group_create(int n_arrays, const int* n_inputs, const int* n_ch
       fail(CORR_ERR_ARG, "corr_group_create: sub-array " + std::to_string(i) + ": " + msg);
       return nullptr;
     }
-  }
-  if (group_build_items(g) != CORR_OK) {
-    const std::string msg = corr_last_error();
-    corr_group_destroy(g);
-    fail(CORR_ERR_OOM, "corr_group_create: " + msg);
-    return nullptr;
   }
   return g;
 }
@@ -271,12 +177,12 @@ int corr_group_autotune(corr_group* g, const void* const* d_samples, int* plans_
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
   if (rc != CORR_OK) return rc;
-  // a captured graph refers to the old work list: drop it (corr_group_capture records a new one)
+  // a captured graph would keep the old plans' launches: drop it (corr_group_capture records a new one)
   if (g->graph) {
     cudaGraphExecDestroy(g->graph);
     g->graph = nullptr;
   }
-  return group_build_items(g);
+  return CORR_OK;
 }
 
 int corr_group_capture(corr_group* g, const void* const* d_samples, void* stream) {
@@ -323,7 +229,6 @@ int corr_group_destroy(corr_group* g) {
   if (!g) return CORR_OK;
   int rc = CORR_OK;
   if (g->graph) cudaGraphExecDestroy(g->graph);
-  cudaFree(g->d_items);
   for (int i = 0; i < g->n; ++i)
     if (g->ctx[i] && corr_destroy(g->ctx[i]) != CORR_OK) rc = CORR_ERR_CUDA;
   delete g;

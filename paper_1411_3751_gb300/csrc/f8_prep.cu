@@ -2,8 +2,6 @@
 // the GPU): packed bytes in[T][C][N] -> op[C][T_pad][R] (offset e4m3 bytes, group row order, MN-major:
 // one contiguous row of R bytes per channel and sample) plus the per-input offset sums. Streams
 // through HBM. Operand encoding and row order: f8_common.cuh.
-#include <cstring>
-
 #include "corr_internal.cuh"
 #include "f8_common.cuh"
 
@@ -25,11 +23,12 @@ using namespace f8;
 //    int64 sums with one atomic per input and block.
 constexpr int PREP_ROWS_PER_THREAD_MAX = 2048;
 
-// The build of one block (bx, bz) of the grid: bx picks 8 units, bz the time range.
-__device__ __forceinline__ void prep_block(const uint8_t* __restrict__ in, int N, int C, int T, int T_run, int T_stride,
-                                           int t_base, int R, int rows_per_split, int vec, uint8_t* __restrict__ op,
-                                           long long* __restrict__ s1, long long* __restrict__ s2, long long bx,
-                                           int bz) {
+__global__ void __launch_bounds__(256) f8_prep_kernel(const uint8_t* __restrict__ in, int N, int C, int T, int T_run,
+                                                      int T_stride, int t_base, int R, int rows_per_split, int vec,
+                                                      uint8_t* __restrict__ op, long long* __restrict__ s1,
+                                                      long long* __restrict__ s2) {
+  const long long bx = blockIdx.x;  // 8 units
+  const int bz = blockIdx.z;        // time range
   const int G = R / 32;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int tl = lane >> 3, us = lane & 7;
@@ -141,38 +140,6 @@ __device__ __forceinline__ void prep_block(const uint8_t* __restrict__ in, int N
   }
 }
 
-__global__ void __launch_bounds__(256) f8_prep_kernel(const uint8_t* __restrict__ in, int N, int C, int T, int T_run,
-                                                      int T_stride, int t_base, int R, int rows_per_split, int vec,
-                                                      uint8_t* __restrict__ op, long long* __restrict__ s1,
-                                                      long long* __restrict__ s2) {
-  prep_block(in, N, C, T, T_run, T_stride, t_base, R, rows_per_split, vec, op, s1, s2, blockIdx.x, blockIdx.z);
-}
-
-// Several arrays' builds in one launch (groups of sub-arrays): job i owns the linear blocks
-// [blk0_i, blk0_{i+1}), gx_i unit blocks by its time split, as its own launch would lay them out.
-struct PrepJob {
-  const uint8_t* in;
-  uint8_t* op;
-  long long* s1;
-  long long* s2;
-  long long blk0;
-  int N, C, R, T_stride, t_base, rows, gx, vec;
-};
-struct PrepGroupArgs {
-  PrepJob job[kMaxGroupArrays];
-  int n, T, T_run;
-};
-
-__global__ void __launch_bounds__(256) f8_prep_group_kernel(const __grid_constant__ PrepGroupArgs a) {
-  const long long b = blockIdx.x;
-  int i = 0;
-  while (i + 1 < a.n && b >= a.job[i + 1].blk0) ++i;
-  const PrepJob& j = a.job[i];
-  const long long local = b - j.blk0;
-  prep_block(j.in, j.N, j.C, a.T, a.T_run, j.T_stride, j.t_base, j.R, j.rows, j.vec, j.op, j.s1, j.s2,
-             local % j.gx, (int)(local / j.gx));
-}
-
 // Widest load (16, 8 or 4 bytes, else 1) that keeps every unit's 16 input bytes aligned: the rows of
 // in[T][C][N] start at multiples of N bytes.
 int load_width(int N, const void* in) {
@@ -201,42 +168,6 @@ void prep_geometry(const Shape& s, int T_run, int R, long long* gx, int* split_o
 }
 
 }  // namespace
-
-cudaError_t launch_f8_prep_group(const PrepJobDesc* jobs, int n, int T_blk, int T_run, cudaStream_t st) {
-  if (T_run == 0 || n <= 0) return cudaSuccess;
-  if (n > kMaxGroupArrays) return cudaErrorInvalidValue;
-  PrepGroupArgs a;
-  std::memset(&a, 0, sizeof(a));
-  a.n = n;
-  a.T = T_blk;
-  a.T_run = T_run;
-  long long blocks = 0;
-  for (int i = 0; i < n; ++i) {
-    const PrepJobDesc& d = jobs[i];
-    PrepJob& j = a.job[i];
-    int split = 1, rows = 0;
-    long long gx = 0;
-    prep_geometry(d.s, T_run, d.R, &gx, &split, &rows);
-    j.in = d.in;
-    j.op = d.op;
-    j.s1 = d.s1;
-    j.s2 = d.s2;
-    j.blk0 = blocks;
-    j.N = d.s.N;
-    j.C = d.s.C;
-    j.R = d.R;
-    j.T_stride = d.T_stride;
-    j.t_base = d.t_base;
-    j.rows = rows;
-    j.gx = (int)gx;
-    j.vec = load_width(d.s.N, d.in);
-    blocks += gx * split;
-  }
-  if (blocks == 0) return cudaSuccess;
-  if (blocks > 0x7FFFFFFFLL) return cudaErrorInvalidConfiguration;
-  f8_prep_group_kernel<<<(unsigned)blocks, 256, 0, st>>>(a);
-  return cudaGetLastError();
-}
 
 cudaError_t launch_f8_prep(const Shape& s, const uint8_t* d_in, int T_blk, int T_run, int T_stride, int t_base, int R,
                            uint8_t* d_op, long long* d_s1, long long* d_s2, cudaStream_t st) {
