@@ -92,6 +92,11 @@ __device__ __forceinline__ void tma_load_2d(void* smem_dst, const CUtensorMap* m
       : "memory");
 }
 
+// Bring `bytes` (a multiple of 16, from a 16-byte boundary) into L2.
+__device__ __forceinline__ void prefetch_l2(const void* g, uint32_t bytes) {
+  asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(g), "r"(bytes) : "memory");
+}
+
 // ---- ldmatrix -------------------------------------------------------------------------------
 // Two 16 x 16 byte matrices (rows at the addresses of lanes 0-15 and 16-31), transposed: lane l gets in
 // register 2 m + h the bytes of matrix m's column l / 4 + 8 h, rows 4 (l % 4) .. + 3.

@@ -87,6 +87,22 @@ struct Item {
   }
 };
 
+// The item's cells of this CTA into L2 while its MMAs run: for each a-station one run of the 64 c-inputs' products,
+// so that the loads of the old sums wait for L2 and not for DRAM. Short integrations are bound by the epilogue:
+// 512 inputs x 2400 channels x 240 samples 3.58 ms, 3.27 with the prefetch, 2.87 with the combined chunks below.
+__device__ __forceinline__ void prefetch_cells(const xd::Args& a, const Item& it, uint32_t rank, int w, int lane, int lp,
+                                               const long long* cross_f) {
+  const int sc0 = (it.c0 + 64 * (int)rank) >> lp, n_sc = 64 >> lp, S = a.N >> lp;
+  for (int i = 32 * w + lane; i < 128 >> lp; i += 32 * D_EPI_WARPS) {
+    const int sa = (it.a0 >> lp) + i;
+    const int end = min(min(sc0 + n_sc, sa + 1), S);
+    if (sa < S && sc0 < end) {
+      const unsigned b = (unsigned)sa * (unsigned)(sa + 1) / 2 + (unsigned)sc0;
+      ptx::prefetch_l2(cross_f + 2 * ((long long)b << (2 * lp)), (uint32_t)(end - sc0) << (4 + 2 * lp));
+    }
+  }
+}
+
 template <bool ADD>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(D_THREADS, 1)
     xeng_direct_kernel(const __grid_constant__ xd::Args args) {
@@ -349,6 +365,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(D_THREADS, 1)
       const int c = it.c0 + 64 * (int)rank + 16 * q + (lane & 15);
       long long* cross_f = args.cross + (long long)it.f * args.Bs * args.npol * args.npol * 2;
       long long* autos_f = args.autos + (long long)it.f * args.N;
+      prefetch_cells(args, it, rank, warp - 12, lane, lp, cross_f);
       for (int k0 = it.k0; k0 < it.k1; k0 += chunk_k) {
         if (__any_sync(0xffffffffu, *abort_flag != 0)) {
           ok = false;
@@ -370,13 +387,17 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(D_THREADS, 1)
         __syncwarp();
         if (lane == 0) ptx::mbar_arrive_remote(ptx::mapa_shared(tempty, 0));
         ++use;
+        int re[4][8], im[4][8];
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {  // the first chunk has 128 accumulator words beside it, the others room
+        for (int j = 0; j < 4; ++j) xd::combine_chunk<16>(v[j], im_lane, re[j], im[j]);
+        const int c_min = it.c0 + 64 * (int)rank + 16 * q, c_max = c_min + 15;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
           const int a_base = it.a0 + 64 * half + 16 * j;
-          if (j == 0)
-            xd::add_chunk<16, ADD, 4>(v[j], im_lane, c, a_base, args.N, lp, cross_f, autos_f);
-          else
-            xd::add_chunk<16, ADD, 8>(v[j], im_lane, c, a_base, args.N, lp, cross_f, autos_f);
+          if (lp == 1 && a_base > c_max && a_base + 16 <= args.N && c_max < args.N)
+            xd::add_chunk_full<ADD>(re[j], im[j], im_lane, c, a_base, cross_f);
+          else if (a_base + 15 >= c_min - lp && a_base < args.N && c_min < args.N)  // not all above the diagonal or past N
+            xd::add_chunk<ADD>(re[j], im[j], im_lane, c, a_base, args.N, lp, cross_f, autos_f);
         }
       }
     }

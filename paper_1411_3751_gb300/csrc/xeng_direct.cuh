@@ -28,63 +28,88 @@ struct Args {
   int* err;
 };
 
-// Adds one 32-column chunk of an accumulator (16 a-inputs from a_base: column 8 (k / 4) + k % 4 = Re a_k, + 4 =
-// Im a_k) to cross[f] and, on the diagonal, autos[f]. The lanes holding Re c and Im c of one c-input are
-// XOR apart; they exchange half of their columns and own 8 a-inputs each. ADD: 64-bit reductions (items
-// that share cells), else load, add, store, G (4 or 8) cells in flight.
-template <int XOR, bool ADD, int G>
-__device__ __forceinline__ void add_chunk(const uint32_t (&v)[32], bool im_lane, int c, int a_base, int N, int lp,
-                                          long long* __restrict__ cross_f, long long* __restrict__ autos_f) {
-  // lp = log2(n_pol): station n >> lp, polarisation n & lp (n_pol is 1 or 2)
+// One 32-column chunk of an accumulator (16 a-inputs: column 8 (k / 4) + k % 4 = Re a_k, + 4 = Im a_k) as complex
+// products: the lanes holding Re c and Im c of one c-input are XOR apart, exchange half of their columns and own
+// 8 a-inputs each, the Re lane the even, the Im lane the odd ones. (With two polarisations a warp's access then
+// covers whole station pairs, 512 neighbouring bytes.) Combining all of an accumulator first halves the words a
+// thread holds, and leaves registers for eight cells in flight.
+template <int XOR>
+__device__ __forceinline__ void combine_chunk(const uint32_t (&v)[32], bool im_lane, int (&re)[8], int (&im)[8]) {
+#pragma unroll
+  for (int k = 0; k < 8; ++k) {
+    const int jr = 8 * (k >> 1) + 2 * (k & 1), ji = jr + 4;  // columns of the even input; the odd one's follow
+    const int own_r = f8::to_int(__uint_as_float(im_lane ? v[jr + 1] : v[jr]));
+    const int own_i = f8::to_int(__uint_as_float(im_lane ? v[ji + 1] : v[ji]));
+    const int recv_r = f8::to_int(__shfl_xor_sync(0xffffffffu, __uint_as_float(im_lane ? v[jr] : v[jr + 1]), XOR));
+    const int recv_i = f8::to_int(__shfl_xor_sync(0xffffffffu, __uint_as_float(im_lane ? v[ji] : v[ji + 1]), XOR));
+    // Re lane: own row Re c, partner Im c; Im lane the other way round
+    re[k] = im_lane ? recv_r + own_i : own_r + recv_i;
+    im[k] = im_lane ? recv_i - own_r : own_i - recv_r;
+  }
+}
+
+template <bool ADD>
+__device__ __forceinline__ void add_cells(longlong2* const (&cell)[8], uint32_t valid, const int (&re)[8], const int (&im)[8]) {
+  if (ADD) {
+#pragma unroll
+    for (int m = 0; m < 8; ++m)
+      if (valid & (1u << m)) {
+        atomicAdd(reinterpret_cast<unsigned long long*>(cell[m]), (unsigned long long)(long long)re[m]);
+        atomicAdd(reinterpret_cast<unsigned long long*>(cell[m]) + 1, (unsigned long long)(long long)im[m]);
+      }
+  } else {
+    longlong2 old[8];
+#pragma unroll
+    for (int m = 0; m < 8; ++m) old[m] = *cell[m];
+#pragma unroll
+    for (int m = 0; m < 8; ++m)
+      if (valid & (1u << m)) *cell[m] = make_longlong2(old[m].x + re[m], old[m].y + im[m]);
+  }
+}
+
+// Adds a combined chunk of a-inputs from a_base (the lane's own a_base + im_lane + 2 k) to cross[f] and, on the
+// diagonal, autos[f]. ADD: 64-bit reductions (items that share cells), else load, add, store.
+// lp = log2(n_pol): station n >> lp, polarisation n & lp (n_pol is 1 or 2).
+template <bool ADD>
+__device__ __forceinline__ void add_chunk(const int (&re)[8], const int (&im)[8], bool im_lane, int c, int a_base, int N,
+                                          int lp, long long* __restrict__ cross_f, long long* __restrict__ autos_f) {
   const unsigned sc = (unsigned)c >> lp, pc = (unsigned)c & (unsigned)lp;
+  longlong2* cell[8];
+  uint32_t valid = 0u;
 #pragma unroll
-  for (int k0 = 0; k0 < 8; k0 += G) {
-    int re[G], im[G];
-    long long* cell[G];
-    uint32_t valid = 0u;
-#pragma unroll
-    for (int m = 0; m < G; ++m) {
-      const int k = k0 + m, jr = 8 * (k >> 2) + (k & 3), ji = jr + 4;  // columns of a_k within the 16 kept
-      const float own_r = __uint_as_float(im_lane ? v[16 + jr] : v[jr]);
-      const float own_i = __uint_as_float(im_lane ? v[16 + ji] : v[ji]);
-      const float recv_r = __shfl_xor_sync(0xffffffffu, __uint_as_float(im_lane ? v[jr] : v[16 + jr]), XOR);
-      const float recv_i = __shfl_xor_sync(0xffffffffu, __uint_as_float(im_lane ? v[ji] : v[16 + ji]), XOR);
-      // Re lane: own row Re c, partner Im c; Im lane the other way round
-      re[m] = im_lane ? f8::to_int(recv_r) + f8::to_int(own_i) : f8::to_int(own_r) + f8::to_int(recv_i);
-      im[m] = im_lane ? f8::to_int(recv_i) - f8::to_int(own_r) : f8::to_int(own_i) - f8::to_int(recv_r);
-      const int a = a_base + (im_lane ? 8 : 0) + k;
-      cell[m] = cross_f;  // in-bounds placeholder for skipped cells (loaded, never stored)
-      if (a >= 0 && a < N && c >= 0 && c < N) {
-        const unsigned sa = (unsigned)a >> lp;
-        if (sa >= sc) {
-          const unsigned b = sa * (sa + 1) / 2 + sc;
-          cell[m] = cross_f + 2 * (((long long)b << (2 * lp)) + ((((unsigned)a & (unsigned)lp) << lp) + pc));
-          valid |= 1u << m;
-          if (a == c) {
-            if (ADD)
-              atomicAdd(reinterpret_cast<unsigned long long*>(autos_f + a), (unsigned long long)(long long)re[m]);
-            else
-              autos_f[a] += re[m];
-          }
+  for (int k = 0; k < 8; ++k) {
+    const int a = a_base + (im_lane ? 1 : 0) + 2 * k;
+    cell[k] = reinterpret_cast<longlong2*>(cross_f);  // in-bounds placeholder for skipped cells (loaded, never stored)
+    if (a >= 0 && a < N && c >= 0 && c < N) {
+      const unsigned sa = (unsigned)a >> lp;
+      if (sa >= sc) {
+        const unsigned b = sa * (sa + 1) / 2 + sc;
+        cell[k] += ((long long)b << (2 * lp)) + ((((unsigned)a & (unsigned)lp) << lp) + pc);
+        valid |= 1u << k;
+        if (a == c) {
+          if (ADD)
+            atomicAdd(reinterpret_cast<unsigned long long*>(autos_f + a), (unsigned long long)(long long)re[k]);
+          else
+            autos_f[a] += re[k];
         }
       }
     }
-    if (ADD) {
-#pragma unroll
-      for (int m = 0; m < G; ++m)
-        if (valid & (1u << m)) {
-          atomicAdd(reinterpret_cast<unsigned long long*>(cell[m]), (unsigned long long)(long long)re[m]);
-          atomicAdd(reinterpret_cast<unsigned long long*>(cell[m]) + 1, (unsigned long long)(long long)im[m]);
-        }
-    } else {
-      longlong2 old[G];
-#pragma unroll
-      for (int m = 0; m < G; ++m) old[m] = *reinterpret_cast<const longlong2*>(cell[m]);
-#pragma unroll
-      for (int m = 0; m < G; ++m)
-        if (valid & (1u << m)) *reinterpret_cast<longlong2*>(cell[m]) = make_longlong2(old[m].x + re[m], old[m].y + im[m]);
-    }
   }
+  add_cells<ADD>(cell, valid, re, im);
+}
+
+// The same for two polarisations where every cell of the chunk is stored and off the diagonal: no checks, and the
+// eight a-stations' cells at simple steps (b grows by sa + 1 from station to station).
+template <bool ADD>
+__device__ __forceinline__ void add_chunk_full(const int (&re)[8], const int (&im)[8], bool im_lane, int c, int a_base,
+                                               long long* __restrict__ cross_f) {
+  const unsigned sa = (unsigned)a_base >> 1;
+  longlong2* p = reinterpret_cast<longlong2*>(cross_f) + 4 * (long long)(sa * (sa + 1) / 2 + ((unsigned)c >> 1)) + (c & 1) +
+                 (im_lane ? 2 : 0);
+  longlong2* cell[8];
+#pragma unroll
+  for (int k = 0; k < 8; ++k) cell[k] = p + 4 * (k * sa + (unsigned)(k * (k + 1) / 2));
+  add_cells<ADD>(cell, 0xFFu, re, im);
 }
 
 // Stage k of an item's blocks: block k / n_kb, sample 128 (k % n_kb).

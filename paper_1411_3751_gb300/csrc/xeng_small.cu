@@ -321,7 +321,9 @@ __global__ void __launch_bounds__(S_THREADS, 1) xeng_small_kernel(const __grid_c
             uint32_t v[32];
             ptx::tmem_ld_32x32b_x32(tbase + 256 * acc + 128 * h + ((uint32_t)(32 * q) << 16) + 32 * cc, v);
             ptx::tmem_ld_wait();
-            xd::add_chunk<4, ADD, 8>(v, im_lane, live ? c : -1, 16 * cc - ch * args.ld, args.N, lp, cross_f, autos_f);
+            int re[8], im[8];
+            xd::combine_chunk<4>(v, im_lane, re, im);
+            xd::add_chunk<ADD>(re, im, im_lane, live ? c : -1, 16 * cc - ch * args.ld, args.N, lp, cross_f, autos_f);
           }
         }
         ptx::tc_fence_before();
