@@ -461,12 +461,12 @@ int direct_splits(long long items, int slots, int n_k, int overhead) {
   return best;
 }
 
-cudaError_t direct_args(const DirectJob& j, int box_bytes, bool swizzle, xd::Args* a) {
+cudaError_t direct_args(const DirectJob& j, int box_bytes, xd::Args* a) {
   std::memset(a, 0, sizeof(*a));
   if (j.n > xd::MAX_BLOCKS) return cudaErrorInvalidValue;
   for (int b = 0; b < j.n; ++b) {
     std::string err;
-    if (encode_raw_tensor_map(&a->map[b], j.blocks[b], (long long)j.s.C * j.ld, j.T_blk, box_bytes, swizzle, &err) != 0) {
+    if (encode_raw_tensor_map(&a->map[b], j.blocks[b], (long long)j.s.C * j.ld, j.T_blk, box_bytes, &err) != 0) {
       set_last_error(err);
       return cudaErrorInvalidValue;
     }
@@ -493,7 +493,7 @@ cudaError_t launch_xeng_direct(const DirectJob& j, int num_sms, cudaStream_t st)
   cudaError_t e = set_smem_limit(reinterpret_cast<const void*>(xeng_direct_kernel<false>), D_SMEM);
   if (e == cudaSuccess) e = set_smem_limit(reinterpret_cast<const void*>(xeng_direct_kernel<true>), D_SMEM);
   xd::Args a;
-  if (e == cudaSuccess) e = direct_args(j, 64, true, &a);
+  if (e == cudaSuccess) e = direct_args(j, 64, &a);
   if (e != cudaSuccess) return e;
   int pairs = std::max(1, num_sms / 2);
   const int fit = direct_max_pairs();

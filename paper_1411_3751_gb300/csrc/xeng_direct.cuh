@@ -28,16 +28,17 @@ struct Args {
   int* err;
 };
 
-// One 32-column chunk of an accumulator (16 a-inputs: column 8 (k / 4) + k % 4 = Re a_k, + 4 = Im a_k) as complex
-// products: the lanes holding Re c and Im c of one c-input are XOR apart, exchange half of their columns and own
+// One 32-column chunk of an accumulator (16 a-inputs: column 8 (k / 4) + k % 4 = Re a_k, + 4 = Im a_k; with HALVES
+// columns k and 16 + k) as complex products: the lanes holding Re c and Im c of one c-input are XOR apart, exchange half of their columns and own
 // 8 a-inputs each, the Re lane the even, the Im lane the odd ones. (With two polarisations a warp's access then
 // covers whole station pairs, 512 neighbouring bytes.) Combining all of an accumulator first halves the words a
 // thread holds, and leaves registers for eight cells in flight.
-template <int XOR>
+template <int XOR, bool HALVES = false>
 __device__ __forceinline__ void combine_chunk(const uint32_t (&v)[32], bool im_lane, int (&re)[8], int (&im)[8]) {
 #pragma unroll
   for (int k = 0; k < 8; ++k) {
-    const int jr = 8 * (k >> 1) + 2 * (k & 1), ji = jr + 4;  // columns of the even input; the odd one's follow
+    // columns of the even input; the odd one's follow
+    const int jr = HALVES ? 2 * k : 8 * (k >> 1) + 2 * (k & 1), ji = jr + (HALVES ? 16 : 4);
     const int own_r = f8::to_int(__uint_as_float(im_lane ? v[jr + 1] : v[jr]));
     const int own_i = f8::to_int(__uint_as_float(im_lane ? v[ji + 1] : v[ji]));
     const int recv_r = f8::to_int(__shfl_xor_sync(0xffffffffu, __uint_as_float(im_lane ? v[jr] : v[jr + 1]), XOR));
@@ -146,7 +147,7 @@ struct DirectJob {
 // Items' stages are divided by direct_splits() where whole items leave SMs idle: the division of n_k stages that
 // minimises waves x (stages + overhead), `slots` items running at once.
 int direct_splits(long long items, int slots, int n_k, int overhead);
-// The kernels' common arguments; boxes of box_bytes x 128 samples.
-cudaError_t direct_args(const DirectJob& j, int box_bytes, bool swizzle, xd::Args* a);
+// The kernels' common arguments; boxes of box_bytes (64 or 128, swizzled as wide) x 128 samples.
+cudaError_t direct_args(const DirectJob& j, int box_bytes, xd::Args* a);
 
 }  // namespace corr

@@ -9,9 +9,20 @@
 // used either. An item is two neighbouring units, so that TMA boxes are 128 bytes x 128 samples, and a
 // range of stages of 128 samples.
 //
-// Roles (one CTA per SM): warp 0 TMA producer; warp 1 TMEM allocation and MMA issuer (each unit has two of
-// the four 128-column accumulators); warps 2-9 converters: 16 bytes of one time -> 32 operand bytes of the
-// MN-major, 128-byte swizzled tile, and the inputs' offset sums; warps 10-17 epilogue, four a unit.
+// A and B of a unit's MMA are the same rows. With both read from one shared-memory tile a stage moved 128 KB
+// through shared memory (MMA reads 64, conversion 48, TMA 16) and took 660 ns, 1.3 times what HBM needs; so A
+// comes from TMEM: ldmatrix.trans.b8 brings the samples into registers transposed (four samples of an input a
+// word), a shift and logic operations make the operand words, and these go both to TMEM (A, tcgen05.st) and to
+// the K-major, 128-byte swizzled tile (B): 96 KB a stage.
+//
+// Roles (one CTA per SM): warp 0 TMA producer; warp 1 TMEM allocation and MMA issuer; warps 4-19 converters, two
+// sets that take the stages in turn, a warp for a TMEM lane quarter (16 inputs) of one unit, that also form the
+// inputs' offset sums; warps 20-27 epilogue, likewise. The accumulators (256 columns) and the A ring (192) fill
+// TMEM, so there is one accumulator a unit: the epilogue takes it into registers before it adds to the int64
+// sums. The registers are split by setmaxnreg: 128 x 32 + 512 x 56 + 256 x 120 of the 896 x 72 of the launch.
+// 32 inputs x 2400 channels x 4 x 8192 samples: 677 us with both operands in shared memory and one converter set,
+// 705 with A in TMEM, 622 with a second set as well, 598 with the units' MMAs in turn (370 at the measured copy
+// bandwidth). With a quarter of the MMAs it takes 530, without the B stores 25 us less.
 // Every wait is bounded (f8::WAIT_NS).
 #include <algorithm>
 #include <cstring>
@@ -24,7 +35,9 @@ namespace {
 
 using namespace f8;
 
-constexpr int S_THREADS = 576;
+constexpr int S_SETS = 2;                 // sets of eight converter warps that take the stages in turn
+constexpr int S_THREADS = 128 + 256 * S_SETS + 256;
+constexpr int S_EPI_WARP = 4 + 8 * S_SETS;
 constexpr int S_RAW = 6, S_OP = 3;        // ring stages: raw samples, operand tiles
 constexpr int S_RAW_BYTES = 128 * KT;     // two units
 constexpr int S_TILE = 128 * KT;          // one unit's operand
@@ -32,7 +45,9 @@ constexpr int S_OP_BYTES = 2 * S_TILE;
 constexpr int S_OP_OFF = S_RAW * S_RAW_BYTES;
 constexpr int S_BAR_OFF = S_OP_OFF + S_OP * S_OP_BYTES;
 constexpr int S_SMEM = S_BAR_OFF + 512 + 1024;
-constexpr int S_CONV_WARPS = 8;
+constexpr int S_CONV_WARPS = 8;           // of a set
+constexpr int S_A_COL = 256;               // first TMEM column of the A ring, 32 columns a unit and stage
+static_assert(S_A_COL + 64 * S_OP <= 512, "TMEM columns");
 static_assert(S_SMEM <= 227 * 1024, "shared memory");
 
 struct SmallItem {
@@ -54,9 +69,9 @@ __global__ void __launch_bounds__(S_THREADS, 1) xeng_small_kernel(const __grid_c
   uint64_t* raw_empty = raw_full + S_RAW;
   uint64_t* op_full = raw_empty + S_RAW;
   uint64_t* op_empty = op_full + S_OP;
-  uint64_t* tfull = op_empty + S_OP;  // [2]
-  uint64_t* tempty = tfull + 2;       // [2]
-  uint64_t* drain = tempty + 2;
+  uint64_t* tfull = op_empty + S_OP;
+  uint64_t* tempty = tfull + 1;
+  uint64_t* drain = tempty + 1;
   uint32_t* tslot = reinterpret_cast<uint32_t*>(drain + 1);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tslot + 1);
 
@@ -74,10 +89,8 @@ __global__ void __launch_bounds__(S_THREADS, 1) xeng_small_kernel(const __grid_c
       ptx::mbar_init(&op_full[s], S_CONV_WARPS);
       ptx::mbar_init(&op_empty[s], 1);
     }
-    for (int a = 0; a < 2; ++a) {
-      ptx::mbar_init(&tfull[a], 1);
-      ptx::mbar_init(&tempty[a], 8);
-    }
+    ptx::mbar_init(tfull, 1);
+    ptx::mbar_init(tempty, 8);
     ptx::mbar_init(drain, 1);
     *abort_flag = 0;
     ptx::fence_mbar_init();
@@ -91,8 +104,9 @@ __global__ void __launch_bounds__(S_THREADS, 1) xeng_small_kernel(const __grid_c
   ptx::tc_fence_after();
   const uint32_t tbase = *tslot;
 
-  if (warp == 0) {
-    if (lane == 0) {
+  if (warp < 4) {
+    ptx::setmaxnreg_dec<32>();
+    if (warp == 0 && lane == 0) {
       // ---------------- TMA producer ----------------
       int slot = 0;
       uint32_t phase = 0, n_issued = 0;
@@ -119,27 +133,25 @@ __global__ void __launch_bounds__(S_THREADS, 1) xeng_small_kernel(const __grid_c
         const uint32_t uses = n_issued / S_RAW + ((uint32_t)s < n_issued % S_RAW ? 1u : 0u);
         if (uses > 0) ptx::mbar_wait(&raw_full[s], (uses - 1) & 1, WAIT_NS);
       }
-    }
-  } else if (warp == 1) {
-    if (lane == 0) {
+    } else if (warp == 1 && lane == 0) {
       // ---------------- MMA issuer ----------------
-      const uint32_t idesc = ptx::idesc_f8_e4m3(128, 128, 1, 1);
+      const uint32_t idesc = ptx::idesc_f8_e4m3(128, 128, 0, 0);
+      // K-major, 128-byte swizzle: 8 rows x 128 samples per 1024 bytes (SBO); 32 samples on = 32 bytes
       const uint64_t desc0 = ptx::smem_desc(ptx::smem_u32(smem + S_OP_OFF), 16, 1024, 2);
-      int slot = 0, acc = 0;
-      uint32_t phase = 0, use[2] = {0u, 0u};
+      int slot = 0;
+      uint32_t phase = 0, use = 0;
       bool ok = true;
       for (long long w = blockIdx.x; w < total && ok && !*abort_flag; w += gridDim.x) {
         const SmallItem it(args, w, n_pairs);
         const bool two = 2 * it.p + 1 < args.n_units;
         for (int k0 = it.k0; k0 < it.k1 && ok; k0 += chunk_k) {
           const int k1 = min(k0 + chunk_k, it.k1);
-          if (!ptx::mbar_wait(&tempty[acc], (use[acc] & 1) ^ 1, WAIT_NS)) {
+          if (!ptx::mbar_wait(tempty, (use & 1) ^ 1, WAIT_NS)) {
             record_error(err, abort_flag, 2);
             ok = false;
             break;
           }
           ptx::tc_fence_after();
-          const uint32_t d = tbase + 256 * acc;
           for (int k = k0; k < k1; ++k) {
             if (!ptx::mbar_wait(&op_full[slot], phase, WAIT_NS)) {
               record_error(err, abort_flag, 3);
@@ -147,14 +159,15 @@ __global__ void __launch_bounds__(S_THREADS, 1) xeng_small_kernel(const __grid_c
               break;
             }
             ptx::tc_fence_after();
-            const uint64_t dd = desc0 + (uint64_t)((slot * S_OP_BYTES) >> 4);
+            const uint64_t bd = desc0 + (uint64_t)((slot * S_OP_BYTES) >> 4);
+            const uint32_t at = tbase + S_A_COL + 64 * slot;
+            // the units in turn: two MMAs into one accumulator wait for each other
 #pragma unroll
-            for (int kk = 0; kk < KT / 32; ++kk) ptx::mma_f8f6f4(d, dd + kk * 256, dd + kk * 256, idesc, (k > k0 || kk > 0) ? 1u : 0u);
-            if (two) {
-              const uint64_t d2 = dd + (S_TILE >> 4);
-#pragma unroll
-              for (int kk = 0; kk < KT / 32; ++kk)
-                ptx::mma_f8f6f4(d + 128, d2 + kk * 256, d2 + kk * 256, idesc, (k > k0 || kk > 0) ? 1u : 0u);
+            for (int kk = 0; kk < KT / 32; ++kk) {
+              ptx::mma_f8f6f4_ts(tbase, at + 8 * kk, bd + 2 * kk, idesc, (k > k0 || kk > 0) ? 1u : 0u);
+              if (two)
+                ptx::mma_f8f6f4_ts(tbase + 128, at + 32 + 8 * kk, bd + (S_TILE >> 4) + 2 * kk, idesc,
+                                   (k > k0 || kk > 0) ? 1u : 0u);
             }
             ptx::mma_commit(&op_empty[slot]);
             if (++slot == S_OP) {
@@ -163,140 +176,126 @@ __global__ void __launch_bounds__(S_THREADS, 1) xeng_small_kernel(const __grid_c
             }
           }
           if (!ok) break;
-          ptx::mma_commit(&tfull[acc]);
-          ++use[acc];
-          acc ^= 1;
+          ptx::mma_commit(tfull);
+          ++use;
         }
       }
       // all issued MMAs complete before TMEM is released
       ptx::mma_commit(drain);
       ptx::mbar_wait(drain, 0, WAIT_NS);
     }
-  } else if (warp < 2 + S_CONV_WARPS) {
-    // ---------------- converters ----------------
-    // Lane -> 16-byte column c of unit h, sample rows: eight neighbouring lanes read four columns of unit 0
-    // and, a row on, of unit 1, which touches every bank (as the swizzled stores do); in the second
-    // phase of a step the rows swap.
-    const int cw = warp - 2;
-    const int c = lane & 3, h = (lane >> 2) & 1, pr = lane >> 3;  // row pairs 8 i + pr ... of the warp's 16 rows
-    const uint32_t r_col = (uint32_t)(16 * c + h * args.ub);
-    int rs = 0, os = 0;
+  } else if (warp < S_EPI_WARP) {
+    // ---------------- converters: lane quarter q of unit h, every S_SETS-th stage ----------------
+    ptx::setmaxnreg_dec<56>();
+    const int q = warp & 3, h = ((warp - 4) >> 2) & 1, set = (warp - 4) >> 3;
+    // lane l addresses sample row l (+ 32 kk) of the 16-byte column of the quarter's inputs (128-byte swizzle)
+    const uint32_t a_off = ptx::smem_u32(smem) + (uint32_t)lane * 128 + (uint32_t)(((h * args.ub / 16 + q) ^ (lane & 7)) << 4);
+    const uint32_t a_tmem = tbase + S_A_COL + 32 * h + ((uint32_t)(32 * q) << 16);
+    // B row 32 q + lane / 4 (Re; + 8, and + 16 for Im), samples 16 j + 4 (lane % 4) ..: 16-byte chunk j of the row
+    const int br = lane >> 2;
+    uint8_t* b_dst = smem + S_OP_OFF + h * S_TILE + (32 * q + br) * 128 + 4 * (lane & 3);
+    int rs = set, os = set;
     uint32_t rph = 0, oph = 0;
+    int ahead = set;  // stages until the set's next one
     bool ok = true;
-    for (long long w = blockIdx.x; w < total && ok; w += gridDim.x) {
+    for (long long w = blockIdx.x; w < total && ok && !*abort_flag; w += gridDim.x) {
       const SmallItem it(args, w, n_pairs);
-      xd::StagePos p(it.k0, args.n_kb);
-      for (int k0 = it.k0; k0 < it.k1 && ok; k0 += chunk_k) {
-        const int k1 = min(k0 + chunk_k, it.k1);
-        // packed sums of the thread's 16 inputs: bytes over a stage's 4 samples, 16-bit lanes over the chunk
-        // (at most 15 x 4 x 512 stages)
-        uint32_t sre[4][2] = {{0u, 0u}, {0u, 0u}, {0u, 0u}, {0u, 0u}};
-        uint32_t sim[4][2] = {{0u, 0u}, {0u, 0u}, {0u, 0u}, {0u, 0u}};
-        for (int k = k0; k < k1; ++k, p.next(args.n_kb)) {
-          if (*abort_flag) {
-            ok = false;
-            break;
-          }
-          const int n_valid = min(KT, args.T - p.kb * KT);
-          if (!ptx::mbar_wait(&raw_full[rs], rph, WAIT_NS)) {
-            record_error(err, abort_flag, 5);
-            ok = false;
-            break;
-          }
-          const uint8_t* src = smem + rs * S_RAW_BYTES + r_col;
-          uint4 r[4];
-#pragma unroll
-          for (int i = 0; i < 4; ++i) {  // step i >> 1, phase i & 1
-            const int row = 16 * cw + 8 * (i >> 1) + 2 * pr + (h ^ (i & 1));
-            r[i] = *reinterpret_cast<const uint4*>(src + row * 128);
-          }
-          if (!ptx::mbar_wait(&op_empty[os], oph ^ 1, WAIT_NS)) {
-            record_error(err, abort_flag, 6);
-            ok = false;
-            break;
-          }
-          uint8_t* dst = smem + S_OP_OFF + os * S_OP_BYTES + h * S_TILE;
-          uint32_t bre[4] = {0u, 0u, 0u, 0u}, bim[4] = {0u, 0u, 0u, 0u};
-#pragma unroll
-          for (int i = 0; i < 4; ++i) {
-            const int row = 16 * cw + 8 * (i >> 1) + 2 * pr + (h ^ (i & 1));
-            uint4 o0 = make_uint4(flip_hi(r[i].x), flip_lo(r[i].x), flip_hi(r[i].y), flip_lo(r[i].y));
-            uint4 o1 = make_uint4(flip_hi(r[i].z), flip_lo(r[i].z), flip_hi(r[i].w), flip_lo(r[i].w));
-            if (row >= n_valid) o0 = o1 = make_uint4(0u, 0u, 0u, 0u);
-            uint8_t* rowp = dst + (row >> 3) * 1024 + (row & 7) * 128;
-            *reinterpret_cast<uint4*>(rowp + (((2 * c) ^ (row & 7)) << 4)) = o0;
-            *reinterpret_cast<uint4*>(rowp + (((2 * c + 1) ^ (row & 7)) << 4)) = o1;
-            bre[0] += o0.x;
-            bim[0] += o0.y;
-            bre[1] += o0.z;
-            bim[1] += o0.w;
-            bre[2] += o1.x;
-            bim[2] += o1.y;
-            bre[3] += o1.z;
-            bim[3] += o1.w;
-          }
-          ptx::fence_proxy_async_smem();
-          __syncwarp();
-          if (lane == 0) {
-            ptx::mbar_arrive(&op_full[os]);
-            // the stores above needed the loaded samples, so the loads are done; an arrival right behind the
-            // loads overtook them, and the next box landed under them
-            ptx::mbar_arrive(&raw_empty[rs]);
-          }
-          if (++rs == S_RAW) {
-            rs = 0;
-            rph ^= 1;
-          }
-          if (++os == S_OP) {
-            os = 0;
-            oph ^= 1;
-          }
-#pragma unroll
-          for (int i = 0; i < 4; ++i) {
-            sre[i][0] += bre[i] & 0x00FF00FFu;
-            sre[i][1] += (bre[i] >> 8) & 0x00FF00FFu;
-            sim[i][0] += bim[i] & 0x00FF00FFu;
-            sim[i][1] += (bim[i] >> 8) & 0x00FF00FFu;
-          }
+      xd::StagePos p(it.k0 + ahead, args.n_kb);
+      uint32_t sum[4] = {0u, 0u, 0u, 0u};  // Re, Im of inputs lane / 4 and lane / 4 + 8 of the quarter's 16
+      for (int k = it.k0 + ahead; k < it.k1; k += S_SETS, p.next(args.n_kb, S_SETS)) {
+        const int n_valid = args.T - p.kb * KT;  // samples of this stage (at most 128)
+        if (!ptx::mbar_wait(&raw_full[rs], rph, WAIT_NS) || !ptx::mbar_wait(&op_empty[os], oph ^ 1, WAIT_NS)) {
+          record_error(err, abort_flag, 5);
+          ok = false;
+          break;
         }
-        if (!ok) break;
-        // the sums of this chunk over the four lanes of a column; each of them adds 4 of its 16 inputs
-        const long long u = 2 * it.p + h;
+        ptx::tc_fence_after();  // the MMAs that read this A slot have completed
+        const uint32_t raw = a_off + (uint32_t)(rs * S_RAW_BYTES);
+        uint8_t* dst = b_dst + os * S_OP_BYTES;
+        uint32_t x[16];
 #pragma unroll
-        for (int i = 0; i < 4; ++i)
+        for (int kk = 0; kk < 4; ++kk)
+          ptx::ldmatrix_b8_x2_trans(raw + kk * 4096, x[4 * kk], x[4 * kk + 1], x[4 * kk + 2], x[4 * kk + 3]);
 #pragma unroll
-          for (int b = 0; b < 4; ++b) {
-            int re = (int)((sre[i][b & 1] >> (16 * (b >> 1))) & 0xFFFF), im = (int)((sim[i][b & 1] >> (16 * (b >> 1))) & 0xFFFF);
-            re += __shfl_xor_sync(0xffffffffu, re, 8);
-            im += __shfl_xor_sync(0xffffffffu, im, 8);
-            re += __shfl_xor_sync(0xffffffffu, re, 16);
-            im += __shfl_xor_sync(0xffffffffu, im, 16);
-            const int in = 16 * c + 4 * i + b;  // input row of the unit
-            const int ch = in / args.ld, n = in - ch * args.ld;
-            const long long f = u * args.g + ch;
-            if (pr == i && ch < args.g && n < args.N && u < args.n_units && f < args.C) {
-              const long long idx = (f * args.N + n) * 2;
-              atomicAdd(reinterpret_cast<unsigned long long*>(args.s1 + idx), (unsigned long long)re);
-              atomicAdd(reinterpret_cast<unsigned long long*>(args.s1 + idx + 1), (unsigned long long)im);
-              atomicAdd(reinterpret_cast<unsigned long long*>(args.s2 + idx), (unsigned long long)re);
-              atomicAdd(reinterpret_cast<unsigned long long*>(args.s2 + idx + 1), (unsigned long long)im);
+        for (int half = 0; half < 2; ++half) {  // 64 samples at a time
+          uint32_t y[8], z[8];
+#pragma unroll
+          for (int i = 0; i < 8; ++i) {
+            y[i] = flip_hi(x[8 * half + i]);
+            z[i] = flip_lo(x[8 * half + i]);
+          }
+          if (n_valid < KT) {  // samples past the block: zeros
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+              const uint32_t m = byte_mask(n_valid - (64 * half + 16 * (i >> 1) + 4 * (lane & 3)));
+              y[i] &= m;
+              z[i] &= m;
             }
           }
+          ptx::tmem_st_16x128b_x4(a_tmem + 64 * os + 16 * half, y);
+          ptx::tmem_st_16x128b_x4(a_tmem + (16u << 16) + 64 * os + 16 * half, z);
+#pragma unroll
+          for (int i = 0; i < 8; ++i) {  // word 2 j + r: chunk 4 half + j, row + 8 r
+            uint8_t* o = dst + (i & 1) * 1024 + (((4 * half + (i >> 1)) ^ br) << 4);
+            *reinterpret_cast<uint32_t*>(o) = y[i];
+            *reinterpret_cast<uint32_t*>(o + 2048) = z[i];
+            sum[2 * (i & 1)] = __dp4a(y[i], 0x01010101u, sum[2 * (i & 1)]);
+            sum[2 * (i & 1) + 1] = __dp4a(z[i], 0x01010101u, sum[2 * (i & 1) + 1]);
+          }
+        }
+        ptx::tmem_st_wait();
+        ptx::fence_proxy_async_smem();
+        ptx::tc_fence_before();
+        __syncwarp();
+        if (lane == 0) {
+          ptx::mbar_arrive(&op_full[os]);
+          // the stores above needed the loaded samples, so the loads are done (an arrival right behind them
+          // may overtake them, and the next box would land under them)
+          ptx::mbar_arrive(&raw_empty[rs]);
+        }
+        rs += S_SETS;
+        if (rs >= S_RAW) {
+          rs -= S_RAW;
+          rph ^= 1;
+        }
+        os += S_SETS;
+        if (os >= S_OP) {
+          os -= S_OP;
+          oph ^= 1;
+        }
+      }
+      if (!ok) break;
+      ahead = (ahead - (it.k1 - it.k0)) % S_SETS;
+      if (ahead < 0) ahead += S_SETS;
+      const long long u = 2 * it.p + h;
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        // a thread saw a quarter of at most 2^28 samples (direct_max_blocks) of at most 15
+        unsigned long long s = sum[i];
+        s += __shfl_xor_sync(0xffffffffu, s, 1);
+        s += __shfl_xor_sync(0xffffffffu, s, 2);
+        const int in = 16 * q + br + 8 * (i >> 1);  // input row of the unit
+        const int ch = in / args.ld, n = in - ch * args.ld;
+        const long long f = u * args.g + ch;
+        if ((lane & 3) == 0 && ch < args.g && n < args.N && u < args.n_units && f < args.C) {
+          const long long idx = (f * args.N + n) * 2 + (i & 1);
+          atomicAdd(reinterpret_cast<unsigned long long*>(args.s1 + idx), s);
+          atomicAdd(reinterpret_cast<unsigned long long*>(args.s2 + idx), s);
+        }
       }
     }
   } else {
-    // ---------------- epilogue (warps 10..17): four warps, one TMEM lane quarter each, a unit ----------------
-    const int q = warp & 3, h = (warp - 10) >> 2;
-    const bool im_lane = (lane & 4) != 0;
+    // ---------------- epilogue: lane quarter q of unit h ----------------
+    ptx::setmaxnreg_inc<120>();
+    const int q = warp & 3, h = (warp - S_EPI_WARP) >> 2;
+    const bool im_lane = (lane & 16) != 0;
     const int lp = args.npol >> 1;
-    const int row = 32 * q + lane;
-    const int ic = 4 * (row >> 3) + (row & 3);  // c-input of the unit
+    const int ic = 16 * q + (lane & 15);  // c-input of the unit
     const int ch = ic / args.ld, c = ic - ch * args.ld;
     // the chunks (16 a-inputs) that hold this warp's channels, from the diagonal on
     const int last = min(64, ((16 * q + 15) / args.ld + 1) * args.ld);
     const int cc_end = (last + 15) / 16;
-    uint32_t use[2] = {0u, 0u};
-    int acc = 0;
+    uint32_t use = 0;
     bool ok = true;
     for (long long w = blockIdx.x; w < total && ok; w += gridDim.x) {
       const SmallItem it(args, w, n_pairs);
@@ -309,28 +308,32 @@ __global__ void __launch_bounds__(S_THREADS, 1) xeng_small_kernel(const __grid_c
           ok = false;
           break;
         }
-        const bool got = ptx::mbar_wait(&tfull[acc], use[acc] & 1, WAIT_NS);
+        const bool got = ptx::mbar_wait(tfull, use & 1, WAIT_NS);
         if (!__all_sync(0xffffffffu, got)) {
           if (lane == 0) record_error(err, abort_flag, 4);
           ok = false;
           break;
         }
         ptx::tc_fence_after();
-        if (u < args.n_units) {
-          for (int cc = q; cc < cc_end; ++cc) {
-            uint32_t v[32];
-            ptx::tmem_ld_32x32b_x32(tbase + 256 * acc + 128 * h + ((uint32_t)(32 * q) << 16) + 32 * cc, v);
-            ptx::tmem_ld_wait();
-            int re[8], im[8];
-            xd::combine_chunk<4>(v, im_lane, re, im);
-            xd::add_chunk<ADD>(re, im, im_lane, live ? c : -1, 16 * cc - ch * args.ld, args.N, lp, cross_f, autos_f);
-          }
+        const uint32_t t = tbase + 128 * h + ((uint32_t)(32 * q) << 16);
+        int re[4][8], im[4][8];
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {  // two chunks at a time
+          uint32_t v[2][32];
+          ptx::tmem_ld_32x32b_x32(t + 64 * j, v[0]);
+          ptx::tmem_ld_32x32b_x32(t + 64 * j + 32, v[1]);
+          ptx::tmem_ld_wait();
+          xd::combine_chunk<16, true>(v[0], im_lane, re[2 * j], im[2 * j]);
+          xd::combine_chunk<16, true>(v[1], im_lane, re[2 * j + 1], im[2 * j + 1]);
         }
         ptx::tc_fence_before();
         __syncwarp();
-        if (lane == 0) ptx::mbar_arrive(&tempty[acc]);
-        ++use[acc];
-        acc ^= 1;
+        if (lane == 0) ptx::mbar_arrive(tempty);
+        ++use;
+#pragma unroll
+        for (int cc = 0; cc < 4; ++cc)
+          if (u < args.n_units && cc >= q && cc < cc_end)
+            xd::add_chunk<ADD>(re[cc], im[cc], im_lane, live ? c : -1, 16 * cc - ch * args.ld, args.N, lp, cross_f, autos_f);
       }
     }
   }
@@ -360,7 +363,7 @@ cudaError_t launch_xeng_small(const DirectJob& j, int num_sms, cudaStream_t st) 
   cudaError_t e = set_smem_limit(reinterpret_cast<const void*>(xeng_small_kernel<false>), S_SMEM);
   if (e == cudaSuccess) e = set_smem_limit(reinterpret_cast<const void*>(xeng_small_kernel<true>), S_SMEM);
   xd::Args a;
-  if (e == cudaSuccess) e = direct_args(j, 128, false, &a);
+  if (e == cudaSuccess) e = direct_args(j, 128, &a);
   if (e != cudaSuccess) return e;
   a.g = small_group(j.ld);
   a.ub = a.g * j.ld;
