@@ -490,10 +490,9 @@ cudaError_t direct_args(const DirectJob& j, int box_bytes, xd::Args* a) {
 
 cudaError_t launch_xeng_direct(const DirectJob& j, int num_sms, cudaStream_t st) {
   if (j.n == 0 || j.T_blk == 0) return cudaSuccess;
-  cudaError_t e = set_smem_limit(reinterpret_cast<const void*>(xeng_direct_kernel<false>), D_SMEM);
-  if (e == cudaSuccess) e = set_smem_limit(reinterpret_cast<const void*>(xeng_direct_kernel<true>), D_SMEM);
   xd::Args a;
-  if (e == cudaSuccess) e = direct_args(j, 64, &a);
+  cudaError_t e = direct_args(j, 64, &a);
+  if (e == cudaSuccess) e = set_smem_limit(reinterpret_cast<const void*>(xeng_direct_kernel<false>), D_SMEM);
   if (e != cudaSuccess) return e;
   int pairs = std::max(1, num_sms / 2);
   const int fit = direct_max_pairs();
@@ -506,10 +505,13 @@ cudaError_t launch_xeng_direct(const DirectJob& j, int num_sms, cudaStream_t st)
   a.kps = (a.n_k + a.splits - 1) / a.splits;
   a.n_items = items * a.splits;
   const unsigned grid = 2u * (unsigned)std::min<long long>(pairs, a.n_items);
-  if (a.splits > 1)
+  if (a.splits > 1) {
+    e = set_smem_limit(reinterpret_cast<const void*>(xeng_direct_kernel<true>), D_SMEM);
+    if (e != cudaSuccess) return e;
     xeng_direct_kernel<true><<<grid, D_THREADS, D_SMEM, st>>>(a);
-  else
+  } else {
     xeng_direct_kernel<false><<<grid, D_THREADS, D_SMEM, st>>>(a);
+  }
   return cudaGetLastError();
 }
 

@@ -360,10 +360,8 @@ bool xeng_small_supported(const Shape& s, int ld, const void* d_in) {
 
 cudaError_t launch_xeng_small(const DirectJob& j, int num_sms, cudaStream_t st) {
   if (j.n == 0 || j.T_blk == 0) return cudaSuccess;
-  cudaError_t e = set_smem_limit(reinterpret_cast<const void*>(xeng_small_kernel<false>), S_SMEM);
-  if (e == cudaSuccess) e = set_smem_limit(reinterpret_cast<const void*>(xeng_small_kernel<true>), S_SMEM);
   xd::Args a;
-  if (e == cudaSuccess) e = direct_args(j, 128, &a);
+  cudaError_t e = direct_args(j, 128, &a);
   if (e != cudaSuccess) return e;
   a.g = small_group(j.ld);
   a.ub = a.g * j.ld;
@@ -373,6 +371,9 @@ cudaError_t launch_xeng_small(const DirectJob& j, int num_sms, cudaStream_t st) 
   a.kps = (a.n_k + a.splits - 1) / a.splits;
   a.n_items = pairs * a.splits;
   const unsigned grid = (unsigned)std::min<long long>(num_sms, a.n_items);
+  e = set_smem_limit(a.splits > 1 ? reinterpret_cast<const void*>(xeng_small_kernel<true>)
+                                  : reinterpret_cast<const void*>(xeng_small_kernel<false>), S_SMEM);
+  if (e != cudaSuccess) return e;
   if (a.splits > 1)
     xeng_small_kernel<true><<<grid, S_THREADS, S_SMEM, st>>>(a);
   else
