@@ -122,13 +122,24 @@ __device__ __forceinline__ float norm_exact(long long v, long long n) {
 // not change the rounded float, that float is the rounded exact quotient (and so the one the double
 // division rounds to, whose error is 2^-53); else, about one value in 2^18, divide as defined.
 __device__ __forceinline__ float norm_fast(long long v, long long n, float rh, float rl) {
-  const float hi = __ll2float_rn(v);
-  const float lo = __ll2float_rn(v - __float2ll_rn(hi));
+  float hi, lo;
+  if (v >= -(1LL << 30) && v < (1LL << 30)) {  // the usual sums: 32-bit conversions
+    hi = __int2float_rn((int)v);
+    lo = __int2float_rn((int)v - __float2int_rz(hi));
+  } else {
+    hi = __ll2float_rn(v);
+    lo = __ll2float_rn(v - __float2ll_rn(hi));
+  }
   const float p = __fmul_rn(hi, rh);
   const float e = __fmaf_rn(lo, rh, __fmaf_rn(hi, rl, __fmaf_rn(hi, rh, -p)));
   const float d = __fmul_rn(fabsf(p), 5.6843418860808015e-14f);  // 2^-44
   const float q1 = __fadd_rn(p, __fadd_rn(e, d)), q2 = __fadd_rn(p, __fsub_rn(e, d));
   return q1 == q2 ? q1 : norm_exact(v, n);
+}
+
+// float(v)
+__device__ __forceinline__ float nearest(long long v) {
+  return v == (long long)(int)v ? __int2float_rn((int)v) : __ll2float_rn(v);
 }
 
 // Sample count of a normalised dump: n for every cell with rh + rl = 1 / n, or (cells reset
@@ -150,7 +161,7 @@ DumpNorm dump_norm(long long n) {
 // One value in format FMT (CI64: long long, else float); ns = the cell's own count if HAS_BASE.
 template <bool HAS_BASE>
 __device__ __forceinline__ float as_float(long long v, int fmt, const DumpNorm& dn, long long ns) {
-  if (fmt == CORR_FMT_CF32) return __ll2float_rn(v);
+  if (fmt == CORR_FMT_CF32) return nearest(v);
   if (HAS_BASE) return norm_exact(v, ns);
   return dn.n > 0 ? norm_fast(v, dn.n, dn.rh, dn.rl) : 0.f;
 }
