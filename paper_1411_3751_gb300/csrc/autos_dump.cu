@@ -5,17 +5,20 @@ namespace corr {
 namespace {
 
 // Autocorrelations A[f][n] += sum_t |x_{f,n}(t)|^2 (Sec. 2.6: total power of selected inputs at a high
-// cadence). HBM-bound: the samples are read once. A row t is M = C N neighbouring bytes; a thread keeps
-// 16 of them (16 cells) and walks down t with eight 16-byte loads in flight, the 8 warps of a block
-// taking every eighth row of the same 512 bytes; the warps' int32 sums meet in shared memory and are
-// added to the int64 sums by one thread a cell. gridDim.y splits t where the columns alone leave SMs
-// idle (the sums then meet in 64-bit atomics, exact in any order).
-// 512 inputs x 2400 channels x 240 samples: 358 us with one byte a load, 62 us so.
+// cadence) of blocks whose rows TMA does not take (the others: autos_tma.cu). A row t is M = C N neighbouring
+// bytes; a thread keeps 16 of them (16 cells) and walks down t, four rows' loads in flight while four are added
+// up, the 8 warps of a block taking every eighth row of the same 512 bytes; the warps' sums meet in shared memory and
+// are added to the int64 sums by one thread a cell. Block b takes columns b % gx and run b / gx of the rows: t is
+// split where the columns alone leave SMs idle and into runs whose 16-bit sums hold (the sums then meet in
+// 64-bit atomics, exact in any order).
 //
 // A square of a 4-bit component x = m - 8 s (s the sign bit, m the low three) is m^2 or (8 - m)^2: a byte
 // permute with the nibbles as selectors looks four of them up at once, the selectors' top bit making
-// the other sign's entries zero (the permute then repeats the entry's top bit, clear in every entry).
-constexpr int AU_NT = 256, AU_W = AU_NT / 32, AU_U = 8;
+// the other sign's entries zero (the permute then repeats the entry's top bit, clear in every entry). Three
+// rows' squares (at most 64) fit a byte lane; then the halves of a sample are added into 16-bit lanes.
+// (A dp4a a sample for the sums runs at a quarter of the other instructions' rate: 85 us at 512 inputs x 2400
+// channels x 240 aligned samples, 77 so, 358 with one byte a load.)
+constexpr int AU_NT = 256, AU_W = AU_NT / 32, AU_U = 4;
 
 // squares of the four components in the low 16 bits of w (wx = w ^ 0x88888888), one byte each
 __device__ __forceinline__ uint32_t squares4(uint32_t w, uint32_t wx) {
@@ -25,22 +28,24 @@ __device__ __forceinline__ uint32_t squares4(uint32_t w, uint32_t wx) {
   return p | q;
 }
 
-// acc[0..3] += |x|^2 of the four samples of w
-__device__ __forceinline__ void add_power4(int (&acc)[16], int k, uint32_t w) {
-  const uint32_t wx = w ^ 0x88888888u;
-  const uint32_t lo = squares4(w, wx), hi = squares4(w >> 16, wx >> 16);
-  acc[4 * k + 0] = (int)__dp4a(lo, 0x00000101u, (unsigned)acc[4 * k + 0]);
-  acc[4 * k + 1] = (int)__dp4a(lo, 0x01010000u, (unsigned)acc[4 * k + 1]);
-  acc[4 * k + 2] = (int)__dp4a(hi, 0x00000101u, (unsigned)acc[4 * k + 2]);
-  acc[4 * k + 3] = (int)__dp4a(hi, 0x01010000u, (unsigned)acc[4 * k + 3]);
+// acc[0], acc[1] (16-bit lanes, samples 0, 1 and 2, 3 of the words) += |x|^2 over the same word of R <= 3 rows.
+template <int R>
+__device__ __forceinline__ void add_power4(uint32_t (&acc)[2], const uint32_t (&w)[R]) {
+  uint32_t lo = 0u, hi = 0u;
+#pragma unroll
+  for (int r = 0; r < R; ++r) {
+    const uint32_t wx = w[r] ^ 0x88888888u;
+    lo += squares4(w[r], wx);
+    hi += squares4(w[r] >> 16, wx >> 16);
+  }
+  acc[0] += (lo & 0x00FF00FFu) + ((lo >> 8) & 0x00FF00FFu);
+  acc[1] += (hi & 0x00FF00FFu) + ((hi >> 8) & 0x00FF00FFu);
 }
+constexpr int AU_ROWS = AU_W * 504;  // rows a block takes at most: 504 samples of at most 128 a 16-bit lane
 
-// VEC: 16-byte loads (rows and buffer multiples of 16 bytes); else 16 bytes at any address: the five
-// aligned words around them, shifted together, or byte by byte where those words would leave the
-// buffer [in, end).
-template <bool VEC>
+// The 16 bytes at any address p: the five aligned words around them, shifted together, or byte by byte where those
+// words would leave the buffer [in, end).
 __device__ __forceinline__ uint4 autos_load(const uint8_t* p, int nv, const uint8_t* in, const uint8_t* end) {
-  if (VEC) return __ldg(reinterpret_cast<const uint4*>(p));
   const uint32_t sh = (uint32_t)(reinterpret_cast<uintptr_t>(p) & 3);
   const uint8_t* q = p - sh;
   uint32_t x[5] = {0u, 0u, 0u, 0u, 0u};
@@ -55,50 +60,57 @@ __device__ __forceinline__ uint4 autos_load(const uint8_t* p, int nv, const uint
   return make_uint4(x[0], x[1], x[2], x[3]);
 }
 
-template <bool VEC>
 __global__ void __launch_bounds__(AU_NT) autos_kernel(const uint8_t* __restrict__ in, long long M, int T, int rows,
-                                                      long long* __restrict__ autos) {
+                                                      unsigned gx, bool split, long long* __restrict__ autos) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const long long col = blockIdx.x * 512LL + 16 * lane;
+  const unsigned run = blockIdx.x / gx, bx = blockIdx.x - run * gx;
+  const long long col = bx * 512LL + 16 * lane;
   const int nv = M - col >= 16 ? 16 : (M > col ? (int)(M - col) : 0);
-  const int t_end = (int)min((long long)T, (blockIdx.y + 1LL) * rows);
+  const int t_end = (int)min((long long)T, (run + 1LL) * rows);
   const uint8_t* end = in + (size_t)T * M;
-  int acc[16];
-#pragma unroll
-  for (int k = 0; k < 16; ++k) acc[k] = 0;
+  uint32_t acc[4][2] = {{0u, 0u}, {0u, 0u}, {0u, 0u}, {0u, 0u}};  // word k: its samples' sums in 16-bit lanes
   if (nv > 0) {
-    // long: the last steps of a row count near 2^31 would overflow an int
-    for (long long t0 = (long long)blockIdx.y * rows + warp; t0 < t_end; t0 += AU_W * AU_U) {
-      uint4 w[AU_U];
+    // the next four rows' loads are in flight while four are added up
+    // (long: the last steps of a row count near 2^31 would overflow an int)
+    auto load = [&](uint4 (&w)[AU_U], long long t0) {
 #pragma unroll
       for (int u = 0; u < AU_U; ++u) {
         const long long t = t0 + AU_W * u;
-        w[u] = t < t_end ? autos_load<VEC>(in + (size_t)t * M + col, nv, in, end) : make_uint4(0u, 0u, 0u, 0u);
+        w[u] = t < t_end ? autos_load(in + (size_t)t * M + col, nv, in, end) : make_uint4(0u, 0u, 0u, 0u);
+      }
+    };
+    long long t0 = (long long)run * rows + warp;
+    uint4 w[AU_U], nx[AU_U];
+    load(w, t0);
+    while (t0 < t_end) {
+      t0 += AU_W * AU_U;
+      load(nx, t0);
+#pragma unroll
+      for (int u = 0; u < AU_U; u += 2) {
+        add_power4<2>(acc[0], {w[u].x, w[u + 1].x});
+        add_power4<2>(acc[1], {w[u].y, w[u + 1].y});
+        add_power4<2>(acc[2], {w[u].z, w[u + 1].z});
+        add_power4<2>(acc[3], {w[u].w, w[u + 1].w});
       }
 #pragma unroll
-      for (int u = 0; u < AU_U; ++u) {
-        add_power4(acc, 0, w[u].x);
-        add_power4(acc, 1, w[u].y);
-        add_power4(acc, 2, w[u].z);
-        add_power4(acc, 3, w[u].w);
-      }
+      for (int u = 0; u < AU_U; ++u) w[u] = nx[u];
     }
   }
   __shared__ __align__(16) int part[AU_W][512];
 #pragma unroll
   for (int k = 0; k < 4; ++k)
     *reinterpret_cast<int4*>(&part[warp][16 * lane + 4 * k]) =
-        make_int4(acc[4 * k], acc[4 * k + 1], acc[4 * k + 2], acc[4 * k + 3]);
+        make_int4((int)(acc[k][0] & 0xFFFFu), (int)(acc[k][0] >> 16), (int)(acc[k][1] & 0xFFFFu), (int)(acc[k][1] >> 16));
   __syncthreads();
 #pragma unroll
   for (int h = 0; h < 2; ++h) {
     const int i = threadIdx.x + AU_NT * h;
-    const long long cell = blockIdx.x * 512LL + i;
+    const long long cell = bx * 512LL + i;
     if (cell >= M) break;
     long long sum = 0;
 #pragma unroll
     for (int v = 0; v < AU_W; ++v) sum += part[v][i];
-    if (gridDim.y == 1)
+    if (!split)
       autos[cell] += sum;
     else
       atomicAdd(reinterpret_cast<unsigned long long*>(autos + cell), (unsigned long long)sum);
@@ -407,17 +419,15 @@ cudaError_t launch_autos(const Shape& s, const uint8_t* d_in, int T_blk, long lo
   const long long M = (long long)s.C * s.N;
   const long long gx = (M + 511) / 512;
   // rows per block: all of them while the columns fill the GPU (four blocks an SM), else at least 64 (8 a
-  // warp, one step of loads); at most 2^20 (8 x 2^17 samples of at most 128 in an int32 sum)
+  // warp, one step of loads); at most AU_ROWS
   const long long want = (4LL * sm_count() + gx - 1) / gx;
   long long rows = ((long long)T_blk + want - 1) / want;
   if (rows < 64) rows = 64;
-  if (rows > (1 << 20)) rows = 1 << 20;
+  if (rows > AU_ROWS) rows = AU_ROWS;
   if (rows > T_blk) rows = T_blk;
-  const dim3 grid((unsigned)gx, (unsigned)((T_blk + rows - 1) / rows));
-  if (M % 16 == 0 && reinterpret_cast<uintptr_t>(d_in) % 16 == 0)
-    autos_kernel<true><<<grid, AU_NT, 0, st>>>(d_in, M, T_blk, (int)rows, d_autos);
-  else
-    autos_kernel<false><<<grid, AU_NT, 0, st>>>(d_in, M, T_blk, (int)rows, d_autos);
+  const long long runs = (T_blk + rows - 1) / rows;
+  const unsigned grid = (unsigned)(gx * runs);
+  autos_kernel<<<grid, AU_NT, 0, st>>>(d_in, M, T_blk, (int)rows, (unsigned)gx, runs > 1, d_autos);
   return cudaGetLastError();
 }
 

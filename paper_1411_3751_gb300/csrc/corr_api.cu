@@ -1138,8 +1138,10 @@ int corr_accumulate_autos(corr_ctx* c, const void* d_samples, void* stream) {
   if (!c) return fail(CORR_ERR_ARG, "corr_accumulate_autos: NULL context");
   if (!d_samples) return fail(CORR_ERR_ARG, "corr_accumulate_autos: NULL samples");
   const bool tb = timer_begin(c, CORR_KERNEL_AUTOS, (cudaStream_t)stream);
-  cudaError_t e = launch_autos(c->L.s, static_cast<const uint8_t*>(d_samples), c->L.s.T, c->d_autos,
-                               (cudaStream_t)stream);
+  const uint8_t* in = static_cast<const uint8_t*>(d_samples);
+  const cudaError_t e = autos_tma_supported(c->L.s, in)
+                            ? launch_autos_tma(c->L.s, in, c->L.s.T, c->d_autos, c->d_err, (cudaStream_t)stream)
+                            : launch_autos(c->L.s, in, c->L.s.T, c->d_autos, (cudaStream_t)stream);
   timer_end(c, CORR_KERNEL_AUTOS, (cudaStream_t)stream, tb);
   if (e != cudaSuccess) return cuda_fail(e, "corr_accumulate_autos: launch");
   c->n_auto += c->L.s.T;

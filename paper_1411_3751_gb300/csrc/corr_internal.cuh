@@ -109,7 +109,9 @@ inline long long round_up(long long x, long long m) { return (x + m - 1) / m * m
 cudaError_t launch_fp32(const Shape& s, const uint8_t* d_in, int T_blk, int flush_len, const int2* d_tiles,
                         int n_tiles, long long* d_cross, long long* d_autos, cudaStream_t st);
 
-// Autocorrelations of a block.
+// Autocorrelations of a block: launch_autos_tma where the rows allow it (autos_tma.cu), else launch_autos.
+bool autos_tma_supported(const Shape& s, const void* d_in);
+cudaError_t launch_autos_tma(const Shape& s, const uint8_t* d_in, int T_blk, long long* d_autos, int* d_err, cudaStream_t st);
 cudaError_t launch_autos(const Shape& s, const uint8_t* d_in, int T_blk, long long* d_autos, cudaStream_t st);
 
 // Fused unpack + tcgen05 X-engine (offset-domain products into d_cross, diagonal into d_autos).

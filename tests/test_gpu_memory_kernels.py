@@ -29,6 +29,17 @@ def _at_offset(torch, shape, dtype, skip):
     return torch.full((n + skip,), 7, dtype=dtype, device="cuda")[skip:].view(shape)
 
 
+def test_total_power_of_the_largest_samples(env):
+    """-8 - 8 i throughout: 128 a sample, every 16-bit sum of a full run of rows at its largest."""
+    corr, synth, torch = env
+    for N, C, T in ((1024, 700, 4500), (16, 1, 20000)):
+        x = torch.full((T, C, N), 0x88, dtype=torch.uint8, device="cuda")
+        with corr.Correlator(N, C, T, 2) as xc:
+            xc.accumulate_autos(x)
+            assert torch.all(xc.dump(corr.CORR_WHAT_AUTO) == 128 * T).item()
+            xc.sync()
+
+
 # channels of one block, of several blocks and of a block and a bit; both polarisation counts
 @pytest.mark.parametrize("N,C,T,npol", [(2, 5, 77, 2), (1, 3, 50, 1), (64, 7, 301, 2), (91, 3, 301, 1), (130, 2, 999, 2),
                                         (260, 2, 129, 2)])
@@ -68,7 +79,9 @@ def test_normalised_dump_is_the_nearest_float(env):
 
 
 # a few columns, many columns, a last partial column, one sample, a split time range; odd pointers
-@pytest.mark.parametrize("N,C,T", [(1, 1, 1), (2, 3, 5000), (7, 5, 65), (512, 3, 63), (33, 31, 129), (256, 400, 40)])
+@pytest.mark.parametrize("N,C,T", [(1, 1, 1), (2, 3, 5000), (7, 5, 65), (512, 3, 63), (33, 31, 129), (256, 400, 40),
+                                   (3, 1, 9001), (512, 160, 4100)])
+# and runs of the rows at the most that 16-bit sums hold, of the largest samples
 @pytest.mark.parametrize("skip", [0, 1, 5])
 def test_total_power_columns(env, N, C, T, skip):
     corr, synth, torch = env
