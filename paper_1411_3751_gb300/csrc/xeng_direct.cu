@@ -22,12 +22,13 @@
 // Roles: warp 0 TMA producer; warp 1 TMEM allocation and, in the even CTA, the MMA issuer; warps 4-11
 // converters (two sets of four warps, one TMEM lane quarter each, that take the stages in turn); warps
 // 12-19 epilogue. The accumulator takes 256 of the 512 columns and the A ring 192, so there is one
-// accumulator: the epilogue takes all of it into registers (128 a thread) before it adds to the int64
-// sums, and the MMAs wait for those loads only, about 1000 clocks an item. The register file is split by
-// setmaxnreg: 128 x 32 + 256 x 72 + 256 x 152 of the 640 x 96 of the launch.
+// accumulator: the epilogue takes all of it into registers, combined to complex products on the way (64 a
+// thread), before it adds to the int64 sums, and the MMAs wait for those loads only, about 1000 clocks an
+// item. The register file is split by setmaxnreg: 128 x 24 + 256 x 80 + 256 x 144 of the 640 x 96 of the
+// launch. (80 and 144, 512 inputs x 109 channels x 8000 samples: 388 us; 88 and 136: 393, 96 and 128: 397.)
 //
-// What bounds it: 512 inputs x 128 channels x 4 blocks of 8192 samples take 1.64 ms a launch (the two passes:
-// 1.245 + 4 x 0.253), 378 ns a stage. The MMAs alone need 62 x 4, with every barrier and copy but no conversion
+// What bounds it: 512 inputs x 128 channels x 4 blocks of 8192 samples take 1.60 ms a launch (the two passes:
+// 1.245 + 4 x 0.253), 370 ns a stage. The MMAs alone need 62 x 4, with every barrier and copy but no conversion
 // the stage takes 311; the rest is the converters' shared-memory traffic beside the MMAs' operand reads: without
 // the ldmatrix 340, without the B stores 332. A third set of converter warps, separate A and B warps and other
 // ring depths (5 + 8, 6 + 7) measured the same or slower.
@@ -89,7 +90,7 @@ struct Item {
 
 // The item's cells of this CTA into L2 while its MMAs run: for each a-station one run of the 64 c-inputs' products,
 // so that the loads of the old sums wait for L2 and not for DRAM. Short integrations are bound by the epilogue:
-// 512 inputs x 2400 channels x 240 samples 3.58 ms, 3.27 with the prefetch, 2.87 with the combined chunks below.
+// 512 inputs x 2400 channels x 240 samples 2.63 ms without the prefetch, 2.44 with it; x 109 x 8000 397 and 389 us.
 __device__ __forceinline__ void prefetch_cells(const xd::Args& a, const Item& it, uint32_t rank, int w, int lane, int lp,
                                                const long long* cross_f) {
   const int sc0 = (it.c0 + 64 * (int)rank) >> lp, n_sc = 64 >> lp, S = a.N >> lp;
@@ -153,7 +154,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(D_THREADS, 1)
   const uint32_t peer_abort = ptx::mapa_shared(const_cast<int*>(abort_flag), rank ^ 1u);
 
   if (warp < 4) {
-    ptx::setmaxnreg_dec<32>();
+    ptx::setmaxnreg_dec<24>();
     if (warp == 0 && lane == 0) {
       // ---------------- TMA producer (both CTAs) ----------------
       int slot = 0;
@@ -161,6 +162,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(D_THREADS, 1)
       for (long long w = pair; w < total && !*abort_flag; w += n_pairs) {
         const Item it(args, w);
         const int xc = it.f * args.ld + it.c0 + 64 * (int)rank, xa = it.f * args.ld + it.a0 + 64 * (int)rank;
+        const bool diag = it.c0 == it.a0;  // A and B are of the same inputs: one box
         xd::StagePos p(it.k0, args.n_kb);
         for (int k = it.k0; k < it.k1; ++k, p.next(args.n_kb)) {
           if (!ptx::mbar_wait(&raw_empty[slot], phase ^ 1, WAIT_NS)) {
@@ -168,9 +170,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(D_THREADS, 1)
             break;
           }
           uint8_t* dst = smem + slot * D_RAW_BYTES;
-          ptx::mbar_arrive_expect_tx(&raw_full[slot], D_RAW_BYTES);
+          ptx::mbar_arrive_expect_tx(&raw_full[slot], diag ? D_BOX : D_RAW_BYTES);
           ptx::tma_load_2d(dst, &args.map[p.blk], &raw_full[slot], xc, p.kb * KT);
-          ptx::tma_load_2d(dst + D_BOX, &args.map[p.blk], &raw_full[slot], xa, p.kb * KT);
+          if (!diag) ptx::tma_load_2d(dst + D_BOX, &args.map[p.blk], &raw_full[slot], xa, p.kb * KT);
           ++n_issued;
           if (++slot == D_RAW) {
             slot = 0;
@@ -233,7 +235,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(D_THREADS, 1)
     }
   } else if (warp < D_EPI_WARP) {
     // ---------------- converters ----------------
-    ptx::setmaxnreg_dec<72>();
+    ptx::setmaxnreg_dec<80>();
     const int q = warp & 3, set = (warp - 4) >> 2;
     const uint32_t raw0 = ptx::smem_u32(smem);
     // A: lane l addresses sample row l (+ 32 kk) of the warp's 16-byte column of inputs
@@ -241,7 +243,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(D_THREADS, 1)
     const uint32_t a_tmem = tbase + D_A_COL + ((uint32_t)(32 * q) << 16);
     // B: lane -> 16-byte column c, sample rows 32 q + 8 i + kr
     const int c = lane & 3, kr = lane >> 2;
-    const uint32_t b_off = (uint32_t)D_BOX + (uint32_t)(32 * q + kr) * 64 + (uint32_t)((c ^ ((kr >> 1) & 3)) << 4);
+    const uint32_t b_off = (uint32_t)(32 * q + kr) * 64 + (uint32_t)((c ^ ((kr >> 1) & 3)) << 4);
     const uint32_t o_off = (uint32_t)D_OP_OFF + (uint32_t)(4 * q) * 1024 + (uint32_t)kr * 128;
     const uint32_t o0_off = o_off + (uint32_t)(((2 * c) ^ kr) << 4), o1_off = o_off + (uint32_t)(((2 * c + 1) ^ kr) << 4);
     int rs = set, os = set;
@@ -268,7 +270,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(D_THREADS, 1)
 #pragma unroll
         for (int kk = 0; kk < 4; ++kk)
           ptx::ldmatrix_b8_x2_trans(raw + a_off + kk * 2048, x[4 * kk], x[4 * kk + 1], x[4 * kk + 2], x[4 * kk + 3]);
-        const uint8_t* b_src = smem + rs * D_RAW_BYTES + b_off;
+        const uint8_t* b_src = smem + rs * D_RAW_BYTES + (diag ? 0 : D_BOX) + b_off;
         uint4 r[4];
 #pragma unroll
         for (int i = 0; i < 4; ++i) r[i] = *reinterpret_cast<const uint4*>(b_src + i * 512);
@@ -354,7 +356,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(D_THREADS, 1)
     }
   } else {
     // ---------------- epilogue (both CTAs) ----------------
-    ptx::setmaxnreg_inc<152>();
+    ptx::setmaxnreg_inc<144>();
     const int q = warp & 3, half = (warp - D_EPI_WARP) >> 2;  // lane quarter; a-inputs 64 half .. + 63
     const bool im_lane = (lane & 16) != 0;
     const int lp = args.npol >> 1;
@@ -378,18 +380,21 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(D_THREADS, 1)
           break;
         }
         ptx::tc_fence_after();
-        uint32_t v[4][32];
+        int re[4][8], im[4][8];
         const uint32_t t = tbase + ((uint32_t)(32 * q) << 16) + 128 * half;
 #pragma unroll
-        for (int j = 0; j < 4; ++j) ptx::tmem_ld_32x32b_x32(t + 32 * j, v[j]);
-        ptx::tmem_ld_wait();
+        for (int j = 0; j < 4; j += 2) {  // all four at once: 128 words, and spills
+          uint32_t v[2][32];
+          ptx::tmem_ld_32x32b_x32(t + 32 * j, v[0]);
+          ptx::tmem_ld_32x32b_x32(t + 32 * j + 32, v[1]);
+          ptx::tmem_ld_wait();
+          xd::combine_chunk<16>(v[0], im_lane, re[j], im[j]);
+          xd::combine_chunk<16>(v[1], im_lane, re[j + 1], im[j + 1]);
+        }
         ptx::tc_fence_before();
         __syncwarp();
         if (lane == 0) ptx::mbar_arrive_remote(ptx::mapa_shared(tempty, 0));
         ++use;
-        int re[4][8], im[4][8];
-#pragma unroll
-        for (int j = 0; j < 4; ++j) xd::combine_chunk<16>(v[j], im_lane, re[j], im[j]);
         const int c_min = it.c0 + 64 * (int)rank + 16 * q, c_max = c_min + 15;
 #pragma unroll
         for (int j = 0; j < 4; ++j) {

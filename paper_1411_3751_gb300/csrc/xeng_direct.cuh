@@ -31,8 +31,8 @@ struct Args {
 // One 32-column chunk of an accumulator (16 a-inputs: column 8 (k / 4) + k % 4 = Re a_k, + 4 = Im a_k; with HALVES
 // columns k and 16 + k) as complex products: the lanes holding Re c and Im c of one c-input are XOR apart, exchange half of their columns and own
 // 8 a-inputs each, the Re lane the even, the Im lane the odd ones. (With two polarisations a warp's access then
-// covers whole station pairs, 512 neighbouring bytes.) Combining all of an accumulator first halves the words a
-// thread holds, and leaves registers for eight cells in flight.
+// covers whole station pairs, 512 neighbouring bytes.) Combining first halves the words a thread holds, and leaves
+// registers for eight cells in flight.
 template <int XOR, bool HALVES = false>
 __device__ __forceinline__ void combine_chunk(const uint32_t (&v)[32], bool im_lane, int (&re)[8], int (&im)[8]) {
 #pragma unroll
@@ -49,22 +49,25 @@ __device__ __forceinline__ void combine_chunk(const uint32_t (&v)[32], bool im_l
   }
 }
 
+// Cells as 32-bit offsets from the channel's first (a channel has less than 2^31 of them): pointers took twice the
+// registers and made the epilogue spill (512 inputs x 300 channels x 2048 samples 445 us, 359 with offsets).
 template <bool ADD>
-__device__ __forceinline__ void add_cells(longlong2* const (&cell)[8], uint32_t valid, const int (&re)[8], const int (&im)[8]) {
+__device__ __forceinline__ void add_cells(longlong2* __restrict__ base, const uint32_t (&cell)[8], uint32_t valid,
+                                          const int (&re)[8], const int (&im)[8]) {
   if (ADD) {
 #pragma unroll
     for (int m = 0; m < 8; ++m)
       if (valid & (1u << m)) {
-        atomicAdd(reinterpret_cast<unsigned long long*>(cell[m]), (unsigned long long)(long long)re[m]);
-        atomicAdd(reinterpret_cast<unsigned long long*>(cell[m]) + 1, (unsigned long long)(long long)im[m]);
+        atomicAdd(reinterpret_cast<unsigned long long*>(base + cell[m]), (unsigned long long)(long long)re[m]);
+        atomicAdd(reinterpret_cast<unsigned long long*>(base + cell[m]) + 1, (unsigned long long)(long long)im[m]);
       }
   } else {
     longlong2 old[8];
 #pragma unroll
-    for (int m = 0; m < 8; ++m) old[m] = *cell[m];
+    for (int m = 0; m < 8; ++m) old[m] = base[cell[m]];
 #pragma unroll
     for (int m = 0; m < 8; ++m)
-      if (valid & (1u << m)) *cell[m] = make_longlong2(old[m].x + re[m], old[m].y + im[m]);
+      if (valid & (1u << m)) base[cell[m]] = make_longlong2(old[m].x + re[m], old[m].y + im[m]);
   }
 }
 
@@ -75,17 +78,17 @@ template <bool ADD>
 __device__ __forceinline__ void add_chunk(const int (&re)[8], const int (&im)[8], bool im_lane, int c, int a_base, int N,
                                           int lp, long long* __restrict__ cross_f, long long* __restrict__ autos_f) {
   const unsigned sc = (unsigned)c >> lp, pc = (unsigned)c & (unsigned)lp;
-  longlong2* cell[8];
+  uint32_t cell[8];
   uint32_t valid = 0u;
 #pragma unroll
   for (int k = 0; k < 8; ++k) {
     const int a = a_base + (im_lane ? 1 : 0) + 2 * k;
-    cell[k] = reinterpret_cast<longlong2*>(cross_f);  // in-bounds placeholder for skipped cells (loaded, never stored)
+    cell[k] = 0u;  // in-bounds placeholder for skipped cells (loaded, never stored)
     if (a >= 0 && a < N && c >= 0 && c < N) {
       const unsigned sa = (unsigned)a >> lp;
       if (sa >= sc) {
         const unsigned b = sa * (sa + 1) / 2 + sc;
-        cell[k] += ((long long)b << (2 * lp)) + ((((unsigned)a & (unsigned)lp) << lp) + pc);
+        cell[k] = (b << (2 * lp)) + ((((unsigned)a & (unsigned)lp) << lp) + pc);
         valid |= 1u << k;
         if (a == c) {
           if (ADD)
@@ -96,7 +99,7 @@ __device__ __forceinline__ void add_chunk(const int (&re)[8], const int (&im)[8]
       }
     }
   }
-  add_cells<ADD>(cell, valid, re, im);
+  add_cells<ADD>(reinterpret_cast<longlong2*>(cross_f), cell, valid, re, im);
 }
 
 // The same for two polarisations where every cell of the chunk is stored and off the diagonal: no checks, and the
@@ -105,12 +108,11 @@ template <bool ADD>
 __device__ __forceinline__ void add_chunk_full(const int (&re)[8], const int (&im)[8], bool im_lane, int c, int a_base,
                                                long long* __restrict__ cross_f) {
   const unsigned sa = (unsigned)a_base >> 1;
-  longlong2* p = reinterpret_cast<longlong2*>(cross_f) + 4 * (long long)(sa * (sa + 1) / 2 + ((unsigned)c >> 1)) + (c & 1) +
-                 (im_lane ? 2 : 0);
-  longlong2* cell[8];
+  const unsigned p = 4 * (sa * (sa + 1) / 2 + ((unsigned)c >> 1)) + (unsigned)(c & 1) + (im_lane ? 2u : 0u);
+  uint32_t cell[8];
 #pragma unroll
   for (int k = 0; k < 8; ++k) cell[k] = p + 4 * (k * sa + (unsigned)(k * (k + 1) / 2));
-  add_cells<ADD>(cell, 0xFFu, re, im);
+  add_cells<ADD>(reinterpret_cast<longlong2*>(cross_f), cell, 0xFFu, re, im);
 }
 
 // Stage k of an item's blocks: block k / n_kb, sample 128 (k % n_kb).
