@@ -19,6 +19,10 @@
 // Why A in TMEM: with both operands in shared memory a stage moves 48 KB through the load/store path in the
 // 512 clocks of its MMAs; so it is 32 KB, and the MMAs read only B from shared memory.
 //
+// Rows of any length: a TMA box starts on a 16-byte boundary, so channel f's tiles start at the boundary at or
+// below its first byte, (f N) mod 16 inputs before input 0. Both sides are shifted alike; the rows that belong
+// to the neighbouring channel give products that the epilogue leaves out, as it does those past N.
+//
 // Roles: warp 0 TMA producer; warp 1 TMEM allocation and, in the even CTA, the MMA issuer; warps 4-11
 // converters (two sets of four warps, one TMEM lane quarter each, that take the stages in turn); warps
 // 12-19 epilogue. The accumulator takes 256 of the 512 columns and the A ring 192, so there is one
@@ -70,7 +74,7 @@ __device__ __forceinline__ void direct_error(int* err, volatile int* abort_flag,
 }
 
 struct Item {
-  int f, c0, a0, k0, k1;
+  int f, c0, a0, k0, k1;  // c0, a0: -15 .. N - 1
   __device__ __forceinline__ Item(const xd::Args& a, long long w) {
     int t = (int)(w % a.n_tiles);
     const long long r = w / a.n_tiles;
@@ -81,8 +85,9 @@ struct Item {
       t -= a.nb - ci;
       ++ci;
     }
-    c0 = 128 * ci;
-    a0 = 128 * (ci + t);
+    const int shift = (int)((long long)f * a.ld & 15);  // inputs before input 0 that the first tile holds
+    c0 = 128 * ci - shift;
+    a0 = 128 * (ci + t) - shift;
     k0 = sp * a.kps;
     k1 = min(a.n_k, k0 + a.kps);
   }
@@ -93,10 +98,10 @@ struct Item {
 // 512 inputs x 2400 channels x 240 samples 2.63 ms without the prefetch, 2.44 with it; x 109 x 8000 397 and 389 us.
 __device__ __forceinline__ void prefetch_cells(const xd::Args& a, const Item& it, uint32_t rank, int w, int lane, int lp,
                                                const long long* cross_f) {
-  const int sc0 = (it.c0 + 64 * (int)rank) >> lp, n_sc = 64 >> lp, S = a.N >> lp;
+  const int c0 = (it.c0 + 64 * (int)rank) >> lp, sc0 = max(c0, 0), S = a.N >> lp;
   for (int i = 32 * w + lane; i < 128 >> lp; i += 32 * D_EPI_WARPS) {
     const int sa = (it.a0 >> lp) + i;
-    const int end = min(min(sc0 + n_sc, sa + 1), S);
+    const int end = min(min(c0 + (64 >> lp), sa + 1), S);
     if (sa < S && sc0 < end) {
       const unsigned b = (unsigned)sa * (unsigned)(sa + 1) / 2 + (unsigned)sc0;
       ptx::prefetch_l2(cross_f + 2 * ((long long)b << (2 * lp)), (uint32_t)(end - sc0) << (4 + 2 * lp));
@@ -345,7 +350,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(D_THREADS, 1)
 #pragma unroll
           for (int i = 0; i < 4; ++i) {
             const int n = it.c0 + 64 * (int)rank + 16 * q + (lane >> 2) + 8 * (i >> 1);
-            if (n < args.N && s[i] != 0) {
+            if (n >= 0 && n < args.N && s[i] != 0) {
               const long long idx = ((long long)it.f * args.N + n) * 2 + (i & 1);
               atomicAdd(reinterpret_cast<unsigned long long*>(args.s1 + idx), s[i]);
               atomicAdd(reinterpret_cast<unsigned long long*>(args.s2 + idx), s[i]);
@@ -399,7 +404,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(D_THREADS, 1)
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
           const int a_base = it.a0 + 64 * half + 16 * j;
-          if (lp == 1 && a_base > c_max && a_base + 16 <= args.N && c_max < args.N)
+          if (lp == 1 && c_min >= 0 && a_base > c_max && a_base + 16 <= args.N)
             xd::add_chunk_full<ADD>(re[j], im[j], im_lane, c, a_base, cross_f);
           else if (a_base + 15 >= c_min - lp && a_base < args.N && c_min < args.N)  // not all above the diagonal or past N
             xd::add_chunk<ADD>(re[j], im[j], im_lane, c, a_base, args.N, lp, cross_f, autos_f);
@@ -445,8 +450,13 @@ int direct_max_pairs() {
 
 }  // namespace
 
+// Whole rows of 16 bytes (TMA's stride). Where channels start between 16-byte boundaries the first tile holds up to
+// 16 - gcd(N, 16) inputs of the channel before; that may not take one more row of tiles (repack.cu takes those).
 bool xeng_direct_supported(const Shape& s, int ld, const void* d_in) {
-  return s.N > 64 && ld % 16 == 0 && reinterpret_cast<uintptr_t>(d_in) % 16 == 0 && (long long)ld * s.C < (1LL << 31);
+  const long long row = (long long)ld * s.C;
+  const int shift = (16 - (ld & -ld)) & 15;  // the largest of any channel
+  return s.N > 64 && row % 16 == 0 && reinterpret_cast<uintptr_t>(d_in) % 16 == 0 && row < (1LL << 31) &&
+         (s.N + shift + 127) / 128 == (s.N + 127) / 128;
 }
 
 int direct_splits(long long items, int slots, int n_k, int overhead) {

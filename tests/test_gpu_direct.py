@@ -106,6 +106,16 @@ def test_rows_that_tma_does_not_take(env, N, C, npol, skip, T, blocks):
     _check(env, _host(env[1], N, C, T, blocks), npol, skip=skip, blocks=blocks)
 
 
+# whole rows of 16 bytes, channels between: every shift of the tiles (steps of 1, 2, 4 and 8 inputs), counts that with
+# the largest shift just fill the last tile (113, 114, 116, 120, 241, 242, 248) and one that does not (122, repacked)
+@pytest.mark.parametrize("N,C,npol", [(65, 16, 1), (66, 8, 2), (68, 4, 2), (72, 2, 2), (72, 4, 1), (113, 16, 1), (114, 8, 2),
+                                      (116, 4, 2), (120, 2, 2), (122, 8, 2), (131, 16, 1), (200, 2, 2), (241, 16, 1),
+                                      (242, 8, 2), (248, 2, 2), (340, 4, 2)])
+@pytest.mark.parametrize("T,blocks", [(1, 1), (129, 1), (700, 2)])
+def test_channels_between_16_byte_boundaries(env, N, C, npol, T, blocks):
+    _check(env, _host(env[1], N, C, T, blocks), npol, blocks=blocks)
+
+
 def test_schedules_that_were_asked_for_mix_with_the_default(env):
     """Default, tile plan, build schedule and FP32 launches in one integration."""
     corr, synth, torch = env
