@@ -7,7 +7,9 @@
 // inputs, or g channels of N inputs with g N <= 64 (their products are the diagonal blocks; those across
 // channels are not used). With 33 to 63 inputs the unit runs into the next channel, whose rows are not
 // used either. An item is two neighbouring units, so that TMA boxes are 128 bytes x 128 samples, and a
-// range of stages of 128 samples.
+// range of stages of 128 samples. A unit that starts between 16-byte boundaries takes the columns from the
+// boundary below on, and the rows of the unit before are not used: g leaves room for them. (Without that, such
+// counts were repacked first: 20 inputs x 1200 channels x 4096 samples 91 us, 52 in place; 31 inputs 115 and 94.)
 //
 // A and B of a unit's MMA are the same rows. With both read from one shared-memory tile a stage moved 128 KB
 // through shared memory (MMA reads 64, conversion 48, TMA 16) and took 660 ns, 1.3 times what HBM needs; so A
@@ -112,7 +114,7 @@ __global__ void __launch_bounds__(S_THREADS, 1) xeng_small_kernel(const __grid_c
       uint32_t phase = 0, n_issued = 0;
       for (long long w = blockIdx.x; w < total && !*abort_flag; w += gridDim.x) {
         const SmallItem it(args, w, n_pairs);
-        const int x = (int)(it.p * 2 * args.ub);
+        const int x = (int)(it.p * 2 * args.ub) & ~15;
         xd::StagePos p(it.k0, args.n_kb);
         for (int k = it.k0; k < it.k1; ++k, p.next(args.n_kb)) {
           if (!ptx::mbar_wait(&raw_empty[slot], phase ^ 1, WAIT_NS)) {
@@ -188,8 +190,7 @@ __global__ void __launch_bounds__(S_THREADS, 1) xeng_small_kernel(const __grid_c
     // ---------------- converters: lane quarter q of unit h, every S_SETS-th stage ----------------
     ptx::setmaxnreg_dec<56>();
     const int q = warp & 3, h = ((warp - 4) >> 2) & 1, set = (warp - 4) >> 3;
-    // lane l addresses sample row l (+ 32 kk) of the 16-byte column of the quarter's inputs (128-byte swizzle)
-    const uint32_t a_off = ptx::smem_u32(smem) + (uint32_t)lane * 128 + (uint32_t)(((h * args.ub / 16 + q) ^ (lane & 7)) << 4);
+    const uint32_t raw0 = ptx::smem_u32(smem) + (uint32_t)lane * 128;
     const uint32_t a_tmem = tbase + S_A_COL + 32 * h + ((uint32_t)(32 * q) << 16);
     // B row 32 q + lane / 4 (Re; + 8, and + 16 for Im), samples 16 j + 4 (lane % 4) ..: 16-byte chunk j of the row
     const int br = lane >> 2;
@@ -200,6 +201,9 @@ __global__ void __launch_bounds__(S_THREADS, 1) xeng_small_kernel(const __grid_c
     bool ok = true;
     for (long long w = blockIdx.x; w < total && ok && !*abort_flag; w += gridDim.x) {
       const SmallItem it(args, w, n_pairs);
+      // lane l addresses sample row l (+ 32 kk) of the 16-byte column of the quarter's inputs (128-byte swizzle)
+      const int x0 = (int)(it.p * 2 * args.ub) & 15, col = ((x0 + h * args.ub) >> 4) + q, shift = (x0 + h * args.ub) & 15;
+      const uint32_t a_off = raw0 + (uint32_t)((col ^ (lane & 7)) << 4);
       xd::StagePos p(it.k0 + ahead, args.n_kb);
       uint32_t sum[4] = {0u, 0u, 0u, 0u};  // Re, Im of inputs lane / 4 and lane / 4 + 8 of the quarter's 16
       for (int k = it.k0 + ahead; k < it.k1; k += S_SETS, p.next(args.n_kb, S_SETS)) {
@@ -274,10 +278,10 @@ __global__ void __launch_bounds__(S_THREADS, 1) xeng_small_kernel(const __grid_c
         unsigned long long s = sum[i];
         s += __shfl_xor_sync(0xffffffffu, s, 1);
         s += __shfl_xor_sync(0xffffffffu, s, 2);
-        const int in = 16 * q + br + 8 * (i >> 1);  // input row of the unit
+        const int in = 16 * q + br + 8 * (i >> 1) - shift;  // input row of the unit
         const int ch = in / args.ld, n = in - ch * args.ld;
         const long long f = u * args.g + ch;
-        if ((lane & 3) == 0 && ch < args.g && n < args.N && u < args.n_units && f < args.C) {
+        if ((lane & 3) == 0 && in >= 0 && ch < args.g && n < args.N && u < args.n_units && f < args.C) {
           const long long idx = (f * args.N + n) * 2 + (i & 1);
           atomicAdd(reinterpret_cast<unsigned long long*>(args.s1 + idx), s);
           atomicAdd(reinterpret_cast<unsigned long long*>(args.s2 + idx), s);
@@ -290,17 +294,19 @@ __global__ void __launch_bounds__(S_THREADS, 1) xeng_small_kernel(const __grid_c
     const int q = warp & 3, h = (warp - S_EPI_WARP) >> 2;
     const bool im_lane = (lane & 16) != 0;
     const int lp = args.npol >> 1;
-    const int ic = 16 * q + (lane & 15);  // c-input of the unit
-    const int ch = ic / args.ld, c = ic - ch * args.ld;
-    // the chunks (16 a-inputs) that hold this warp's channels, from the diagonal on
-    const int last = min(64, ((16 * q + 15) / args.ld + 1) * args.ld);
-    const int cc_end = (last + 15) / 16;
     uint32_t use = 0;
     bool ok = true;
     for (long long w = blockIdx.x; w < total && ok; w += gridDim.x) {
       const SmallItem it(args, w, n_pairs);
-      const long long u = 2 * it.p + h, f = u * args.g + ch;
-      const bool live = ch < args.g && u < args.n_units && f < args.C;
+      const long long u = 2 * it.p + h;
+      const int shift = (int)(u * args.ub) & 15;
+      const int ic = 16 * q + (lane & 15) - shift;  // c-input of the unit
+      const int ch = ic / args.ld, c = ic - ch * args.ld;
+      // the chunks (16 a-inputs) that hold this warp's channels, from the diagonal on
+      const int last = min(64, ((16 * q + 15 - shift) / args.ld + 1) * args.ld + shift);
+      const int cc_end = (last + 15) / 16;
+      const long long f = u * args.g + ch;
+      const bool live = ic >= 0 && ch < args.g && u < args.n_units && f < args.C;
       long long* cross_f = args.cross + (live ? f : 0) * args.Bs * args.npol * args.npol * 2;
       long long* autos_f = args.autos + (live ? f : 0) * args.N;
       for (int k0 = it.k0; k0 < it.k1; k0 += chunk_k) {
@@ -333,7 +339,7 @@ __global__ void __launch_bounds__(S_THREADS, 1) xeng_small_kernel(const __grid_c
 #pragma unroll
         for (int cc = 0; cc < 4; ++cc)
           if (u < args.n_units && cc >= q && cc < cc_end)
-            xd::add_chunk<ADD>(re[cc], im[cc], im_lane, live ? c : -1, 16 * cc - ch * args.ld, args.N, lp, cross_f, autos_f);
+            xd::add_chunk<ADD>(re[cc], im[cc], im_lane, live ? c : -1, 16 * cc - shift - ch * args.ld, args.N, lp, cross_f, autos_f);
       }
     }
   }
@@ -343,11 +349,11 @@ __global__ void __launch_bounds__(S_THREADS, 1) xeng_small_kernel(const __grid_c
   if (warp == 1) ptx::tmem_dealloc(tbase, TMEM_COLS);
 }
 
-// Channels (of ld stored inputs) per 64-input unit: as many as fit with a unit of whole 16-byte columns; 0 if none.
+// Channels (of ld stored inputs) per 64-input unit: as many as fit behind the inputs that a unit's first 16-byte
+// column may hold of the one before (16 - gcd(16, unit) at most); 0 if not even one does.
 int small_group(int ld) {
-  if (ld > 64) return 0;
   for (int g = 64 / ld; g >= 1; --g)
-    if (g * ld % 16 == 0) return g;
+    if (g * ld + ((16 - (g * ld & -(g * ld))) & 15) <= 64) return g;
   return 0;
 }
 

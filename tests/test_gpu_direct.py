@@ -107,10 +107,13 @@ def test_rows_that_tma_does_not_take(env, N, C, npol, skip, T, blocks):
 
 
 # whole rows of 16 bytes, channels between: every shift of the tiles (steps of 1, 2, 4 and 8 inputs), counts that with
-# the largest shift just fill the last tile (113, 114, 116, 120, 241, 242, 248) and one that does not (122, repacked)
+# the largest shift just fill the last tile (113, 114, 116, 120, 241, 242, 248) and one that does not (122, repacked);
+# up to 64 inputs units of one or more channels, the same (5, 10, 31, 49, 50, 52, 56 fill the unit; 60 is repacked)
 @pytest.mark.parametrize("N,C,npol", [(65, 16, 1), (66, 8, 2), (68, 4, 2), (72, 2, 2), (72, 4, 1), (113, 16, 1), (114, 8, 2),
                                       (116, 4, 2), (120, 2, 2), (122, 8, 2), (131, 16, 1), (200, 2, 2), (241, 16, 1),
-                                      (242, 8, 2), (248, 2, 2), (340, 4, 2)])
+                                      (242, 8, 2), (248, 2, 2), (340, 4, 2), (3, 48, 1), (5, 48, 1), (7, 32, 1), (10, 24, 2),
+                                      (14, 8, 2), (20, 12, 2), (22, 8, 2), (28, 4, 2), (31, 32, 1), (49, 16, 1), (50, 8, 2),
+                                      (52, 4, 2), (56, 6, 2), (60, 4, 2)])
 @pytest.mark.parametrize("T,blocks", [(1, 1), (129, 1), (700, 2)])
 def test_channels_between_16_byte_boundaries(env, N, C, npol, T, blocks):
     _check(env, _host(env[1], N, C, T, blocks), npol, blocks=blocks)
