@@ -73,8 +73,17 @@ __device__ __forceinline__ void direct_error(int* err, volatile int* abort_flag,
   atomicCAS(err, 0, code);
 }
 
+// Inputs of the channel before that the first tile of channel f starts with.
+__device__ __forceinline__ int tile_shift(const xd::Args& a, int f) { return (int)((unsigned)f * (unsigned)a.ld & 15u); }
+
 struct Item {
-  int f, c0, a0, k0, k1;  // c0, a0: -15 .. N - 1
+  int f, c0, a0, k0, k1;  // c0, a0: rows of the channel's tiles
+  // From tile rows to inputs, -15 .. N - 1.
+  __device__ __forceinline__ void to_inputs(const xd::Args& a) {
+    const int shift = tile_shift(a, f);
+    c0 -= shift;
+    a0 -= shift;
+  }
   __device__ __forceinline__ Item(const xd::Args& a, long long w) {
     int t = (int)(w % a.n_tiles);
     const long long r = w / a.n_tiles;
@@ -85,9 +94,8 @@ struct Item {
       t -= a.nb - ci;
       ++ci;
     }
-    const int shift = (int)((long long)f * a.ld & 15);  // inputs before input 0 that the first tile holds
-    c0 = 128 * ci - shift;
-    a0 = 128 * (ci + t) - shift;
+    c0 = 128 * ci;
+    a0 = 128 * (ci + t);
     k0 = sp * a.kps;
     k1 = min(a.n_k, k0 + a.kps);
   }
@@ -165,7 +173,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(D_THREADS, 1)
       int slot = 0;
       uint32_t phase = 0, n_issued = 0;
       for (long long w = pair; w < total && !*abort_flag; w += n_pairs) {
-        const Item it(args, w);
+        Item it(args, w);
+        it.to_inputs(args);
         const int xc = it.f * args.ld + it.c0 + 64 * (int)rank, xa = it.f * args.ld + it.a0 + 64 * (int)rank;
         const bool diag = it.c0 == it.a0;  // A and B are of the same inputs: one box
         xd::StagePos p(it.k0, args.n_kb);
@@ -338,6 +347,11 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(D_THREADS, 1)
       ahead = (ahead - (it.k1 - it.k0)) % D_SETS;
       if (ahead < 0) ahead += D_SETS;
       if (diag && ok) {
+        // anew, not from `it`: the shift kept over the loop above slows the conversion down (1.640 ms a launch, 1.620)
+        long long wl = w;
+        asm volatile("" : "+l"(wl));
+        Item d(args, wl);
+        d.to_inputs(args);
         unsigned long long s[4];
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
@@ -349,9 +363,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(D_THREADS, 1)
         if ((lane & 3) == 0) {
 #pragma unroll
           for (int i = 0; i < 4; ++i) {
-            const int n = it.c0 + 64 * (int)rank + 16 * q + (lane >> 2) + 8 * (i >> 1);
+            const int n = d.c0 + 64 * (int)rank + 16 * q + (lane >> 2) + 8 * (i >> 1);
             if (n >= 0 && n < args.N && s[i] != 0) {
-              const long long idx = ((long long)it.f * args.N + n) * 2 + (i & 1);
+              const long long idx = ((long long)d.f * args.N + n) * 2 + (i & 1);
               atomicAdd(reinterpret_cast<unsigned long long*>(args.s1 + idx), s[i]);
               atomicAdd(reinterpret_cast<unsigned long long*>(args.s2 + idx), s[i]);
             }
@@ -368,7 +382,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(D_THREADS, 1)
     uint32_t use = 0;
     bool ok = true;
     for (long long w = pair; w < total && ok; w += n_pairs) {
-      const Item it(args, w);
+      Item it(args, w);
+      it.to_inputs(args);
       const int c = it.c0 + 64 * (int)rank + 16 * q + (lane & 15);
       long long* cross_f = args.cross + (long long)it.f * args.Bs * args.npol * args.npol * 2;
       long long* autos_f = args.autos + (long long)it.f * args.N;
