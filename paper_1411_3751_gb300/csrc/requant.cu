@@ -7,16 +7,21 @@
 // Per component: x = fl32(gain * v) (one IEEE single-precision product, v converted to float
 // first), q = clip(round-half-even(x), lo, 7) with lo = -8 (or -7 when symmetric), NaN -> 0.
 //
-// HBM-bound transpose: a block stages a 128-channel x 32-input tile of one time sample in shared
-// memory. Each warp reads 128 consecutive channels of 4 inputs (1 KiB contiguous per input row) and
-// the block writes 128 output rows of 32 consecutive input bytes.
+// HBM-bound transpose: a block stages a 64-channel x 32-input tile of one time sample in shared
+// memory. Each warp reads 64 consecutive channels of 4 inputs (512 contiguous bytes per input row) and
+// the block writes 64 output rows of 32 consecutive input bytes. Small tiles, because the block's loads
+// and stores alternate: eight blocks an SM in different phases keep the memory busy, where 128-channel
+// tiles (16 loads a thread) allowed five. 512 inputs x 256 spectra x 2398 of 4096 channels 500 -> 460 us (90%
+// of the measured copy bandwidth); tiles of 64 inputs 551, of 256 channels 1423, of 32 channels 533.
+#include <algorithm>
+
 #include "corr_internal.cuh"
 
 namespace corr {
 namespace {
 
-constexpr int RQ_CH = 128, RQ_IN = 32, RQ_NT = 256;
-constexpr int RQ_CPL = RQ_CH / 32;            // channels per lane (4)
+constexpr int RQ_CH = 64, RQ_IN = 32, RQ_NT = 256;
+constexpr int RQ_CPL = RQ_CH / 32;            // channels per lane (2)
 constexpr int RQ_IPW = RQ_IN / (RQ_NT / 32);  // inputs per warp (4)
 
 // x = fl32(g v); round to nearest even with cvt.rni (NaN converts to 0, out-of-range values saturate),
@@ -37,37 +42,42 @@ __device__ __forceinline__ float2 as_float2<float2>(const float2& v) {
   return v;
 }
 
-// Position of a block in its sequence of steps: item = (input tile nt, time t), chunk of channels.
-// Items advance by gridDim.x = (dnt, dt) in (tile, time) coordinates; no division per step.
+// Position of a block in its sequence of steps: item = (input tile nt, q = time and segment of the channels),
+// chunk of channels. Items advance by gridDim.x = (dnt, dq); no division per step.
 struct RqIter {
-  int nt, t, chunk;
-  __device__ __forceinline__ void next(int chunks, int tiles_n, int dnt, int dt) {
-    if (++chunk == chunks) {
-      chunk = 0;
-      nt += dnt;
-      t += dt;
-      if (nt >= tiles_n) {
-        nt -= tiles_n;
-        ++t;
-      }
+  int nt, q, t, chunk, end;
+  __device__ __forceinline__ void open(int chunks, int segs, int cps) {
+    t = segs == 1 ? q : q / segs;
+    chunk = (q - t * segs) * cps;
+    end = min(chunks, chunk + cps);
+  }
+  __device__ __forceinline__ void next(int tiles_n, int dnt, int dq, int chunks, int segs, int cps) {
+    if (++chunk < end) return;
+    nt += dnt;
+    q += dq;
+    if (nt >= tiles_n) {
+      nt -= tiles_n;
+      ++q;
     }
+    open(chunks, segs, cps);
   }
 };
 
-// Persistent: work item w = (input tile w % tiles_n, time sample w / tiles_n); block b takes items
-// b, b + gridDim.x, ... and walks each item's rows across the selected channels in 128-channel
-// chunks. Blocks running together hold consecutive time samples of every input tile. Warp w owns
+// Persistent: work item w = (input tile w % tiles_n, time sample and segment of the channels w / tiles_n); block b
+// takes items b, b + gridDim.x, ... and walks each item's rows across its channels in 64-channel
+// chunks. Blocks running together hold neighbouring times of every input tile. Warp w owns
 // inputs n0 + 4 w .. + 3 and lane l channels c0 + l + 32 k, so a thread packs its four inputs' bytes
-// into one 32-bit shared-memory store per channel; the next chunk's 16 loads are in flight while the
+// into one 32-bit shared-memory store per channel; the next chunk's 8 loads are in flight while the
 // current tile is written out.
 template <typename T2>
-__global__ void __launch_bounds__(RQ_NT) requant_kernel(const T2* __restrict__ in, int N, int T, int F, int chan0,
+__global__ void __launch_bounds__(RQ_NT, 8) requant_kernel(const T2* __restrict__ in, int N, int T, int F, int chan0,
                                                         int C, float gain, const float* __restrict__ gains, int lo,
-                                                        bool words, uint8_t* __restrict__ out) {
+                                                        bool words, int segs, int cps, uint8_t* __restrict__ out) {
   __shared__ __align__(16) uint8_t tile[RQ_CH][RQ_IN + 4];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int tiles_n = (N + RQ_IN - 1) / RQ_IN, chunks = (C + RQ_CH - 1) / RQ_CH;
-  const int dnt = (int)(gridDim.x % (unsigned)tiles_n), dt = (int)(gridDim.x / (unsigned)tiles_n);
+  const int dnt = (int)(gridDim.x % (unsigned)tiles_n), dq = (int)(gridDim.x / (unsigned)tiles_n);
+  const int q_end = T * segs;
   float2 v[RQ_IPW][RQ_CPL];
   auto load = [&](const RqIter& it) {
     const int n0 = it.nt * RQ_IN + RQ_IPW * warp, c0 = it.chunk * RQ_CH + lane;
@@ -82,9 +92,10 @@ __global__ void __launch_bounds__(RQ_NT) requant_kernel(const T2* __restrict__ i
       }
     }
   };
-  RqIter it{(int)(blockIdx.x % (unsigned)tiles_n), (int)(blockIdx.x / (unsigned)tiles_n), 0};
-  if (it.t < T) load(it);
-  while (it.t < T) {
+  RqIter it{(int)(blockIdx.x % (unsigned)tiles_n), (int)(blockIdx.x / (unsigned)tiles_n), 0, 0, 0};
+  it.open(chunks, segs, cps);
+  if (it.q < q_end) load(it);
+  while (it.q < q_end) {
     const int n0 = it.nt * RQ_IN, c0 = it.chunk * RQ_CH, t = it.t;
 #pragma unroll
     for (int k = 0; k < RQ_CPL; ++k) {
@@ -97,9 +108,9 @@ __global__ void __launch_bounds__(RQ_NT) requant_kernel(const T2* __restrict__ i
     }
     __syncthreads();
     RqIter nx = it;
-    nx.next(chunks, tiles_n, dnt, dt);
-    if (nx.t < T) load(nx);  // next chunk's loads in flight during the writes
-    // write: 128 channel rows x 32 input bytes, as 32-bit words where the row allows
+    nx.next(tiles_n, dnt, dq, chunks, segs, cps);
+    if (nx.q < q_end) load(nx);  // next chunk's loads in flight during the writes
+    // write: 64 channel rows x 32 input bytes, as 32-bit words where the row allows
     if (words) {
       for (int w = tid; w < RQ_CH * (RQ_IN / 4); w += RQ_NT) {
         const int cr = w / (RQ_IN / 4), nw = (w % (RQ_IN / 4)) * 4;
@@ -131,18 +142,27 @@ cudaError_t launch_requant(const void* d_in, int in_type, int N, int T, int F, i
     e = in_type == 0 ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, requant_kernel<int2>, RQ_NT, 0)
                      : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, requant_kernel<float2>, RQ_NT, 0);
   if (e != cudaSuccess) return e;
-  const long long items = (long long)((N + RQ_IN - 1) / RQ_IN) * T;
+  const long long rows = (long long)((N + RQ_IN - 1) / RQ_IN) * T;
   long long blocks = (long long)sms * (per_sm > 0 ? per_sm : 1);
+  const int chunks = (C + RQ_CH - 1) / RQ_CH;
+  // Where whole rows would give a block fewer than eight items the channels are divided: few times leave blocks
+  // idle (512 inputs x 8 spectra 46 us undivided, 19), and a last round of items that few blocks have takes as long as
+  // a full one (64 spectra x 2048 channels: 103 us from four items a block on, 98 from eight, 103 from sixteen).
+  int segs = 1;
+  if (rows < 8 * blocks) segs = (int)std::min<long long>(chunks, (8 * blocks + rows - 1) / rows);
+  const int cps = (chunks + segs - 1) / segs;
+  segs = (chunks + cps - 1) / cps;
+  const long long items = rows * segs;
   if (blocks > items) blocks = items;
   const dim3 grid((unsigned)blocks);
   const int lo = symmetric ? -7 : -8;
   const bool words = (N & 3) == 0 && (reinterpret_cast<uintptr_t>(d_out) & 3) == 0;  // 32-bit stores stay aligned
   if (in_type == 0)
     requant_kernel<int2><<<grid, RQ_NT, 0, st>>>(static_cast<const int2*>(d_in), N, T, F, chan0, C, gain, d_gains, lo,
-                                                  words, d_out);
+                                                  words, segs, cps, d_out);
   else
     requant_kernel<float2><<<grid, RQ_NT, 0, st>>>(static_cast<const float2*>(d_in), N, T, F, chan0, C, gain, d_gains,
-                                                    lo, words, d_out);
+                                                    lo, words, segs, cps, d_out);
   return cudaGetLastError();
 }
 

@@ -118,3 +118,14 @@ def test_corner_turn_granules(env, T, C, n_local, chan_b, in_b, skip):
     d_in.copy_(torch.from_numpy(src))
     corr.corr_corner_turn_unpack(d_in.data_ptr(), T, C, N, in_b, d_out.data_ptr(), st)
     assert np.array_equal(d_out.cpu().numpy(), y)
+
+
+# chunks of 64 channels: one, an edge, a last one of 1; rows divided into segments of one and of several chunks, with
+# a shorter last one; more rows than are divided
+@pytest.mark.parametrize("N,T,F,chan0,C", [(1, 1, 64, 0, 64), (33, 1, 200, 1, 65), (40, 2, 4096, 0, 4096), (35, 3, 700, 9, 641),
+                                           (512, 40, 1100, 3, 1090), (512, 300, 140, 0, 129), (30, 6000, 70, 2, 66)])
+def test_requantize_segments(env, N, T, F, chan0, C):
+    corr, _, torch = env
+    x = np.random.default_rng(N + T).integers(-1 << 17, 1 << 17, (N, T, F, 2), dtype=np.int32)
+    got = corr.requantize(torch.from_numpy(x).cuda(), chan0, C, gain=2.0 ** -14).cpu().numpy()
+    assert np.array_equal(got, oracle.requantize(x, chan0, C, gain=2.0 ** -14))
