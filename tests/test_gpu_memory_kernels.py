@@ -78,6 +78,25 @@ def test_normalised_dump_is_the_nearest_float(env):
         xc.sync()
 
 
+# sums about 2^30, 2^31 and past 32 bits (one input pair of the most negative samples, a few of them different), both signs
+@pytest.mark.parametrize("T", [(1 << 23) + 5, (1 << 24) - 1, (1 << 24) + 9, (1 << 25) + 3])
+@pytest.mark.parametrize("npol", [1, 2])
+def test_normalised_dump_of_large_sums(env, T, npol):
+    corr, _, torch = env
+    x = torch.full((T, 1, 4), 0x88, dtype=torch.uint8, device="cuda")
+    x[:, 0, 2] = 0x78  # 7 - 8i: products of both signs in both parts
+    x[::1001, 0, 1] = 0x3F
+    with corr.Correlator(4, 1, T, npol) as xc:
+        xc.accumulate(x)
+        v = xc.dump(corr.CORR_WHAT_CROSS)
+        assert int(v.abs().max()) > 1 << 30
+        q = xc.dump(corr.CORR_WHAT_CROSS, corr.CORR_FMT_CF32_NORM)
+        f = xc.dump(corr.CORR_WHAT_CROSS, corr.CORR_FMT_CF32)
+        xc.sync()
+    assert torch.equal(q, (v.double() / float(T)).float())
+    assert torch.equal(f, v.float())
+
+
 # a few columns, many columns, a last partial column, one sample, a split time range; odd pointers
 @pytest.mark.parametrize("N,C,T", [(1, 1, 1), (2, 3, 5000), (7, 5, 65), (512, 3, 63), (33, 31, 129), (256, 400, 40),
                                    (3, 1, 9001), (512, 160, 4100)])
