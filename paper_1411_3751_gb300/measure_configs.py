@@ -4,14 +4,13 @@
   bound case (the FP32 path is the paper's arithmetic);
 
 * small: 32 and 64 inputs (LWA1's 64-input system) x 2400 channels x 4 blocks of 8192 samples, FP8
-  tensor path: Tera-CMAC/s and the HBM traffic of the two passes (input read once, operand written
-  and read back) against the measured copy bandwidth, the bound for these small arrays;
+  tensor path: Tera-CMAC/s and the samples' bytes, read once, against the measured copy bandwidth;
 * precision: 512 inputs x 256 channels x 65536 samples with saturation-heavy segments; X-engine time
   with in-chip partial sums flushed to int64 every 4096 / 16384 / 65536 samples on the FP8 tcgen05
   path and every 16384 / 65536 samples on the int8 mma.sync path (the flush overhead is the
   difference to the 65536 case);
 * group: sub-arrays of 32, 64, 200, 256 and 512 inputs with 2400, 600, 300, 150 and 109 channels of
-  4096 samples: one autotuned grouped launch replayed from a CUDA graph vs separate per-array launches;
+  4096 samples: as a group replayed from a CUDA graph vs separate per-array accumulates;
 * stream: one 512-input x 2400-channel stream and three 64-input streams in 10 ms blocks with 9 s
   cross-power and 1 s total-power dumps over >= 100 s-equivalent; real-time factor and dump latency;
 * requant: the F-engine tail at the paper's sizes: 512 inputs x 1024 spectra of a 4096-channel PFB
@@ -81,9 +80,7 @@ def small(corr, synth, torch, reps=5, path="fp8tc"):
             e1.record()
             torch.cuda.synchronize()
             ms = e0.elapsed_time(e1) / reps
-        r_buf = ((2 * N + 31) // 32) * 32
-        samples = T * B * C
-        moved = samples * N + 2 * samples * r_buf  # input once, operand written and read back
+        moved = T * B * C * N  # the input, read once
         out[str(N)] = {"ms_per_step": ms, "tcmac_s": _useful(N, C, T * B) / (ms / 1e3) / 1e12,
                        "hbm_gbs": moved / (ms / 1e3) / 1e9, "hbm_frac": moved / (ms / 1e3) / 1e9 / hbm,
                        "real_time_factor": (T * B / 24000.0) / (ms / 1e3)}
