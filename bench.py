@@ -3,7 +3,7 @@
 
 One step = one pass of the whole hot path over one batch: 16 corr_accumulate calls of 8192-sample
 blocks (N = 512 inputs = 256 dual-pol stations, C = 128 channels, 4+4-bit Gaussian-plus-tone samples;
-unpack -> cross-multiply -> flush to int64 in one kernel, autos from the diagonal) followed by a dump of the cross
+unpack -> cross-multiply -> flush to int64, autos from the diagonal) followed by a dump of the cross
 and auto accumulators with reset (the integrate-and-dump step). Inputs (16 distinct blocks, 8 GiB)
 are resident in HBM before timing; they exceed L2, so no flush is needed between steps.
 
@@ -72,14 +72,10 @@ def profiled_traffic(kernel_files, profile_md, blocks_per_launch, tile_plan=None
 XENG_SOURCES = ["xeng_fp8tc.cu", "f8_common.cuh", "ptx_sm100.cuh"]
 PAIR_SOURCES = ["xeng_pair.cu", "f8_common.cuh", "ptx_sm100.cuh"]
 PREP_SOURCES = ["f8_prep.cu", "f8_common.cuh"]
-DIRECT_SOURCES = ["xeng_direct.cu", "xeng_direct.cuh", "f8_common.cuh", "ptx_sm100.cuh"]
-DIRECT = -1  # in place of a tile plan: the X-engine that builds its operand on the chip
 
 
 def xeng_profile(tile_plan):
     """(kernel name, its sources, its ncu summary in profiles/) for the X-engine of a tile plan."""
-    if tile_plan == DIRECT:
-        return "xeng_direct_kernel", DIRECT_SOURCES, "xeng_direct_512in_128ch_8192.md"
     if tile_plan == 3:
         return "f8_xeng_pair_kernel", PAIR_SOURCES, "f8_xeng_pair_512in_128ch_8192.md"
     return "f8_xeng_kernel", XENG_SOURCES, "f8_xeng_512in_128ch_8192.md"
@@ -98,7 +94,7 @@ def step_traffic(xeng_launches, prep_launches, blocks_per_launch, tile_plan, ms_
     alg = inp + xeng_launches * 2 * acc + acc
     _, x_src, x_md = xeng_profile(tile_plan)
     x = profiled_traffic(x_src, x_md, blocks_per_launch, tile_plan)
-    pr = profiled_traffic(PREP_SOURCES, "f8_prep_512in_128ch_8192.md", 1) if prep_launches else 0
+    pr = profiled_traffic(PREP_SOURCES, "f8_prep_512in_128ch_8192.md", 1)
     out = {"algorithmic_bytes": alg, "xeng_bytes_per_launch": x, "prep_bytes_per_launch": pr,
            "xeng_launches": xeng_launches, "prep_launches": prep_launches}
     if x is not None and pr is not None:
@@ -140,14 +136,10 @@ def issued_flops_per_sample(n_inputs, n_chans, plan=0):
     """MMA flops the tensor path issues per sample under a tile plan (M = 128 instructions of N = nb
     columns; plan 2 items carry a second half of nb1 = extra & 0xFFFF columns), split into wide
     (N = 256) and narrow (N <= 128) instructions. A plan-3 item is one M = 256, N = 256 instruction on
-    an SM pair: per SM the work of an M = 128, N = 256 one, counted as two wide instructions. The direct
-    X-engine issues the same on its 128 x 128-input tiles."""
+    an SM pair: per SM the work of an M = 128, N = 256 one, counted as two wide instructions."""
     from paper_1411_3751_gb300 import corr
 
     wide = narrow = 0
-    if plan == DIRECT:
-        nb = (n_inputs + 127) // 128
-        return 2 * 256 * 256 * n_chans * (nb * (nb + 1) // 2), 0
     if plan == 3:
         return 2 * 256 * 256 * n_chans * len(corr.corr_tile_plan(n_inputs, 3)), 0
     for _c0, _a0, nb, extra in corr.corr_tile_plan(n_inputs, plan):
@@ -468,11 +460,9 @@ def main():
     else:
         sm_share = 1.0
     traffic = None
-    # no operand builds in the step: the launches were the direct X-engine's
-    x_plan = DIRECT if args.path == "fp8tc" and unpack_n == 0 else xc_plan
-    x_kernel, x_src, x_md = xeng_profile(x_plan)
+    x_kernel, x_src, x_md = xeng_profile(xc_plan)
     if args.path == "fp8tc":
-        traffic = profiled_traffic(x_src, x_md, blocks_per_launch, x_plan)
+        traffic = profiled_traffic(x_src, x_md, blocks_per_launch, xc_plan)
     roof = {"bound": bound, "achieved": achieved, "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak,
             "traffic": traffic, "kernel": {"fp8tc": x_kernel, "fp8tc_fused": "f8_fused_kernel",
                                            "i8mma": "xeng_i8mma_kernel"}.get(args.path, "xeng_fp32_kernel"),
@@ -483,7 +473,7 @@ def main():
     if args.path.startswith("fp8tc") and probe:
         # the same kernel against the tcgen05 issue rate measured on this GPU just before the timed
         # region: the ideal launch time of the MMAs the tile plan issues, and the useful rate's share
-        wide, narrow = issued_flops_per_sample(N_IN, N_CHAN, x_plan)
+        wide, narrow = issued_flops_per_sample(N_IN, N_CHAN, xc_plan)
         samples = T_BLOCK * blocks_per_launch
         ideal_ms = (wide * samples / (probe["tflops_n256"] * 1e12) + narrow * samples / (probe["tflops_n128"] * 1e12)) * 1e3
         roof["issue_probe"] = dict(probe)
@@ -491,12 +481,12 @@ def main():
         roof["frac_issue"] = ideal_ms / per_launch_ms
         roof["frac_useful_of_issue_peak"] = achieved / probe["tflops_n256"]
     if args.path == "fp8tc":
-        roof["step_traffic"] = step_traffic(xeng_n / args.steps, unpack_n / args.steps, blocks_per_launch, x_plan,
+        roof["step_traffic"] = step_traffic(xeng_n / args.steps, unpack_n / args.steps, blocks_per_launch, xc_plan,
                                             ms_step, peaks.get("hbm_gbs") if peaks else None)
     if args.path == "fp8tc" and prep_sms > 0 and launches_per_batch > 1:
         # the step overlaps the operand build with the multiply, so the X-engine launches above ran on
-        # fewer SMs beside a build; the same blocks without the concurrent build, i.e. through the
-        # X-engine that builds its operand on the chip, on the whole GPU, after the step's timed region
+        # fewer SMs beside a build; the same kernel on the same launches with the passes in sequence
+        # (the whole GPU, nothing beside it), timed after the step's timed region
         xc.set_prep_sms(0)
         step()
         xc.sync()
@@ -510,12 +500,13 @@ def main():
         iso_launch = iso_ms / max(1, iso_n)
         # a few launches on the whole GPU with nothing beside them: against the burst peak
         iso_peak = 2.0 * peaks["bf16_tflops"] if peaks and "bf16_tflops" in peaks else peak
-        iso_flops = 8.0 * useful_cmacs(N_IN, N_CHAN, T_BLOCK) * N_BLOCKS * 5 / max(1, iso_n)
-        iso = {"launch_ms": iso_launch, "achieved": iso_flops / (iso_launch / 1e3) / 1e12, "peak": iso_peak,
-               "peak_source": "%s bf16 burst x 2 (whole GPU, nothing beside them)" % peak_src,
-               "what": "the same blocks without the concurrent build (xeng_direct_kernel on the whole GPU), 5 steps "
-                       "after the timed region"}
+        iso = {"launch_ms": iso_launch, "achieved": flops_launch / (iso_launch / 1e3) / 1e12, "peak": iso_peak,
+               "peak_source": "%s bf16 burst x 2 (20 launches on the whole GPU, nothing beside them)" % peak_src,
+               "what": "the same kernel and launches with the batch's two passes in sequence (whole GPU, no "
+                       "concurrent build), 5 steps after the timed region"}
         iso["frac"] = iso["achieved"] / iso_peak
+        if probe:
+            iso["frac_issue"] = ideal_ms / iso_launch
         roof["isolated"] = iso
 
     # end-to-end through the public API from pinned host buffers

@@ -65,11 +65,11 @@ typedef enum corr_path {
                           unpacked in shared memory inside the kernel; the integer tensor path */
   CORR_PATH_FP8TC = 3, /* tcgen05 kind::f8f6f4 (e4m3 operands, FP32 accumulation in TMEM). The default. A
                           TMA-fed persistent kernel builds the offset operand and the per-input sums
-                          on the chip, multiplies and adds the autos from its diagonal; samples
-                          that TMA does not take (blocks not 16-byte aligned, N C not a multiple of
-                          16) are copied to padded rows in device scratch first. Where a tile plan
-                          other than the default or a build schedule was asked for, an unpack pass
-                          writes the operand to device scratch for such a kernel (two passes). */
+                          on the chip, multiplies and adds the autos from its diagonal, where the
+                          rows allow TMA (16-byte aligned blocks; N a multiple of 16, or an array of
+                          at most 64 inputs whose channels pack into such rows) and neither a tile
+                          plan other than the default nor a build schedule was asked for; else an
+                          unpack pass writes the operand to device scratch for such a kernel. */
   CORR_PATH_FP8TC_FUSED = 4 /* same arithmetic with the unpack done inside the X-engine by converter
                                warps (no scratch; slower on this input layout, kept for comparison) */
 } corr_path;
@@ -81,7 +81,7 @@ typedef enum corr_fmt { CORR_FMT_CI64 = 0, CORR_FMT_CF32 = 1, CORR_FMT_CF32_NORM
 /* Kernel classes for corr_profile_read. */
 typedef enum corr_kernel {
   CORR_KERNEL_XENG = 0,   /* cross-multiply-accumulate (FP32 or tensor-core X-engine) */
-  CORR_KERNEL_UNPACK = 1, /* 4+4-bit -> e4m3 operand build, or the copy to padded rows (tensor path) */
+  CORR_KERNEL_UNPACK = 1, /* 4+4-bit -> e4m3 operand build (tensor path) */
   CORR_KERNEL_AUTOS = 2,  /* total-power kernel of corr_accumulate_autos */
   CORR_KERNEL_DUMP = 3,   /* dump / format conversion */
   CORR_KERNEL_COUNT = 4
@@ -120,10 +120,9 @@ int corr_get_path(const corr_ctx* ctx);
  * Arrays of at most 32 inputs run plans 0 and 1 as channel groups: one item multiplies channels
  * f .. f + g - 1 stacked in one 128-row tile (g = 2 for 17 to 32 inputs, 64 operand rows per channel;
  * g = 4 for at most 16 inputs, 32 rows), g times the useful products per operand byte of a
- * one-channel item. On a new context's own plan the tensor path does not run in two passes
- * (CORR_PATH_FP8TC) unless corr_set_prep_sms asks for a concurrent build.
+ * one-channel item (group launches do the same for such members).
  * Results are identical for every plan. Waits for the device (queued launches read the current work
- * list). CORR_ERR_ARG for another value. Group launches (corr_group_*) do not use the plan, and the
+ * list). CORR_ERR_ARG for another value. Group launches (corr_group_*) always use plan 0 or 1, and the
  * overlapped build (corr_set_prep_sms) runs with plans 0, 1 and 3. corr_get_tile_plan returns the
  * current plan (CORR_ERR_ARG for a NULL context).
  */
@@ -154,17 +153,16 @@ int corr_channel_group(int n_inputs, int plan);
 
 /*
  * corr_set_prep_sms - how corr_accumulate_batch schedules the two passes of the tensor path (Sec. 2.4's
- * unpack ahead of Sec. 2.5's cross-multiply); a positive value selects the two passes. With 0 < sms < SMs, a batch of more than one launch
+ * unpack ahead of Sec. 2.5's cross-multiply). With 0 < sms < SMs, a batch of more than one launch
  * builds the operand of launch j + 1 on `sms` SMs of its own (a TMA-fed build kernel on an internal
  * stream) while the X-engine multiplies launch j on the other SMs; with sms == SMs a small build CTA
  * runs beside the X-engine on every SM. The first build and the last multiply use the whole GPU. The
  * first such batch allocates a second operand buffer of the first one's size (see
  * corr_footprint_bytes); if that fails, or the shape does not suit the TMA build (n_inputs % 16 != 0,
  * n_inputs < 128, T < 128, tile plan 2, or a block not 16-byte aligned), batches run the two passes in
- * sequence. 0: no concurrent build (a two-pass tile plan runs its passes in sequence); -1 (the default) is the
- * automatic choice, 0, and corr_autotune times the overlapped schedules on the caller's blocks: with tile plan 3 at
- * 512 inputs the build on about 2/7 of the SMs balances the multiply on the others (+7% over the passes in
- * sequence measured; the default without two passes is a third faster than either); with the one-SM
+ * sequence. 0 runs them in sequence always; -1 (the default) is the automatic choice, 0, and
+ * corr_autotune times the overlapped schedules on the caller's blocks: with tile plan 3 at 512 inputs
+ * the build on about 2/7 of the SMs balances the multiply on the others (+7% measured); with the one-SM
  * plans the X-engine slows by more than the SMs it gives up. With plan 3, sms == SMs leaves the build
  * no room beside the X-engine CTAs (it then runs between them). Results are identical either way.
  * CORR_ERR_ARG outside -1 .. SMs.
@@ -175,10 +173,9 @@ int corr_get_prep_sms(const corr_ctx* ctx);
 
 /*
  * corr_set_batch_blocks - blocks of n_time_per_block samples that corr_accumulate_batch multiplies per
- * tensor-core launch (each launch reads and writes the int64 accumulators
- * once, Sec. 2.5's integration of groups of spectra; longer launches cost less per sample, on the two-pass path until
- * the operand the SMs share no longer fits in L2). 0 restores the default: corr_batch_blocks in two passes, else up to
- * 16 blocks (at most 16 for any setting then). Resizes the
+ * tensor-core launch of the two-pass tensor path (each launch reads and writes the int64 accumulators
+ * once, Sec. 2.5's integration of groups of spectra; longer launches cost less per sample until the
+ * operand the SMs share no longer fits in L2). 0 restores the default (corr_batch_blocks). Resizes the
  * operand buffers (K blocks each) after waiting for the device; CORR_ERR_OOM leaves the previous
  * size. CORR_ERR_ARG above the shape's cap (8 GiB of operand). corr_get_batch_blocks returns the value
  * in use. Results are identical for every value.
@@ -196,13 +193,13 @@ typedef struct corr_tuning {
 } corr_tuning;
 
 /*
- * corr_autotune - times the tensor path's schedules on the caller's own n_blocks device
+ * corr_autotune - times the two-pass tensor path's schedules on the caller's own n_blocks device
  * blocks (uint8[T][C][N] each; the batch of corr_accumulate_batch) and keeps the fastest for this
  * context: tile plan 0, 1, 2 or 3 x blocks per launch 1, 2, 4, 8 and the default (within n_blocks and
  * the operand cap) x SMs of a concurrent operand build (0, 1/5, 1/4, 2/7 and 1/3 of the SMs, and all of
  * them for plans 0 and 1; only for batches of several launches on shapes the build takes). Each schedule runs the batch once to warm up
  * and `reps` (1 .. 100) times timed with CUDA events on cuda_stream; the default schedule (the
- * shape's default plan, no concurrent build: the operand built on the chip) is timed first and another replaces the best only when at least 1% faster.
+ * shape's default plan) is timed first and another replaces the best only when at least 1% faster.
  * The results are cached in-process by (N, C, T, n_pol, SMs, n_blocks), and in the file named by
  * CORR_AUTOTUNE_CACHE if set; a cached
  * choice is applied without timing. Afterwards the accumulators and sample counts are zero (the trials
@@ -232,8 +229,8 @@ int corr_accumulate(corr_ctx* ctx, const void* d_samples, void* cuda_stream);
 /*
  * corr_accumulate_batch - add n_blocks blocks, d_blocks[b] each a device uint8[T][C][N], in order;
  * the result equals n_blocks corr_accumulate calls (the paper integrates 27 groups of spectra per
- * dump, Sec. 2.5). Consecutive blocks share tensor-core launches (up to 16; in two passes as many as keep the
- * operand of the channels in flight within L2: 4 blocks of 8192 samples at 512 inputs), so the int64 flush and the
+ * dump, Sec. 2.5). Consecutive blocks share tensor-core launches (as many as keep the operand of the
+ * channels in flight within L2: 4 blocks of 8192 samples at 512 inputs), so the int64 flush and the
  * launch cost are paid once per group of blocks. The pointer array is read during the call only.
  */
 int corr_accumulate_batch(corr_ctx* ctx, const void* const* d_blocks, int n_blocks, void* cuda_stream);
@@ -388,7 +385,7 @@ size_t corr_footprint_bytes(int n_inputs, int n_chans, int n_time_per_block, int
 /* Number of station pairs B_s = S (S + 1) / 2 for n_inputs / n_pol stations (0 if invalid). */
 long long corr_n_baselines(int n_inputs, int n_pol);
 
-/* Blocks that corr_accumulate_batch multiplies per tensor-core launch in two passes for this shape (host only; 0 if
+/* Blocks that corr_accumulate_batch multiplies per tensor-core launch for this shape (host only; 0 if
  * invalid): as many as keep the operand rows of the channels in flight (152 CTAs / tiles per channel)
  * within 256 MiB of L2, at most 65536 samples per launch (the exactness bound of the FP32 partial
  * sums) and an 8 GiB operand buffer, at least one. 4 for 512 inputs x 8192-sample blocks. */
@@ -463,19 +460,18 @@ int corr_probe_mma_rate(int n_mma, int n_cols, double* tflops, double* cycles_pe
  * Groups of sub-arrays. The paper's architecture scales by giving each GPU its own slice of the
  * problem (Sec. 2.5, Sec. 6: 109 channels per GPU, the same code from 32 to 512 inputs); a group
  * correlates several independent sub-arrays of different input and channel counts (sharing the
- * block length T and n_pol) on one GPU, each array's tensor-core launch behind the other's on one stream, which a
- * CUDA graph can replay.
+ * block length T and n_pol) on one GPU, with one persistent tensor-core launch covering the work
+ * of all of them, so small arrays do not each pay a partly empty wave.
  *
  * corr_group_create   n_arrays (1..8) sub-arrays; each is an ordinary corr_ctx (tensor path).
  * corr_group_member   the i-th sub-array's context, for corr_dump / corr_reset / counters; owned by
  *                     the group (do not destroy it).
  * corr_group_accumulate  one block per sub-array (d_samples[i] device uint8[T][C_i][N_i]); mode 0:
- *                     each sub-array through the X-engine that builds its operand on the chip, whatever
- *                     its tile plan; mode 1: as corr_accumulate on each context, tile plans and build
- *                     schedules included (for comparison). Results are identical.
- * corr_group_autotune times tile plans 0 and 1 of each sub-array on the given blocks, keeps the
- *                     faster one for the context (mode 1 and calls on the member;
- *                     cached in-process by (N, C, T, n_pol, SM count), and in the file
+ *                     ONE operand-build launch over all sub-arrays, then ONE grouped X-engine
+ *                     launch; mode 1: separate per-array launches (for comparison). Results are
+ *                     identical.
+ * corr_group_autotune times the two tile plans of each sub-array on the given blocks, keeps the
+ *                     faster one (cached in-process by (N, C, T, n_pol, SM count), and in the file
  *                     named by CORR_AUTOTUNE_CACHE if set), then zeroes the accumulators it touched.
  *                     Synchronizes the stream. plans_out (optional) receives the chosen plans.
  *                     A graph captured earlier is dropped (capture again afterwards).

@@ -81,13 +81,15 @@ __global__ void __launch_bounds__(AT_THREADS, 2) autos_tma_kernel(const __grid_c
   }
   // lane l addresses sample row l (+ 32 kk) of the warp's column (128-byte swizzle)
   const uint32_t src = ptx::smem_u32(smem) + (uint32_t)lane * 128 + (uint32_t)((warp ^ (lane & 7)) << 4);
-  for (long long w = blockIdx.x; w < a.n_items && !*abort_flag; w += gridDim.x) {
+  for (long long w = blockIdx.x; w < a.n_items; w += gridDim.x) {
+    if (__any_sync(0xffffffffu, *abort_flag != 0)) return;
     const int run = (int)(w / a.n_cols);
     const long long x = (w - run * a.n_cols) * 128;
     const int k1 = min(a.n_k, (run + 1) * a.kps);
     int acc[2] = {0, 0};  // inputs lane / 4 and lane / 4 + 8 of the column
     for (int k = run * a.kps; k < k1; ++k) {
-      if (!ptx::mbar_wait(&full[slot], phase, WAIT_NS)) {
+      // all lanes out of their waits: ldmatrix is for whole warps
+      if (!__all_sync(0xffffffffu, ptx::mbar_wait(&full[slot], phase, WAIT_NS))) {
         record_error(a.err, abort_flag, 8);
         return;
       }

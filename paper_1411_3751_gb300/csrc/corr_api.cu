@@ -13,7 +13,7 @@
 
 #include "corr_ctx.cuh"
 #include "corr_internal.cuh"
-#include "xeng_direct.cuh"
+#include "xeng_small.cuh"
 
 #include <cmath>
 
@@ -274,18 +274,18 @@ void free_ctx(corr_ctx* c) {
 
 XengArgs xeng_args(const corr_ctx* c, int buf, int T_run, int flush);  // buf: operand buffer d_op (0) or d_op2 (1)
 
-// How a block takes the tensor path: without an operand in HBM (launch_xeng_direct, launch_xeng_small) from its own
-// rows or from rows repacked to whole 16-byte columns, or in the two passes, which a tile plan or a build
-// schedule that was asked for keeps.
+// How a block takes the tensor path: arrays of at most 64 inputs without an operand in HBM (launch_xeng_small) from
+// their own rows or from rows repacked to whole 16-byte columns; others, and where a tile plan or a build
+// schedule was asked for, in the two passes.
 enum Route { ROUTE_TWO_PASS, ROUTE_DIRECT, ROUTE_REPACK };
 
 int repacked_inputs(const corr_ctx* c) { return (int)round_up(c->L.s.N, 16); }
 
 Route direct_route(const corr_ctx* c, const uint8_t* d_in) {
   const Shape& s = c->L.s;
-  if (xeng_small_supported(s, s.N, d_in) || xeng_direct_supported(s, s.N, d_in)) return ROUTE_DIRECT;
+  if (xeng_small_supported(s, s.N, d_in)) return ROUTE_DIRECT;
   const int Np = repacked_inputs(c);
-  if (c->d_op && (xeng_small_supported(s, Np, c->d_op) || xeng_direct_supported(s, Np, c->d_op))) return ROUTE_REPACK;
+  if (c->d_op && xeng_small_supported(s, Np, c->d_op)) return ROUTE_REPACK;
   return ROUTE_TWO_PASS;
 }
 
@@ -332,7 +332,7 @@ int accumulate_direct(corr_ctx* c, const uint8_t* const* blocks, int n, int T_bl
       }
     }
     const bool tb = timer_begin(c, CORR_KERNEL_XENG, st);
-    const cudaError_t e = c->L.s.N <= 64 ? launch_xeng_small(j, c->num_sms, st) : launch_xeng_direct(j, c->num_sms, st);
+    const cudaError_t e = launch_xeng_small(j, c->num_sms, st);
     timer_end(c, CORR_KERNEL_XENG, st, tb);
     if (e != cudaSuccess) return cuda_fail(e, "tensor x-engine launch");
     c->n_off += (long long)T_blk * j.n;
@@ -377,7 +377,7 @@ int enqueue_group(corr_ctx* const* ctx, int n, const uint8_t* const* in, cudaStr
       j.n = 1;
       j.flush_len = flush;
       j.err = c0->d_err;
-      e = c->L.s.N <= 64 ? launch_xeng_small(j, c->num_sms, st) : launch_xeng_direct(j, c->num_sms, st);
+      e = launch_xeng_small(j, c->num_sms, st);
     }
     if (e != cudaSuccess) return cuda_fail(e, "group x-engine launch");
   }
@@ -657,8 +657,7 @@ int accumulate_batch_chunks(corr_ctx* c, const uint8_t* const* blocks, int n, cu
   bool same = route != ROUTE_TWO_PASS;
   for (int b = 1; b < n && same; ++b) same = route_of(c, blocks[b]) == route;
   if (same)
-    // as many blocks per launch as fit it (512 inputs x 128 channels x 16 blocks of 8192 samples: 6.38 ms in one
-    // launch, 6.55 in four), or the number that was asked for
+    // as many blocks per launch as fit it (each launch reads and writes the sums once), or the number that was asked for
     return accumulate_direct(c, blocks, n, c->L.s.T, c->L.K_batch == c->K_default ? xd::MAX_BLOCKS : c->L.K_batch, route, st);
   // overlapped schedule when there are at least two chunks and the TMA build takes the shape (the wide
   // plan 2 fills both accumulators per item and is not overlapped)

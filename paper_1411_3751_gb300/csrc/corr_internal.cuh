@@ -197,13 +197,10 @@ int encode_input_tensor_map(CUtensorMap* map, const void* d_in, int N, int C, in
 int encode_raw_tensor_map(CUtensorMap* map, const void* d_in, long long row_bytes, int T, int box_bytes,
                           std::string* err);
 
-// X-engines that build their operand on the chip (xeng_direct.cuh): n blocks of one array, products into
-// cross and autos, offset sums into s1 and s2. launch_xeng_direct: SM pairs, more than 64 inputs;
-// launch_xeng_small: at most 64. xeng_*_supported: the shapes, row lengths ld (inputs a channel as
-// stored) and alignments each takes.
+// X-engine that builds its operand on the chip (xeng_small.cu), at most 64 inputs: n blocks of one array, products
+// into cross and autos, offset sums into s1 and s2. xeng_small_supported: the shapes, row lengths ld (inputs a
+// channel as stored) and alignments it takes.
 struct DirectJob;
-cudaError_t launch_xeng_direct(const DirectJob& j, int num_sms, cudaStream_t st);
-bool xeng_direct_supported(const Shape& s, int ld, const void* d_in);
 cudaError_t launch_xeng_small(const DirectJob& j, int num_sms, cudaStream_t st);
 bool xeng_small_supported(const Shape& s, int ld, const void* d_in);
 // in[rows][N] -> out[rows][Np], Np = N rounded up to a multiple of 16 (repack.cu).

@@ -92,11 +92,6 @@ __device__ __forceinline__ void tma_load_2d(void* smem_dst, const CUtensorMap* m
       : "memory");
 }
 
-// Bring `bytes` (a multiple of 16, from a 16-byte boundary) into L2.
-__device__ __forceinline__ void prefetch_l2(const void* g, uint32_t bytes) {
-  asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(g), "r"(bytes) : "memory");
-}
-
 // ---- ldmatrix -------------------------------------------------------------------------------
 // Two 16 x 16 byte matrices (rows at the addresses of lanes 0-15 and 16-31), transposed: lane l gets in
 // register 2 m + h the bytes of matrix m's column l / 4 + 8 h, rows 4 (l % 4) .. + 3.
@@ -224,13 +219,6 @@ __device__ __forceinline__ void cluster_sync() {
 __device__ __forceinline__ void mbar_arrive_cluster(uint32_t cluster_addr) {
   asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
 }
-// Arrive on an mbarrier of any CTA of the cluster without cluster-scope release: for writes that the arriving warp
-// has completed already by other means (tcgen05.wait::st, fence.proxy.async of its own shared memory). The release of
-// mbar_arrive_cluster waits for the SM's memory traffic in flight: measured 950 to 1590 clocks beside TMA loads, 40
-// without it.
-__device__ __forceinline__ void mbar_arrive_remote(uint32_t cluster_addr) {
-  asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
-}
 __device__ __forceinline__ void st_shared_cluster_u32(uint32_t cluster_addr, uint32_t v) {
   asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(cluster_addr), "r"(v) : "memory");
 }
@@ -255,16 +243,6 @@ __device__ __forceinline__ void tmem_relinquish_pair() {
 }
 __device__ __forceinline__ void tmem_dealloc_pair(uint32_t taddr, uint32_t ncols) {
   asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncols) : "memory");
-}
-// The same with A in TMEM: each CTA's 128 rows of A are lanes of its TMEM at a_tmem, K-major, four 8-bit
-// elements per 32-bit column (8 columns for K = 32).
-__device__ __forceinline__ void mma_f8f6f4_pair_ts(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc, uint32_t idesc,
-                                                   uint32_t accumulate) {
-  asm volatile(
-      "{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\n"
-      "tcgen05.mma.cta_group::2.kind::f8f6f4 [%0], [%1], %2, %3, p;\n}\n" ::"r"(d_tmem),
-      "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate)
-      : "memory");
 }
 // 2-SM MMA, issued by one thread of the pair's even CTA: A (M = 256) is 128 rows in each CTA's shared
 // memory and B (N) N / 2 rows in each, both at the descriptors' addresses; each CTA's TMEM at d_tmem

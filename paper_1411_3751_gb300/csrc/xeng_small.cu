@@ -30,7 +30,7 @@
 #include <cstring>
 
 #include "corr_internal.cuh"
-#include "xeng_direct.cuh"
+#include "xeng_small.cuh"
 
 namespace corr {
 namespace {
@@ -97,6 +97,7 @@ __global__ void __launch_bounds__(S_THREADS, 1) xeng_small_kernel(const __grid_c
     *abort_flag = 0;
     ptx::fence_mbar_init();
   }
+  __syncwarp();
   if (warp == 1) {
     ptx::tmem_alloc(tslot, TMEM_COLS);
     ptx::tmem_relinquish();
@@ -199,7 +200,8 @@ __global__ void __launch_bounds__(S_THREADS, 1) xeng_small_kernel(const __grid_c
     uint32_t rph = 0, oph = 0;
     int ahead = set;  // stages until the set's next one
     bool ok = true;
-    for (long long w = blockIdx.x; w < total && ok && !*abort_flag; w += gridDim.x) {
+    for (long long w = blockIdx.x; w < total && ok; w += gridDim.x) {
+      if (__any_sync(0xffffffffu, *abort_flag != 0)) break;
       const SmallItem it(args, w, n_pairs);
       // lane l addresses sample row l (+ 32 kk) of the 16-byte column of the quarter's inputs (128-byte swizzle)
       const int x0 = (int)(it.p * 2 * args.ub) & 15, col = ((x0 + h * args.ub) >> 4) + q, shift = (x0 + h * args.ub) & 15;
@@ -208,7 +210,9 @@ __global__ void __launch_bounds__(S_THREADS, 1) xeng_small_kernel(const __grid_c
       uint32_t sum[4] = {0u, 0u, 0u, 0u};  // Re, Im of inputs lane / 4 and lane / 4 + 8 of the quarter's 16
       for (int k = it.k0 + ahead; k < it.k1; k += S_SETS, p.next(args.n_kb, S_SETS)) {
         const int n_valid = args.T - p.kb * KT;  // samples of this stage (at most 128)
-        if (!ptx::mbar_wait(&raw_full[rs], rph, WAIT_NS) || !ptx::mbar_wait(&op_empty[os], oph ^ 1, WAIT_NS)) {
+        const bool got = ptx::mbar_wait(&raw_full[rs], rph, WAIT_NS) && ptx::mbar_wait(&op_empty[os], oph ^ 1, WAIT_NS);
+        // together again: the lanes leave their waits one by one, and ldmatrix and tcgen05.st are for whole warps
+        if (!__all_sync(0xffffffffu, got)) {
           record_error(err, abort_flag, 5);
           ok = false;
           break;
@@ -329,8 +333,8 @@ __global__ void __launch_bounds__(S_THREADS, 1) xeng_small_kernel(const __grid_c
           ptx::tmem_ld_32x32b_x32(t + 64 * j, v[0]);
           ptx::tmem_ld_32x32b_x32(t + 64 * j + 32, v[1]);
           ptx::tmem_ld_wait();
-          xd::combine_chunk<16, true>(v[0], im_lane, re[2 * j], im[2 * j]);
-          xd::combine_chunk<16, true>(v[1], im_lane, re[2 * j + 1], im[2 * j + 1]);
+          xd::combine_chunk(v[0], im_lane, re[2 * j], im[2 * j]);
+          xd::combine_chunk(v[1], im_lane, re[2 * j + 1], im[2 * j + 1]);
         }
         ptx::tc_fence_before();
         __syncwarp();
@@ -343,9 +347,11 @@ __global__ void __launch_bounds__(S_THREADS, 1) xeng_small_kernel(const __grid_c
       }
     }
   }
+  __syncwarp();  // the roles ran on single lanes: what follows is for whole warps (a second release of TMEM traps)
   ptx::tc_fence_before();
   __syncthreads();
   ptx::tc_fence_after();
+  __syncwarp();
   if (warp == 1) ptx::tmem_dealloc(tbase, TMEM_COLS);
 }
 
@@ -355,6 +361,52 @@ int small_group(int ld) {
   for (int g = 64 / ld; g >= 1; --g)
     if (g * ld + ((16 - (g * ld & -(g * ld))) & 15) <= 64) return g;
   return 0;
+}
+
+// Items' stages are divided where whole items leave SMs idle: the division of n_k stages that minimises waves x (stages
+// + overhead), `slots` items running at once.
+int direct_splits(long long items, int slots, int n_k, int overhead) {
+  int best = 1;
+  double best_t = 1e300;
+  for (int s = 1; s <= n_k && s <= 256; ++s) {
+    const int kps = (n_k + s - 1) / s;
+    if ((n_k + kps - 1) / kps != s) continue;  // the same division as a smaller s
+    const double waves = (double)((items * s + slots - 1) / slots);
+    const double t = waves * (kps + overhead + (s > 1 ? 1 : 0));
+    if (t < 0.97 * best_t) {
+      best = s;
+      best_t = t;
+    }
+    if (items * s >= 8LL * slots) break;
+  }
+  return best;
+}
+
+cudaError_t direct_args(const DirectJob& j, int box_bytes, xd::Args* a) {
+  std::memset(a, 0, sizeof(*a));
+  if (j.n > xd::MAX_BLOCKS) return cudaErrorInvalidValue;
+  for (int b = 0; b < j.n; ++b) {
+    std::string err;
+    if (encode_raw_tensor_map(&a->map[b], j.blocks[b], (long long)j.s.C * j.ld, j.T_blk, box_bytes, &err) != 0) {
+      set_last_error(err);
+      return cudaErrorInvalidValue;
+    }
+  }
+  a->cross = j.cross;
+  a->autos = j.autos;
+  a->s1 = j.s1;
+  a->s2 = j.s2;
+  a->Bs = j.s.Bs;
+  a->N = j.s.N;
+  a->ld = j.ld;
+  a->C = j.s.C;
+  a->npol = j.s.npol;
+  a->T = j.T_blk;
+  a->n_kb = (j.T_blk + KT - 1) / KT;
+  a->n_k = a->n_kb * j.n;
+  a->chunk_k = j.flush_len / KT;
+  a->err = j.err;
+  return cudaSuccess;
 }
 
 }  // namespace

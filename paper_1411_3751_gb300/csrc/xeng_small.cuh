@@ -1,6 +1,5 @@
-// Shared by the two X-engines that read the packed samples themselves (no operand in HBM): xeng_direct.cu
-// (SM pairs, more than 64 inputs) and xeng_small.cu (at most 64 inputs). Operand encoding and the sums
-// that undo it: f8_common.cuh.
+// Parts of the X-engine that reads the packed samples itself (no operand in HBM, xeng_small.cu). Operand encoding and
+// the sums that undo it: f8_common.cuh.
 #pragma once
 
 #include "f8_common.cuh"
@@ -22,35 +21,31 @@ struct Args {
   int n_kb, n_k;        // 128-sample stages of a block (the last one may be short) and of all blocks
   int chunk_k;          // stages per in-chip partial sum
   int splits, kps;      // the stages of an item are divided over `splits` items of kps stages
-  int n_units, g, ub;   // xeng_small: 64-input units, channels and bytes of one
-  int nb, n_tiles;      // xeng_direct: 128-input blocks, tiles of the triangle
+  int n_units, g, ub;   // 64-input units, channels and bytes of one
   long long n_items;
   int* err;
 };
 
-// One 32-column chunk of an accumulator (16 a-inputs: column 8 (k / 4) + k % 4 = Re a_k, + 4 = Im a_k; with HALVES
-// columns k and 16 + k) as complex products: the lanes holding Re c and Im c of one c-input are XOR apart, exchange half of their columns and own
-// 8 a-inputs each, the Re lane the even, the Im lane the odd ones. (With two polarisations a warp's access then
-// covers whole station pairs, 512 neighbouring bytes.) Combining first halves the words a thread holds, and leaves
-// registers for eight cells in flight.
-template <int XOR, bool HALVES = false>
+// One 32-column chunk of an accumulator (16 a-inputs: columns k and 16 + k = Re and Im of a_k) as complex products: the
+// lanes holding Re c and Im c of one c-input are 16 apart, exchange half of their columns and own 8 a-inputs
+// each, the Re lane the even, the Im lane the odd ones. Combining first halves the words a thread holds, and
+// leaves registers for eight cells in flight.
 __device__ __forceinline__ void combine_chunk(const uint32_t (&v)[32], bool im_lane, int (&re)[8], int (&im)[8]) {
 #pragma unroll
   for (int k = 0; k < 8; ++k) {
     // columns of the even input; the odd one's follow
-    const int jr = HALVES ? 2 * k : 8 * (k >> 1) + 2 * (k & 1), ji = jr + (HALVES ? 16 : 4);
+    const int jr = 2 * k, ji = jr + 16;
     const int own_r = f8::to_int(__uint_as_float(im_lane ? v[jr + 1] : v[jr]));
     const int own_i = f8::to_int(__uint_as_float(im_lane ? v[ji + 1] : v[ji]));
-    const int recv_r = f8::to_int(__shfl_xor_sync(0xffffffffu, __uint_as_float(im_lane ? v[jr] : v[jr + 1]), XOR));
-    const int recv_i = f8::to_int(__shfl_xor_sync(0xffffffffu, __uint_as_float(im_lane ? v[ji] : v[ji + 1]), XOR));
+    const int recv_r = f8::to_int(__shfl_xor_sync(0xffffffffu, __uint_as_float(im_lane ? v[jr] : v[jr + 1]), 16));
+    const int recv_i = f8::to_int(__shfl_xor_sync(0xffffffffu, __uint_as_float(im_lane ? v[ji] : v[ji + 1]), 16));
     // Re lane: own row Re c, partner Im c; Im lane the other way round
     re[k] = im_lane ? recv_r + own_i : own_r + recv_i;
     im[k] = im_lane ? recv_i - own_r : own_i - recv_r;
   }
 }
 
-// Cells as 32-bit offsets from the channel's first (a channel has less than 2^31 of them): pointers took twice the
-// registers and made the epilogue spill (512 inputs x 300 channels x 2048 samples 445 us, 359 with offsets).
+// Cells as 32-bit offsets from the channel's first (a channel has less than 2^31 of them): half the registers of pointers.
 template <bool ADD>
 __device__ __forceinline__ void add_cells(longlong2* __restrict__ base, const uint32_t (&cell)[8], uint32_t valid,
                                           const int (&re)[8], const int (&im)[8]) {
@@ -102,19 +97,6 @@ __device__ __forceinline__ void add_chunk(const int (&re)[8], const int (&im)[8]
   add_cells<ADD>(reinterpret_cast<longlong2*>(cross_f), cell, valid, re, im);
 }
 
-// The same for two polarisations where every cell of the chunk is stored and off the diagonal: no checks, and the
-// eight a-stations' cells at simple steps (b grows by sa + 1 from station to station).
-template <bool ADD>
-__device__ __forceinline__ void add_chunk_full(const int (&re)[8], const int (&im)[8], bool im_lane, int c, int a_base,
-                                               long long* __restrict__ cross_f) {
-  const unsigned sa = (unsigned)a_base >> 1;
-  const unsigned p = 4 * (sa * (sa + 1) / 2 + ((unsigned)c >> 1)) + (unsigned)(c & 1) + (im_lane ? 2u : 0u);
-  uint32_t cell[8];
-#pragma unroll
-  for (int k = 0; k < 8; ++k) cell[k] = p + 4 * (k * sa + (unsigned)(k * (k + 1) / 2));
-  add_cells<ADD>(reinterpret_cast<longlong2*>(cross_f), cell, 0xFFu, re, im);
-}
-
 // Stage k of an item's blocks: block k / n_kb, sample 128 (k % n_kb).
 struct StagePos {
   int blk, kb;
@@ -145,11 +127,5 @@ struct DirectJob {
   long long *cross, *autos, *s1, *s2;
   int* err;
 };
-
-// Items' stages are divided by direct_splits() where whole items leave SMs idle: the division of n_k stages that
-// minimises waves x (stages + overhead), `slots` items running at once.
-int direct_splits(long long items, int slots, int n_k, int overhead);
-// The kernels' common arguments; boxes of box_bytes (64 or 128, swizzled as wide) x 128 samples.
-cudaError_t direct_args(const DirectJob& j, int box_bytes, xd::Args* a);
 
 }  // namespace corr

@@ -1,6 +1,6 @@
-"""The X-engines that build their operand on the chip (a default context whose rows allow TMA): channel
-grouping of small arrays, tile edges of large ones, short and long rings, several items a CTA, divided
-time ranges, in-chip flushes, more blocks than one launch takes, and the routes that keep the two passes.
+"""The default tensor path: the X-engine that builds its operand on the chip (at most 64 inputs: channel grouping,
+short and long rings, several items a CTA, divided time ranges, in-chip flushes, more blocks than one launch takes,
+rows that TMA does not take) and the two passes above, on the same shapes and options.
 Everything is compared exactly, with the oracle or, at sizes it is slow at, with the int8 path."""
 import numpy as np
 import pytest
@@ -58,7 +58,7 @@ def _check(env, host, npol, **kw):
 
 
 # N: every packing of channels into 64-input units, unit strides of 48 and 64 bytes, the change of kernel at 64,
-# tiles of 128 inputs with 16 .. 128 inputs in the last one. C: one unit, a unit without its pair, a partial last
+# blocks of 128 inputs with 16 .. 128 inputs in the last one. C: one unit, a unit without its pair, a partial last
 # group. T: less than a stage, a stage, a stage and a bit.
 @pytest.mark.parametrize("N,C,npol", [(1, 64, 1), (1, 80, 1), (2, 40, 2), (4, 4, 2), (6, 8, 2), (8, 2, 1), (12, 12, 2),
                                       (16, 1, 2), (16, 9, 2), (24, 3, 2), (24, 2, 1), (32, 1, 2), (32, 5, 2), (48, 1, 2),
