@@ -148,3 +148,17 @@ def test_requantize_segments(env, N, T, F, chan0, C):
     x = np.random.default_rng(N + T).integers(-1 << 17, 1 << 17, (N, T, F, 2), dtype=np.int32)
     got = corr.requantize(torch.from_numpy(x).cuda(), chan0, C, gain=2.0 ** -14).cpu().numpy()
     assert np.array_equal(got, oracle.requantize(x, chan0, C, gain=2.0 ** -14))
+
+
+# every tap count that has its own kernel, and the loop beyond them; one and an odd number of spectra
+@pytest.mark.parametrize("n_taps", [1, 2, 3, 4, 5, 6, 7, 8, 9, 17])
+@pytest.mark.parametrize("n_spectra", [1, 5])
+def test_pfb_tap_counts(env, n_taps, n_spectra):
+    """Within 4 log2(8192) FP32 roundings of each spectrum's L2 norm of the float64 oracle, as in the filterbank's tests."""
+    corr, _, torch = env
+    M = 8192
+    adc = np.random.default_rng(n_taps).integers(-128, 128, (3, (n_spectra + n_taps - 1) * M), dtype=np.int8)
+    X = corr.pfb(torch.from_numpy(adc).cuda(), n_taps=n_taps).cpu().numpy()
+    want, y = oracle.pfb(adc, M, n_taps), oracle.pfb_fir(adc, M, n_taps)
+    tol = 4 * 13 * 2.0 ** -24 * 2.0 ** -13 * np.sqrt(M) * np.sqrt((y.astype(np.float64) ** 2).sum(-1))
+    assert np.all(np.abs(X[..., 0] + 1j * X[..., 1] - want).max(axis=-1) <= tol)
