@@ -65,11 +65,12 @@ typedef enum corr_path {
                           unpacked in shared memory inside the kernel; the integer tensor path */
   CORR_PATH_FP8TC = 3, /* tcgen05 kind::f8f6f4 (e4m3 operands, FP32 accumulation in TMEM). The default. A
                           TMA-fed persistent kernel builds the offset operand and the per-input sums
-                          on the chip, multiplies and adds the autos from its diagonal, where the
-                          rows allow TMA (16-byte aligned blocks; N a multiple of 16, or an array of
-                          at most 64 inputs whose channels pack into such rows) and neither a tile
-                          plan other than the default nor a build schedule was asked for; else an
-                          unpack pass writes the operand to device scratch for such a kernel. */
+                          on the chip, multiplies and adds the autos from its diagonal for arrays of
+                          at most 64 inputs (samples that TMA does not take, i.e. blocks not 16-byte
+                          aligned or N C not a multiple of 16, are copied to padded rows in device
+                          scratch first). Larger arrays, and contexts where a tile plan other than
+                          the default or a build schedule was asked for, take two passes: an unpack
+                          pass writes the operand to device scratch for such a kernel. */
   CORR_PATH_FP8TC_FUSED = 4 /* same arithmetic with the unpack done inside the X-engine by converter
                                warps (no scratch; slower on this input layout, kept for comparison) */
 } corr_path;
@@ -81,7 +82,7 @@ typedef enum corr_fmt { CORR_FMT_CI64 = 0, CORR_FMT_CF32 = 1, CORR_FMT_CF32_NORM
 /* Kernel classes for corr_profile_read. */
 typedef enum corr_kernel {
   CORR_KERNEL_XENG = 0,   /* cross-multiply-accumulate (FP32 or tensor-core X-engine) */
-  CORR_KERNEL_UNPACK = 1, /* 4+4-bit -> e4m3 operand build (tensor path) */
+  CORR_KERNEL_UNPACK = 1, /* 4+4-bit -> e4m3 operand build, or the copy to padded rows (tensor path) */
   CORR_KERNEL_AUTOS = 2,  /* total-power kernel of corr_accumulate_autos */
   CORR_KERNEL_DUMP = 3,   /* dump / format conversion */
   CORR_KERNEL_COUNT = 4
@@ -120,10 +121,10 @@ int corr_get_path(const corr_ctx* ctx);
  * Arrays of at most 32 inputs run plans 0 and 1 as channel groups: one item multiplies channels
  * f .. f + g - 1 stacked in one 128-row tile (g = 2 for 17 to 32 inputs, 64 operand rows per channel;
  * g = 4 for at most 16 inputs, 32 rows), g times the useful products per operand byte of a
- * one-channel item (group launches do the same for such members).
+ * one-channel item. Arrays of at most 64 inputs run in two passes, i.e. with a plan at all, only when the plan is
+ * not the default or corr_set_prep_sms asks for a concurrent build (CORR_PATH_FP8TC).
  * Results are identical for every plan. Waits for the device (queued launches read the current work
- * list). CORR_ERR_ARG for another value. Group launches (corr_group_*) always use plan 0 or 1, and the
- * overlapped build (corr_set_prep_sms) runs with plans 0, 1 and 3. corr_get_tile_plan returns the
+ * list). CORR_ERR_ARG for another value. The overlapped build (corr_set_prep_sms) runs with plans 0, 1 and 3. corr_get_tile_plan returns the
  * current plan (CORR_ERR_ARG for a NULL context).
  */
 int corr_set_tile_plan(corr_ctx* ctx, int plan);
@@ -175,7 +176,8 @@ int corr_get_prep_sms(const corr_ctx* ctx);
  * corr_set_batch_blocks - blocks of n_time_per_block samples that corr_accumulate_batch multiplies per
  * tensor-core launch of the two-pass tensor path (each launch reads and writes the int64 accumulators
  * once, Sec. 2.5's integration of groups of spectra; longer launches cost less per sample until the
- * operand the SMs share no longer fits in L2). 0 restores the default (corr_batch_blocks). Resizes the
+ * operand the SMs share no longer fits in L2). 0 restores the default (corr_batch_blocks; without an operand in HBM,
+ * i.e. up to 64 inputs, up to 16 blocks, which is also the most of any setting then). Resizes the
  * operand buffers (K blocks each) after waiting for the device; CORR_ERR_OOM leaves the previous
  * size. CORR_ERR_ARG above the shape's cap (8 GiB of operand). corr_get_batch_blocks returns the value
  * in use. Results are identical for every value.
@@ -229,8 +231,8 @@ int corr_accumulate(corr_ctx* ctx, const void* d_samples, void* cuda_stream);
 /*
  * corr_accumulate_batch - add n_blocks blocks, d_blocks[b] each a device uint8[T][C][N], in order;
  * the result equals n_blocks corr_accumulate calls (the paper integrates 27 groups of spectra per
- * dump, Sec. 2.5). Consecutive blocks share tensor-core launches (as many as keep the operand of the
- * channels in flight within L2: 4 blocks of 8192 samples at 512 inputs), so the int64 flush and the
+ * dump, Sec. 2.5). Consecutive blocks share tensor-core launches (up to 16 for at most 64 inputs, else as many as keep
+ * the operand of the channels in flight within L2: 4 blocks of 8192 samples at 512 inputs), so the int64 flush and the
  * launch cost are paid once per group of blocks. The pointer array is read during the call only.
  */
 int corr_accumulate_batch(corr_ctx* ctx, const void* const* d_blocks, int n_blocks, void* cuda_stream);
@@ -460,16 +462,16 @@ int corr_probe_mma_rate(int n_mma, int n_cols, double* tflops, double* cycles_pe
  * Groups of sub-arrays. The paper's architecture scales by giving each GPU its own slice of the
  * problem (Sec. 2.5, Sec. 6: 109 channels per GPU, the same code from 32 to 512 inputs); a group
  * correlates several independent sub-arrays of different input and channel counts (sharing the
- * block length T and n_pol) on one GPU, with one persistent tensor-core launch covering the work
- * of all of them, so small arrays do not each pay a partly empty wave.
+ * block length T and n_pol) on one GPU, each array's kernels behind the other's on one stream, which a CUDA graph
+ * can replay.
  *
  * corr_group_create   n_arrays (1..8) sub-arrays; each is an ordinary corr_ctx (tensor path).
  * corr_group_member   the i-th sub-array's context, for corr_dump / corr_reset / counters; owned by
  *                     the group (do not destroy it).
  * corr_group_accumulate  one block per sub-array (d_samples[i] device uint8[T][C_i][N_i]); mode 0:
- *                     ONE operand-build launch over all sub-arrays, then ONE grouped X-engine
- *                     launch; mode 1: separate per-array launches (for comparison). Results are
- *                     identical.
+ *                     all operand work first, then all X-engines; sub-arrays of at most 64 inputs
+ *                     without an operand in HBM, whatever their tile plan; mode 1: as corr_accumulate
+ *                     on each context (for comparison). Results are identical.
  * corr_group_autotune times the two tile plans of each sub-array on the given blocks, keeps the
  *                     faster one (cached in-process by (N, C, T, n_pol, SM count), and in the file
  *                     named by CORR_AUTOTUNE_CACHE if set), then zeroes the accumulators it touched.

@@ -341,9 +341,11 @@ int accumulate_direct(corr_ctx* c, const uint8_t* const* blocks, int n, int T_bl
   return CORR_OK;
 }
 
-// One block of every array: the operand work first (repacked rows; where an array takes neither direct route the
-// two-pass build), then the X-engines one behind the other. Counts nothing: a captured launch is counted when
-// it is replayed. Timed and its waits reported on the first array, flushed by its period.
+// One block of every array: the operand work first (repacked rows, or the two-pass build), then the X-engines one
+// behind the other, at most 64 inputs without an operand in HBM, the others on their tile plans. Counts nothing:
+// a captured launch is counted when it is replayed. Timed and its waits reported on the first array, flushed by
+// its period. (One merged launch of all members' items on the one-SM kernel: five arrays of 32 to 512 inputs x 4096
+// samples with their dumps 1563 us, so 1280.)
 int enqueue_group(corr_ctx* const* ctx, int n, const uint8_t* const* in, cudaStream_t st) {
   corr_ctx* c0 = ctx[0];
   const int flush = flush_for(c0, CORR_PATH_FP8TC);
