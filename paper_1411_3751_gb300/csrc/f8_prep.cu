@@ -23,8 +23,13 @@ using namespace f8;
 //    int64 sums with one atomic per input and block.
 constexpr int PREP_ROWS_PER_THREAD_MAX = 2048;
 
+// VEC: the loads' width (load_width). 1 = rows of any length or alignment: the 16 bytes of a unit are the five aligned
+// words around them, shifted together (single bytes where those would leave the block), four samples in flight.
+// 131 inputs x 300 channels x 4096 samples: 229 us by single bytes, 130 so (175 with eight samples in flight);
+// 202 inputs 329 and 175. (Widths as an argument and not a template cost the 16- and 8-byte builds 4 and 6%.)
+template <int VEC>
 __global__ void __launch_bounds__(256) f8_prep_kernel(const uint8_t* __restrict__ in, int N, int C, int T, int T_run,
-                                                      int T_stride, int t_base, int R, int rows_per_split, int vec,
+                                                      int T_stride, int t_base, int R, int rows_per_split,
                                                       uint8_t* __restrict__ op, long long* __restrict__ s1,
                                                       long long* __restrict__ s2) {
   const long long bx = blockIdx.x;  // 8 units
@@ -44,8 +49,9 @@ __global__ void __launch_bounds__(256) f8_prep_kernel(const uint8_t* __restrict_
   uint32_t sre[4][2] = {{0u, 0u}, {0u, 0u}, {0u, 0u}, {0u, 0u}};
   uint32_t sim[4][2] = {{0u, 0u}, {0u, 0u}, {0u, 0u}, {0u, 0u}};
   if (unit_ok) {
-    // 8 samples per thread per iteration, all loads issued before any conversion
-    constexpr int U = 8;
+    // 8 samples per thread per iteration (4 if ANY), all loads issued before any conversion
+    constexpr int U = VEC == 1 ? 4 : 8;
+    const uint8_t* end = in + (size_t)T * C * N;
     for (int t0 = t_begin + 4 * warp + tl; t0 < t_end; t0 += 32 * U) {
       uint4 w[U];
       bool live[U];
@@ -56,21 +62,31 @@ __global__ void __launch_bounds__(256) f8_prep_kernel(const uint8_t* __restrict_
         live[u] = t < t_end && t < T && nv > 0;
         if (live[u]) {
           const uint8_t* src = in + ((size_t)t * C + f) * N + n0;
-          if (vec == 16) {
+          if (VEC == 1) {  // bytes behind the last input are masked by expand16
+            const uint32_t sh = (uint32_t)(reinterpret_cast<uintptr_t>(src) & 3);
+            const uint8_t* q = src - sh;
+            uint32_t x[5] = {0u, 0u, 0u, 0u, 0u};
+            if (q >= in && q + 20 <= end) {
+#pragma unroll
+              for (int k = 0; k < 5; ++k) x[k] = __ldg(reinterpret_cast<const uint32_t*>(q) + k);
+#pragma unroll
+              for (int k = 0; k < 4; ++k) x[k] = __funnelshift_r(x[k], x[k + 1], 8 * sh);
+            } else {
+#pragma unroll
+              for (int k = 0; k < 16; ++k)
+                if (n0 + k < N) x[k >> 2] |= (uint32_t)src[k] << (8 * (k & 3));
+            }
+            w[u] = make_uint4(x[0], x[1], x[2], x[3]);
+          } else if (VEC == 16) {
             w[u] = __ldg(reinterpret_cast<const uint4*>(src));
-          } else if (vec == 8) {  // N % 8 == 0: nv is 8 or >= 16
+          } else if (VEC == 8) {  // N % 8 == 0: nv is 8 or >= 16
             const uint2 lo = __ldg(reinterpret_cast<const uint2*>(src));
             const uint2 hi = nv > 8 ? __ldg(reinterpret_cast<const uint2*>(src) + 1) : make_uint2(0u, 0u);
             w[u] = make_uint4(lo.x, lo.y, hi.x, hi.y);
-          } else if (vec == 4) {  // N % 4 == 0: nv is a multiple of 4
+          } else {  // N % 4 == 0: nv is a multiple of 4
             const uint32_t* s4 = reinterpret_cast<const uint32_t*>(src);
             w[u] = make_uint4(__ldg(s4), nv > 4 ? __ldg(s4 + 1) : 0u, nv > 8 ? __ldg(s4 + 2) : 0u,
                               nv > 12 ? __ldg(s4 + 3) : 0u);
-          } else {
-            uint32_t x[4] = {0u, 0u, 0u, 0u};
-            for (int k = 0; k < 16; ++k)
-              if (n0 + k < N) x[k >> 2] |= (uint32_t)src[k] << (8 * (k & 3));
-            w[u] = make_uint4(x[0], x[1], x[2], x[3]);
           }
         }
       }
@@ -177,8 +193,11 @@ cudaError_t launch_f8_prep(const Shape& s, const uint8_t* d_in, int T_blk, int T
   prep_geometry(s, T_run, R, &gx, &split, &rows);
   dim3 grid((unsigned)gx, 1, split);
   const int vec = load_width(s.N, d_in);
-  f8_prep_kernel<<<grid, 256, 0, st>>>(d_in, s.N, s.C, T_blk, T_run, T_stride, t_base, R, rows, vec, d_op, d_s1,
-                                       d_s2);
+  const auto kernel = vec == 16  ? f8_prep_kernel<16>
+                      : vec == 8 ? f8_prep_kernel<8>
+                      : vec == 4 ? f8_prep_kernel<4>
+                                 : f8_prep_kernel<1>;
+  kernel<<<grid, 256, 0, st>>>(d_in, s.N, s.C, T_blk, T_run, T_stride, t_base, R, rows, d_op, d_s1, d_s2);
   return cudaGetLastError();
 }
 
