@@ -272,7 +272,9 @@ void free_ctx(corr_ctx* c) {
   delete c;
 }
 
-XengArgs xeng_args(const corr_ctx* c, int buf, int T_run, int flush);  // buf: operand buffer d_op (0) or d_op2 (1)
+// The context's two-pass launch on its own work list; buf: operand buffer d_op (0) or d_op2 (1).
+XengArgs xeng_args(const corr_ctx* c, int buf, int T_run, int flush);
+XengArgs xeng_args(const corr_ctx* c, int plan, int buf, int T_run, int flush, const WorkItem* items, long long n_items);
 
 // How a block takes the tensor path: arrays of at most 64 inputs without an operand in HBM (launch_xeng_small) from
 // their own rows or from rows repacked to whole 16-byte columns; others, and where a tile plan or a build
@@ -342,11 +344,11 @@ int accumulate_direct(corr_ctx* c, const uint8_t* const* blocks, int n, int T_bl
 }
 
 // One block of every array: the operand work first (repacked rows, or the two-pass build), then the X-engines one
-// behind the other, at most 64 inputs without an operand in HBM, the others on their tile plans. Counts nothing:
-// a captured launch is counted when it is replayed. Timed and its waits reported on the first array, flushed by
-// its period. (One merged launch of all members' items on the one-SM kernel: five arrays of 32 to 512 inputs x 4096
+// behind the other, at most 64 inputs without an operand in HBM, the others on the group's own lists. Counts
+// nothing: a captured launch is counted when it is replayed. Timed and its waits reported on the first array,
+// flushed by its period. (One merged launch of all members' items on the one-SM kernel: five arrays of 32 to 512 inputs x 4096
 // samples with their dumps 1563 us, so 1280.)
-int enqueue_group(corr_ctx* const* ctx, int n, const uint8_t* const* in, cudaStream_t st) {
+int enqueue_group(corr_ctx* const* ctx, int n, const GroupWork& work, const uint8_t* const* in, cudaStream_t st) {
   corr_ctx* c0 = ctx[0];
   const int flush = flush_for(c0, CORR_PATH_FP8TC);
   bool tb = timer_begin(c0, CORR_KERNEL_UNPACK, st);
@@ -369,7 +371,8 @@ int enqueue_group(corr_ctx* const* ctx, int n, const uint8_t* const* in, cudaStr
     const Route route = direct_route(c, in[i]);
     cudaError_t e;
     if (route == ROUTE_TWO_PASS) {
-      XengArgs a = xeng_args(c, 0, c->L.T_pad, flush);
+      const GroupWork::List& l = work.list[i];
+      XengArgs a = xeng_args(c, l.plan, 0, c->L.T_pad, flush, work.d_items + l.first, l.n);
       a.err = c0->d_err;
       e = launch_f8_xeng(a, c->num_sms, st);
     } else {
@@ -431,21 +434,26 @@ int accumulate_device(corr_ctx* c, const uint8_t* d_in, int T_blk, cudaStream_t 
 }
 
 
-// Tile plan of the tensor paths: the tile list (fused path) and the channel-major work list
-// (two-pass path) for plan 0, 1 or 2 (see f8_tile_plan).
+// Channel-major work list of the two-pass path on a tile plan (see f8_tile_plan).
+std::vector<WorkItem> work_items(const Layout& L, int plan) {
+  std::vector<WorkItem> items;
+  if (const int g = plan < 2 ? channel_group(L) : 0; g > 0) {  // channel groups
+    for (int f = 0; f < L.s.C; f += g) items.push_back(WorkItem{0, f, 0, 0, 128, 0});
+    return items;
+  }
+  const std::vector<F8Tile> tiles = f8_tile_plan(L.s.N, L.R, plan);
+  items.reserve((size_t)L.s.C * tiles.size());
+  for (int f = 0; f < L.s.C; ++f)
+    for (const F8Tile& t : tiles) items.push_back(WorkItem{0, f, t.c0, t.a0, t.nb, t.pad});
+  return items;
+}
+
+// Tile plan of the tensor paths: the tile list (fused path) and the work list (two-pass path).
 
 int set_tile_plan(corr_ctx* c, int plan) {
   // the fused path has no wide mode: it keeps plan 0 under plan 2
   const std::vector<F8Tile> t8 = f8_tile_plan(c->L.s.N, c->L.R, plan >= 2 ? 0 : plan);
-  const std::vector<F8Tile> tw = plan >= 2 ? f8_tile_plan(c->L.s.N, c->L.R, plan) : t8;
-  std::vector<WorkItem> items;
-  items.reserve((size_t)c->L.s.C * tw.size());
-  if (channel_group(c->L) > 0 && plan < 2) {  // channel groups (uses_channel_groups)
-    for (int f = 0; f < c->L.s.C; f += channel_group(c->L)) items.push_back(WorkItem{0, f, 0, 0, 128, 0});
-  } else {
-    for (int f = 0; f < c->L.s.C; ++f)
-      for (const F8Tile& t : tw) items.push_back(WorkItem{0, f, t.c0, t.a0, t.nb, t.pad});
-  }
+  const std::vector<WorkItem> items = work_items(c->L, plan);
   F8Tile* d_t = nullptr;
   WorkItem* d_i = nullptr;
   if (cudaMalloc(&d_t, t8.size() * sizeof(F8Tile)) != cudaSuccess ||
@@ -481,28 +489,30 @@ int default_tile_plan(int N) {
 
 int channel_group(const Layout& L) { return L.R_buf == 64 ? 2 : (L.R_buf == 32 ? 4 : 0); }
 
-bool uses_channel_groups(const corr_ctx* c) { return channel_group(c->L) > 0 && c->tile_plan < 2; }
-
-XengArgs xeng_args(const corr_ctx* c, int buf, int T_run, int flush) {
+XengArgs xeng_args(const corr_ctx* c, int plan, int buf, int T_run, int flush, const WorkItem* items, long long n_items) {
   XengArgs a;
   std::memset(&a, 0, sizeof(a));
-  const bool cp = uses_channel_groups(c);
-  a.a[0].tmap = cp ? (buf ? c->tmap2_cp : c->tmap_cp) : (buf ? c->tmap2 : c->tmap);
+  const int cgroup = plan < 2 ? channel_group(c->L) : 0;
+  a.a[0].tmap = cgroup ? (buf ? c->tmap2_cp : c->tmap_cp) : (buf ? c->tmap2 : c->tmap);
   a.a[0].C = c->L.s.C;
-  a.a[0].cgroup = cp ? channel_group(c->L) : 0;
+  a.a[0].cgroup = cgroup;
   a.a[0].cross = c->d_cross;
   a.a[0].autos = c->d_autos;
   a.a[0].Bs = c->L.s.Bs;
   a.a[0].N = c->L.s.N;
   a.a[0].npol = c->L.s.npol;
-  a.items = c->d_items;
-  a.n_items = c->n_items;
+  a.items = items;
+  a.n_items = n_items;
   a.T_run = T_run;
   a.flush_len = flush;
   a.err = c->d_err;
-  a.wide = c->tile_plan == 2 ? 1 : 0;
-  a.pair = c->tile_plan == 3 ? 1 : 0;
+  a.wide = plan == 2 ? 1 : 0;
+  a.pair = plan == 3 ? 1 : 0;
   return a;
+}
+
+XengArgs xeng_args(const corr_ctx* c, int buf, int T_run, int flush) {
+  return xeng_args(c, c->tile_plan, buf, T_run, flush, c->d_items, c->n_items);
 }
 
 // The two-pass tensor path's operand scratch and its TMA tensor map.

@@ -104,17 +104,25 @@ int default_tile_plan(int N);
 // Channels per item of an array's channel groups: 2 for 64 operand rows per channel (17 .. 32 inputs),
 // 4 for 32 rows (at most 16 inputs), else 0.
 int channel_group(const Layout& L);
-// The two-pass X-engine of this context takes channel-group items: channel_group(L) > 0 and a one-SM
-// tile plan (0 or 1).
-bool uses_channel_groups(const corr_ctx* c);
 // blocks per tensor-core launch of batches (reallocates the operand buffers once the device is idle)
 int set_batch_blocks(corr_ctx* c, int K);
 // largest blocks per launch the operand buffer cap allows for this shape
 int max_batch_blocks(const corr_ctx* c);
 // n device blocks through the two-pass tensor path (batch schedule of the context's settings)
 int accumulate_batch_chunks(corr_ctx* c, const uint8_t* const* blocks, int n, cudaStream_t st);
-// one block in[i] of each of n arrays through the tensor path (no counting; any tile plan)
-int enqueue_group(corr_ctx* const* ctx, int n, const uint8_t* const* in, cudaStream_t st);
+// Channel-major work list of the two-pass path on a tile plan.
+std::vector<WorkItem> work_items(const Layout& L, int plan);
+// Work lists of a group's arrays, owned by the group: a captured launch keeps reading them, whatever becomes of the
+// arrays' own lists (corr_set_tile_plan and corr_autotune replace those).
+struct GroupWork {
+  WorkItem* d_items;  // list i: d_items[first .. first + n - 1], of tile plan `plan`
+  struct List {
+    long long first, n;
+    int plan;
+  } list[kMaxGroupArrays];
+};
+// one block in[i] of each of n arrays through the tensor path (no counting)
+int enqueue_group(corr_ctx* const* ctx, int n, const GroupWork& work, const uint8_t* const* in, cudaStream_t st);
 // T_blk samples of a device block [T_blk][C][N] through the context's current path
 int accumulate_device(corr_ctx* c, const uint8_t* d_in, int T_blk, cudaStream_t st);
 

@@ -20,6 +20,7 @@ using namespace corr::host;
 struct corr_group {
   int n;
   corr_ctx* ctx[kMaxGroupArrays];
+  GroupWork work;
   cudaGraphExec_t graph;
   int T;
 };
@@ -58,13 +59,38 @@ void tune_store(const std::tuple<int, int, int, int, int>& k, int plan) {
   std::fclose(fh);
 }
 
+// The arrays' work lists on their tile plans, one behind the other; replaces the group's lists, so a graph that
+// reads these has to be dropped first.
+int group_build_work(corr_group* g) {
+  GroupWork w{};
+  std::vector<WorkItem> items;
+  for (int i = 0; i < g->n; ++i) {
+    const corr_ctx* c = g->ctx[i];
+    const std::vector<WorkItem> own = work_items(c->L, c->tile_plan);
+    w.list[i] = GroupWork::List{(long long)items.size(), (long long)own.size(), c->tile_plan};
+    items.insert(items.end(), own.begin(), own.end());
+  }
+  if (cudaMalloc(&w.d_items, items.size() * sizeof(WorkItem)) != cudaSuccess) {
+    cudaGetLastError();
+    return fail(CORR_ERR_OOM, "group work list allocation failed");
+  }
+  const cudaError_t e = cudaMemcpy(w.d_items, items.data(), items.size() * sizeof(WorkItem), cudaMemcpyHostToDevice);
+  if (e != cudaSuccess) {
+    cudaFree(w.d_items);
+    return cuda_fail(e, "group work list upload");
+  }
+  cudaFree(g->work.d_items);
+  g->work = w;
+  return CORR_OK;
+}
+
 // One grouped accumulate.
 int group_enqueue(corr_group* g, const uint8_t* const* in, cudaStream_t st) {
   for (int i = 0; i < g->n; ++i)
     if (!g->ctx[i]->d_op)
       return fail(CORR_ERR_STATE, "group member " + std::to_string(i) +
                                       " has no operand scratch (its path was set to FP32 or int8; set a tensor path)");
-  return enqueue_group(g->ctx, g->n, in, st);
+  return enqueue_group(g->ctx, g->n, g->work, in, st);
 }
 
 void group_count(corr_group* g) {
@@ -101,6 +127,12 @@ corr_group* corr_group_create(int n_arrays, const int* n_inputs, const int* n_ch
       fail(CORR_ERR_ARG, "corr_group_create: sub-array " + std::to_string(i) + ": " + msg);
       return nullptr;
     }
+  }
+  if (group_build_work(g) != CORR_OK) {
+    const std::string msg = corr_last_error();
+    corr_group_destroy(g);
+    fail(CORR_ERR_OOM, "corr_group_create: " + msg);
+    return nullptr;
   }
   return g;
 }
@@ -182,7 +214,7 @@ int corr_group_autotune(corr_group* g, const void* const* d_samples, int* plans_
     cudaGraphExecDestroy(g->graph);
     g->graph = nullptr;
   }
-  return CORR_OK;
+  return group_build_work(g);
 }
 
 int corr_group_capture(corr_group* g, const void* const* d_samples, void* stream) {
@@ -229,6 +261,7 @@ int corr_group_destroy(corr_group* g) {
   if (!g) return CORR_OK;
   int rc = CORR_OK;
   if (g->graph) cudaGraphExecDestroy(g->graph);
+  cudaFree(g->work.d_items);
   for (int i = 0; i < g->n; ++i)
     if (g->ctx[i] && corr_destroy(g->ctx[i]) != CORR_OK) rc = CORR_ERR_CUDA;
   delete g;
