@@ -480,7 +480,9 @@ int corr_probe_mma_rate(int n_mma, int n_cols, double* tflops, double* cycles_pe
  * corr_group_capture  records one grouped accumulate of the given buffers into a CUDA graph
  *                     (pointers are baked in: refill the same buffers before each replay); needs a
  *                     non-default stream.
- * corr_group_launch   replays the captured graph (and advances the sample counters).
+ * corr_group_launch   replays the captured graph (and advances the sample counters). Tile plans set on members
+ *                     after the capture do not change it; CORR_ERR_STATE once a member has released operand
+ *                     scratch that the graph uses (corr_set_path, corr_set_batch_blocks, corr_autotune).
  */
 typedef struct corr_group corr_group;
 corr_group* corr_group_create(int n_arrays, const int* n_inputs, const int* n_chans, int n_time_per_block, int n_pol);

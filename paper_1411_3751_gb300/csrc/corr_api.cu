@@ -291,6 +291,8 @@ Route direct_route(const corr_ctx* c, const uint8_t* d_in) {
   return ROUTE_TWO_PASS;
 }
 
+bool uses_operand_scratch(const corr_ctx* c, const uint8_t* d_in) { return direct_route(c, d_in) != ROUTE_DIRECT; }
+
 Route route_of(const corr_ctx* c, const uint8_t* d_in) {
   return c->tile_plan != c->plan_default || c->prep_sms > 0 ? ROUTE_TWO_PASS : direct_route(c, d_in);
 }
@@ -536,6 +538,12 @@ int ensure_operand_scratch(corr_ctx* c) {
   return CORR_OK;
 }
 
+void release_operand_scratch(corr_ctx* c) {
+  cudaFree(c->d_op);
+  c->d_op = nullptr;
+  ++c->op_released;
+}
+
 int max_batch_blocks(const corr_ctx* c) {
   const unsigned long long ob = c->L.op_bytes > 0 ? c->L.op_bytes : 1;
   const unsigned long long k = kMaxOperandBuffer / ob;
@@ -548,9 +556,8 @@ int set_batch_blocks(corr_ctx* c, int K) {
   if (e != cudaSuccess) return cuda_fail(e, "set_batch_blocks: synchronize");
   const bool had_op = c->d_op != nullptr;
   const int old_K = c->L.K_batch;
-  cudaFree(c->d_op);
+  release_operand_scratch(c);
   cudaFree(c->d_op2);
-  c->d_op = nullptr;
   c->d_op2 = nullptr;
   c->L.K_batch = K;
   c->L.op_buf_bytes = c->L.op_bytes * (size_t)K;
@@ -850,8 +857,7 @@ int corr_set_path(corr_ctx* c, int path) {
     // FP32 and int8 paths unpack in shared memory: release the operand scratch once queued work is done
     const cudaError_t e = cudaDeviceSynchronize();
     if (e != cudaSuccess) return cuda_fail(e, "corr_set_path: synchronize");
-    cudaFree(c->d_op);
-    c->d_op = nullptr;
+    release_operand_scratch(c);
   }
   c->path = path;
   return CORR_OK;

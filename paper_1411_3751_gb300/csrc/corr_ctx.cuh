@@ -51,6 +51,7 @@ struct corr_ctx {
   long long n_off_auto;    // same, since the autos reset
   int* d_err;
   uint8_t* d_op;          // operand scratch of the two-pass tensor path (K_batch blocks)
+  unsigned op_released;   // times d_op was released: a captured launch that uses it is valid until then
   CUtensorMap tmap;
   CUtensorMap tmap_cp;    // the same buffer as channel-group boxes (64 or 32 operand rows: at most 32 inputs)
   // overlapped batches: the operand of chunk j + 1 is built on prep_sms SMs (TMA build kernel, on
@@ -121,6 +122,8 @@ struct GroupWork {
     int plan;
   } list[kMaxGroupArrays];
 };
+// a grouped launch on the array's block d_in goes through the operand scratch
+bool uses_operand_scratch(const corr_ctx* c, const uint8_t* d_in);
 // one block in[i] of each of n arrays through the tensor path (no counting)
 int enqueue_group(corr_ctx* const* ctx, int n, const GroupWork& work, const uint8_t* const* in, cudaStream_t st);
 // T_blk samples of a device block [T_blk][C][N] through the context's current path

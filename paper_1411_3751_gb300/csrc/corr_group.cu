@@ -22,6 +22,9 @@ struct corr_group {
   corr_ctx* ctx[kMaxGroupArrays];
   GroupWork work;
   cudaGraphExec_t graph;
+  // members whose operand scratch the graph uses, and their op_released at the capture
+  bool on_scratch[kMaxGroupArrays];
+  unsigned released[kMaxGroupArrays];
   int T;
 };
 
@@ -245,12 +248,21 @@ int corr_group_capture(corr_group* g, const void* const* d_samples, void* stream
   if (e != cudaSuccess) return cuda_fail(e, "corr_group_capture: instantiate");
   if (g->graph) cudaGraphExecDestroy(g->graph);
   g->graph = exec;
+  for (int i = 0; i < g->n; ++i) {
+    g->on_scratch[i] = uses_operand_scratch(g->ctx[i], static_cast<const uint8_t*>(d_samples[i]));
+    g->released[i] = g->ctx[i]->op_released;
+  }
   return CORR_OK;
 }
 
 int corr_group_launch(corr_group* g, void* stream) {
   if (!g) return fail(CORR_ERR_ARG, "corr_group_launch: NULL group");
   if (!g->graph) return fail(CORR_ERR_STATE, "corr_group_launch: no captured graph (call corr_group_capture)");
+  for (int i = 0; i < g->n; ++i)
+    if (g->on_scratch[i] && g->released[i] != g->ctx[i]->op_released)
+      return fail(CORR_ERR_STATE, "corr_group_launch: member " + std::to_string(i) +
+                                      " has released the operand scratch that the graph uses (its path or blocks per "
+                                      "launch changed): call corr_group_capture again");
   cudaError_t e = cudaGraphLaunch(g->graph, (cudaStream_t)stream);
   if (e != cudaSuccess) return cuda_fail(e, "corr_group_launch");
   group_count(g);

@@ -1,5 +1,5 @@
-"""Groups whose members' settings change between calls: a captured launch reads only what the group owns, against
-the oracle."""
+"""Groups whose members' settings change between calls: a captured launch reads only what the group owns, or is
+refused, against the oracle."""
 import numpy as np
 import pytest
 
@@ -55,3 +55,33 @@ def test_captured_group_outlives_its_members_work_lists(env, shapes):
                     dst.copy_(src)
                 g.launch(stream)
             _check(corr, g, blk, npol)
+
+
+@pytest.mark.parametrize("release", ["path", "batch_blocks"])
+def test_captured_group_is_refused_once_its_scratch_is_gone(env, release):
+    """A member's operand scratch is released after the capture (by its path, by its blocks per launch): the graph that
+    writes there is not launched, and a new capture works. Members that do not go through the scratch do not matter."""
+    corr, synth, torch = env
+    shapes, T, npol = [(64, 4), (200, 3)], 600, 2
+    blk = _blocks(synth, shapes, T, 0)
+
+    def let_go(m):
+        if release == "path":
+            m.set_path("fp32")
+            m.set_path("fp8tc")
+        else:
+            m.set_batch_blocks(1 if m.batch_blocks > 1 else 2)
+
+    stream = torch.cuda.Stream()
+    with torch.cuda.stream(stream), corr.Group(shapes, T, npol) as g:
+        stream.synchronize()
+        g.capture(blk, stream)
+        let_go(g.members[0])  # 64 inputs: correlated without the scratch
+        g.launch(stream)
+        let_go(g.members[1])
+        with pytest.raises(corr.CorrError):
+            g.launch(stream)
+        _check(corr, g, [blk], npol)  # the refused launch was not counted
+        g.capture(blk, stream)
+        g.launch(stream)
+        _check(corr, g, [blk, blk], npol)
