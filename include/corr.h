@@ -215,8 +215,9 @@ int corr_autotune(corr_ctx* ctx, const void* const* d_blocks, int n_blocks, int 
  * corr_set_flush_period - maximum number of samples accumulated in on-chip FP32/int32 partial sums
  * before they are added to the int64 accumulators (the paper integrates 8000-spectrum groups and
  * then sums 27 of them, Sec. 2.5; the flush cadence is this library's choice). 0 restores the
- * path default. Values are rounded down to the path's time granule; values above the path's
- * exactness bound (FP32 and FP8 paths: 65536) are rejected with CORR_ERR_ARG.
+ * path default. Values are rounded down to the path's time granule (a value below it, set while another path was
+ * selected, counts as one granule); values above the path's exactness bound (FP32 and FP8 paths: 65536) are
+ * rejected with CORR_ERR_ARG.
  */
 int corr_set_flush_period(corr_ctx* ctx, int n_samples);
 

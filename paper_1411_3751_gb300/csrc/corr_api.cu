@@ -198,8 +198,10 @@ bool valid_path(int path) {
 
 int flush_for(const corr_ctx* c, int path) {
   if (c->flush_len > 0) {
+    // at least one granule: a period set on the FP32 path may be shorter than the tensor paths', whose chunk loops
+    // would not advance by 0
     const int g = path == CORR_PATH_FP32 ? kF32Kt : kF8Kt;
-    return (c->flush_len / g) * g;
+    return std::max(g, (c->flush_len / g) * g);
   }
   return path == CORR_PATH_FP32 ? kDefaultFlushF32 : kDefaultFlushF8;
 }

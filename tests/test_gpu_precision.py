@@ -57,3 +57,20 @@ def test_flush_periods_saturating_input(env):
             assert tuple(cross[f, b, pq]) == tuple(got[k]), (f, b, pq)
     # the all -8-8i segment and the clipped segments saturate: autos stay exact integers >= 0
     assert autos.min() >= 0
+
+
+@pytest.mark.parametrize("path,n_inputs", [("fp8tc", 20), ("fp8tc", 72), ("i8mma", 20), ("fp8tc_fused", 64)])
+def test_flush_period_below_the_granule_of_the_path_that_runs(env, n_inputs, path):
+    """32 samples are the FP32 path's granule and a quarter of the tensor paths': a period set there and kept over a
+    change of path counts as one granule."""
+    corr, synth, torch = env
+    C, T = 2, 300
+    host = synth.generate_host(synth.Spec(kind="gauss_tone", seed=n_inputs), T, C, n_inputs)
+    with corr.Correlator(n_inputs, C, T, 2) as xc:
+        xc.set_path("fp32")
+        xc.set_flush_period(32)
+        xc.set_path(path)
+        xc.accumulate(torch.from_numpy(host).cuda())
+        cross = xc.dump(corr.CORR_WHAT_CROSS).cpu().numpy()
+        xc.sync()
+    assert np.array_equal(cross, oracle.correlate(host, 2, threads=8)[0])
