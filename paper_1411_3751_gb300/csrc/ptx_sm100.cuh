@@ -113,7 +113,13 @@ __device__ __forceinline__ void setmaxnreg_dec() {
 }
 
 // ---- tcgen05 --------------------------------------------------------------------------------
+// TMEM allocation, release and loads and the cluster barrier are for converged warps (.aligned), and stand behind
+// code that lanes leave one by one (roles of a single lane, bounded waits): each reconverges its warp first. A
+// warp that is still split would execute a release twice, which traps. (Costs nothing measurable here; in front of the
+// teardown's __syncthreads, where a role's idle lanes would wait for the working one, it slowed the SM-pair X-engine
+// at 512 inputs x 128 channels x 16 x 8192 samples from 9.19 to 9.32 ms.)
 __device__ __forceinline__ void tmem_alloc(uint32_t* dst_smem_slot, uint32_t ncols) {
+  __syncwarp();
   asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(dst_smem_slot)),
                "r"(ncols)
                : "memory");
@@ -122,6 +128,7 @@ __device__ __forceinline__ void tmem_relinquish() {
   asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
 }
 __device__ __forceinline__ void tmem_dealloc(uint32_t taddr, uint32_t ncols) {
+  __syncwarp();
   asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncols) : "memory");
 }
 // Make this thread's generic-proxy shared-memory writes visible to the async proxy (TMA, tcgen05).
@@ -157,6 +164,7 @@ __device__ __forceinline__ void mma_commit(uint64_t* bar) {
 
 // 32 lanes x 32 columns of 32-bit TMEM words: thread (lane) gets 32 consecutive columns of its lane.
 __device__ __forceinline__ void tmem_ld_32x32b_x32(uint32_t taddr, uint32_t (&r)[32]) {
+  __syncwarp();
   asm volatile(
       "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
       "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
@@ -213,6 +221,7 @@ __device__ __forceinline__ uint32_t mapa_shared(const void* p, uint32_t rank) {
 // All threads of both CTAs: everything before (barrier initialisation, TMEM allocation, shared-memory
 // writes) is visible cluster-wide after.
 __device__ __forceinline__ void cluster_sync() {
+  __syncwarp();
   asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 // Arrive on an mbarrier of any CTA of the cluster (shared::cluster address).
@@ -234,6 +243,7 @@ __device__ __forceinline__ void tma_load_3d_pair(void* smem_dst, const CUtensorM
 }
 // TMEM allocation of a CTA pair: issued by one warp in each of the two CTAs, same ncols.
 __device__ __forceinline__ void tmem_alloc_pair(uint32_t* dst_smem_slot, uint32_t ncols) {
+  __syncwarp();
   asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(dst_smem_slot)),
                "r"(ncols)
                : "memory");
@@ -242,6 +252,7 @@ __device__ __forceinline__ void tmem_relinquish_pair() {
   asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
 }
 __device__ __forceinline__ void tmem_dealloc_pair(uint32_t taddr, uint32_t ncols) {
+  __syncwarp();
   asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncols) : "memory");
 }
 // 2-SM MMA, issued by one thread of the pair's even CTA: A (M = 256) is 128 rows in each CTA's shared

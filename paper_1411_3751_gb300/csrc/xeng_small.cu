@@ -347,11 +347,10 @@ __global__ void __launch_bounds__(S_THREADS, 1) xeng_small_kernel(const __grid_c
       }
     }
   }
-  __syncwarp();  // the roles ran on single lanes: what follows is for whole warps (a second release of TMEM traps)
+  __syncwarp();  // the roles ran on single lanes: what follows is for whole warps
   ptx::tc_fence_before();
   __syncthreads();
   ptx::tc_fence_after();
-  __syncwarp();
   if (warp == 1) ptx::tmem_dealloc(tbase, TMEM_COLS);
 }
 
