@@ -175,32 +175,39 @@ __global__ void __launch_bounds__(PFB_NT, 2) pfb_kernel(const int8_t* __restrict
       for (int s = 0; s < PFB_SPB; ++s) v[s][r] = make_float2((float)y[s][0], (float)y[s][1]);
     }
   } else {
-    // any tap count: a tap of all 16 points at a time, their loads in flight together (point by point, as above, each
-    // load waited for the one before: 512 inputs x 8 spectra, 5 taps 189 us, 99 so)
-    int y[16][PFB_SPB][2], f[16];
+    // any tap count: four points at a time, four taps of each in flight. (A tap of all 16 points at a time was slower:
+    // 512 inputs x 8 spectra, 16 taps 180 us, 155 so, and with few spectra, where each step's latency shows, slower than
+    // the shared-memory FIR that it replaced: 64 inputs x 1 spectrum, 16 taps 16.4 us, 14.5 that one, 14.4 so.)
 #pragma unroll
-    for (int r = 0; r < 16; ++r) {
-      f[r] = load2(x + 512 * r);
-#pragma unroll
-      for (int s = 0; s < PFB_SPB; ++s) y[r][s][0] = y[r][s][1] = 0;
-    }
+    for (int r0 = 0; r0 < 16; r0 += 4) {
+      int y[4][PFB_SPB][2] = {};
 #pragma unroll 1
-    for (int p = 0; p < P; ++p) {
-      const bool more = p + 1 < P || ns > 1;
+      for (int p0 = 0; p0 < P; p0 += 4) {
+        int f[4][5];
+        int2 c[4][4];
 #pragma unroll
-      for (int r = 0; r < 16; ++r) {
-        const int2 c = __ldg(reinterpret_cast<const int2*>(hc + p * PFB_M + 512 * r));
-        y[r][0][0] += c.x * byte0(f[r]);
-        y[r][0][1] += c.y * byte1(f[r]);
-        f[r] = more ? load2(x + (size_t)(p + 1) * PFB_M + 512 * r) : 0;
-        y[r][1][0] += c.x * byte0(f[r]);
-        y[r][1][1] += c.y * byte1(f[r]);
+        for (int j = 0; j < 5; ++j)
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            const size_t at = (size_t)(p0 + j) * PFB_M + 512 * (r0 + i);
+            f[i][j] = p0 + j < P + ns - 1 ? load2(x + at) : 0;
+            if (j < 4) c[i][j] = p0 + j < P ? __ldg(reinterpret_cast<const int2*>(hc + at)) : make_int2(0, 0);
+          }
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+#pragma unroll
+          for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int s = 0; s < PFB_SPB; ++s) {
+              y[i][s][0] += c[i][j].x * byte0(f[i][j + s]);
+              y[i][s][1] += c[i][j].y * byte1(f[i][j + s]);
+            }
       }
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int s = 0; s < PFB_SPB; ++s) v[s][r0 + i] = make_float2((float)y[i][s][0], (float)y[i][s][1]);
     }
-#pragma unroll
-    for (int r = 0; r < 16; ++r)
-#pragma unroll
-      for (int s = 0; s < PFB_SPB; ++s) v[s][r] = make_float2((float)y[r][s][0], (float)y[r][s][1]);
   }
   // pass 1 (span 1): outputs 16 tid + q
 #pragma unroll
@@ -324,8 +331,8 @@ cudaError_t launch_pfb(const int8_t* d_adc, long long stride, int N, int T, int 
   if (e == cudaSuccess) e = ensure_twiddles(dev);
   if (e != cudaSuccess) return e;
   const dim3 grid((unsigned)((T + PFB_SPB - 1) / PFB_SPB), (unsigned)N);
-  // up to eight taps unrolled, every load of a point in flight at once (512 inputs x 8 spectra: 4 taps 83 us, 8 taps
-  // 100); in the loop over taps 5 taps took 99 against 87, 16 take 176
+  // up to eight taps unrolled, every load of a point in flight at once (512 inputs x 8 spectra: 4 taps 82 us, 8 taps
+  // 100); in the loop over taps 9 take 125, 16 take 155
   switch (P) {
     case 1: e = launch_taps<1>(d_adc, stride, T, P, d_h, d_out, grid, st); break;
     case 2: e = launch_taps<2>(d_adc, stride, T, P, d_h, d_out, grid, st); break;

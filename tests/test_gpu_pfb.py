@@ -118,3 +118,14 @@ def test_pfb_rejects_bad_arguments(env):
         corr.corr_pfb(d.data_ptr(), 2, d.stride(0), 4 * M, 4, coeffs.data_ptr(), 2, out.data_ptr(), None)
     with pytest.raises(corr.CorrError):  # misaligned samples
         corr.corr_pfb(d.data_ptr() + 1, 2, d.stride(0), 4 * M - 1, 4, coeffs.data_ptr(), 1, out.data_ptr(), None)
+
+
+@pytest.mark.parametrize("n_taps,T", [(9, 1), (9, 2), (11, 3), (12, 5), (16, 1), (16, 4), (64, 3)])
+def test_pfb_tap_counts_beyond_the_unrolled_ones(env, n_taps, T):
+    """The loop over groups of four taps: whole and partial last groups, one and two spectra in a block, full-scale
+    samples. FIR sums stay below 64 x 128 x 2^17 = 2^30; they are rounded to FP32 as in the other kernels."""
+    corr, torch = env
+    rng = np.random.default_rng(100 * n_taps + T)
+    adc = rng.choice(np.array([-128, -3, 5, 127], dtype=np.int8), size=(2, (T + n_taps - 1) * M))
+    X = corr.pfb(torch.from_numpy(adc).cuda(), n_taps=n_taps).cpu().numpy()
+    _check(X, adc, n_taps)
