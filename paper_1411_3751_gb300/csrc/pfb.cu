@@ -16,9 +16,10 @@
 // only twice: the FIR sums are formed by the threads whose first pass takes them, and in the last pass a
 // thread of a spectrum's 128 holds columns u and 256 - u, whose outputs are each other's mirror images
 // k and 4096 - k, so that the split step needs no exchange either. Twiddles come from tables computed on
-// the host in double precision. 512 inputs x 64 spectra, 4 taps: 753 us before, 588 us so
-// (2 CTAs of 8 warps an SM; without the FIR's loads 465, without the output stores 489; with 80 registers and a
-// third CTA 686, with the samples staged through shared memory by 16-byte loads 613).
+// the host in double precision. 512 inputs x 64 spectra, 4 taps: 753 us before, 573 us so
+// (2 CTAs of 8 warps an SM. At 588 us, with the split factors as products: without the FIR's loads 465, without the
+// output stores 489; with 80 registers and a third CTA 686, with the samples staged through shared memory by
+// 16-byte loads 613).
 #include "corr_internal.cuh"
 
 #include <cmath>
@@ -33,7 +34,7 @@ constexpr int PFB_NT = 256;
 constexpr float PFB_SCALE = 1.0f / 8192.0f;  // 2^-13
 
 __device__ float2 g_w4096[PFB_H];  // exp(-2 pi i j / 4096)
-__device__ float2 g_w8192[PFB_H];  // exp(-2 pi i k / 8192), k < 4096
+__device__ __align__(16) float2 g_w8192[PFB_H / 2];  // exp(-2 pi i k / 8192), k < 2048
 
 __device__ __forceinline__ float2 cmul(float2 a, float2 b) {
   return make_float2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
@@ -86,6 +87,22 @@ __device__ __forceinline__ void dft16(float2 (&v)[16]) {
 constexpr int PFB_SPB = 2;                    // spectra per block (share the coefficient and frame loads)
 constexpr int PFB_ZLEN = PFB_H + PFB_H / 16;  // padded complex buffer per spectrum
 
+// Rows q < 8 of the split step's factors W^(u + 256 q), u <= 128, beside the buffers (the others are -i times these).
+// From the table, each rounded once: as products W^u W^(256 q) their error is 2.4 times as large (the spectrum's 1.44e-7
+// instead of 1.39e-7, relative, 4 taps). They come with cp.async while the FIR runs: at the size above 573 us, as products 588, loaded
+// where they are used 628, all 16 rows so 716.
+constexpr int PFB_WLD = 130;  // row stride
+constexpr int PFB_SMEM = (PFB_SPB * PFB_ZLEN + 8 * PFB_WLD) * (int)sizeof(float2);
+
+__device__ __forceinline__ void fetch_split_factors(float2* ws, int tid) {
+  const int q = tid >> 5, u = 4 * (tid & 31);
+  const uint32_t dst = (uint32_t)__cvta_generic_to_shared(ws + q * PFB_WLD + u);
+  const float2* src = g_w8192 + 256 * q + u;
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + 16), "l"(src + 2) : "memory");
+  if (u == 0) asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(dst + 128 * 8), "l"(src + 128) : "memory");
+}
+
 // v[r] *= w^r for r = 1 .. 15 from w1 = w, w4 = w^4, w8, w12, as w^(4a + b) = w^(4a) w^b, for each of S columns.
 template <int S>
 __device__ __forceinline__ void twiddle16(float2 (&v)[S][16], float2 w1, float2 w4, float2 w8, float2 w12) {
@@ -123,32 +140,15 @@ __device__ __forceinline__ int load2(const int8_t* __restrict__ p) {
 __device__ __forceinline__ int byte0(int w) { return (int)(int8_t)(uint8_t)w; }
 __device__ __forceinline__ int byte1(int w) { return (int)(int8_t)(uint8_t)(w >> 8); }
 
-// W32^q = exp(-2 pi i q / 32): W^(256 q), the split step's factor between a column's outputs
-__device__ constexpr float2 kW32[16] = {
-    {1.f, -0.f},
-    {0.98078528040323043f, -0.19509032201612825f},
-    {0.92387953251128674f, -0.38268343236508977f},
-    {0.83146961230254524f, -0.55557023301960218f},
-    {0.70710678118654757f, -0.70710678118654752f},
-    {0.55557023301960229f, -0.83146961230254524f},
-    {0.38268343236508984f, -0.92387953251128674f},
-    {0.19509032201612833f, -0.98078528040323043f},
-    {0.f, -1.f},
-    {-0.19509032201612819f, -0.98078528040323043f},
-    {-0.38268343236508973f, -0.92387953251128674f},
-    {-0.55557023301960196f, -0.83146961230254546f},
-    {-0.70710678118654746f, -0.70710678118654757f},
-    {-0.83146961230254535f, -0.55557023301960218f},
-    {-0.92387953251128674f, -0.38268343236508989f},
-    {-0.98078528040323043f, -0.19509032201612861f}};
-
 // PT > 0 fixes the tap count at compile time; PT == 0 takes it from P.
 template <int PT>
 __global__ void __launch_bounds__(PFB_NT, 2) pfb_kernel(const int8_t* __restrict__ adc, long long stride, int T,
                                                         int P, const int* __restrict__ h, float2* __restrict__ out) {
-  extern __shared__ float2 zs[];  // PFB_SPB buffers of PFB_ZLEN
+  extern __shared__ __align__(16) float2 zs[];  // PFB_SPB buffers of PFB_ZLEN, the split factors
+  float2* ws = zs + PFB_SPB * PFB_ZLEN;
   const int t0 = blockIdx.x * PFB_SPB, n = blockIdx.y, tid = threadIdx.x;
   const int ns = T - t0 < PFB_SPB ? T - t0 : PFB_SPB;
+  fetch_split_factors(ws, tid);
   float2 v[PFB_SPB][16];
   // FIR: the thread's column of the first pass, points tid + 256 r, i.e. samples 2 tid + 512 r and the next,
   // of both spectra: frames t0 .. t0 + P (the last one only if there is a second spectrum)
@@ -235,6 +235,7 @@ __global__ void __launch_bounds__(PFB_NT, 2) pfb_kernel(const int8_t* __restrict
       for (int q = 0; q < 16; ++q) zs[s * PFB_ZLEN + sidx(base + 16 * q)] = v[s][q];
     }
   }
+  asm volatile("cp.async.wait_all;" ::: "memory");
   __syncthreads();
   // pass 3 (span 256) and split step: threads 128 s .. + 127 take spectrum s, thread u columns u and 256 - u
   // (thread 0: columns 0 and 128, each its own mirror image)
@@ -264,11 +265,11 @@ __global__ void __launch_bounds__(PFB_NT, 2) pfb_kernel(const int8_t* __restrict
   }
   float2* o = out + ((size_t)n * T + t0 + s) * PFB_H;
   if (u != 0) {
-    const float2 w = g_w8192[u];
 #pragma unroll
     for (int q = 0; q < 16; ++q) {  // k = u + 256 q, 4096 - k = 256 - u + 256 (15 - q)
       float2 xk, xm;
-      split_pair(za[q], zb[(16 - q) & 15], cmul(w, kW32[q]), xk, xm);
+      const float2 w = ws[(q & 7) * PFB_WLD + u];
+      split_pair(za[q], zb[(16 - q) & 15], q < 8 ? w : mul_mi(w), xk, xm);
       o[u + 256 * q] = xk;
       o[PFB_H - u - 256 * q] = xm;
     }
@@ -278,15 +279,14 @@ __global__ void __launch_bounds__(PFB_NT, 2) pfb_kernel(const int8_t* __restrict
 #pragma unroll
     for (int q = 1; q < 8; ++q) {  // k = 256 q, 4096 - k = 256 (16 - q)
       float2 xk, xm;
-      split_pair(za[q], za[16 - q], kW32[q], xk, xm);
+      split_pair(za[q], za[16 - q], ws[q * PFB_WLD], xk, xm);
       o[256 * q] = xk;
       o[PFB_H - 256 * q] = xm;
     }
-    const float2 w = g_w8192[128];
 #pragma unroll
     for (int q = 0; q < 8; ++q) {  // k = 128 + 256 q, 4096 - k = 128 + 256 (15 - q)
       float2 xk, xm;
-      split_pair(zb[q + 1], zb[(16 - q) & 15], cmul(w, kW32[q]), xk, xm);
+      split_pair(zb[q + 1], zb[(16 - q) & 15], ws[q * PFB_WLD + 128], xk, xm);
       o[128 + 256 * q] = xk;
       o[PFB_H - 128 - 256 * q] = xm;
     }
@@ -299,11 +299,11 @@ cudaError_t g_tw_err[64];
 cudaError_t ensure_twiddles(int dev) {
   if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
   std::call_once(g_tw_once[dev], [dev]() {
-    float2 w1[PFB_H], w2[PFB_H];
+    float2 w1[PFB_H], w2[PFB_H / 2];
     for (int j = 0; j < PFB_H; ++j) {
       const double a1 = -2.0 * M_PI * j / 4096.0, a2 = -2.0 * M_PI * j / 8192.0;
       w1[j] = make_float2((float)std::cos(a1), (float)std::sin(a1));
-      w2[j] = make_float2((float)std::cos(a2), (float)std::sin(a2));
+      if (j < PFB_H / 2) w2[j] = make_float2((float)std::cos(a2), (float)std::sin(a2));
     }
     cudaError_t e = cudaMemcpyToSymbol(g_w4096, w1, sizeof(w1));
     if (e == cudaSuccess) e = cudaMemcpyToSymbol(g_w8192, w2, sizeof(w2));
@@ -315,9 +315,8 @@ cudaError_t ensure_twiddles(int dev) {
 template <int PT>
 cudaError_t launch_taps(const int8_t* d_adc, long long stride, int T, int P, const int* d_h, float2* d_out, dim3 grid,
                         cudaStream_t st) {
-  constexpr int smem = PFB_SPB * PFB_ZLEN * (int)sizeof(float2);
-  const cudaError_t e = set_smem_limit(reinterpret_cast<const void*>(pfb_kernel<PT>), smem);
-  if (e == cudaSuccess) pfb_kernel<PT><<<grid, PFB_NT, smem, st>>>(d_adc, stride, T, P, d_h, d_out);
+  const cudaError_t e = set_smem_limit(reinterpret_cast<const void*>(pfb_kernel<PT>), PFB_SMEM);
+  if (e == cudaSuccess) pfb_kernel<PT><<<grid, PFB_NT, PFB_SMEM, st>>>(d_adc, stride, T, P, d_h, d_out);
   return e;
 }
 

@@ -129,3 +129,22 @@ def test_pfb_tap_counts_beyond_the_unrolled_ones(env, n_taps, T):
     adc = rng.choice(np.array([-128, -3, 5, 127], dtype=np.int8), size=(2, (T + n_taps - 1) * M))
     X = corr.pfb(torch.from_numpy(adc).cuda(), n_taps=n_taps).cpu().numpy()
     _check(X, adc, n_taps)
+
+
+def test_split_factors_are_rounded_once(env):
+    """One odd sample x: every stage before the split step passes it on unchanged, so X[k] = 2^-13 y W^k (y = h x the
+    integer FIR sum, W = exp(-2 pi i / 8192)) with two roundings a component, the factor's and the product's: at most
+    2^-24 each of the component itself, the factor's from the table entry, plus the second-order term."""
+    corr, torch = env
+    for taps, sample in ((1, 1), (4, 1)):
+        adc = np.zeros((1, taps * M), dtype=np.int8)
+        adc[0, (taps - 1) * M + sample] = 77
+        h = np.zeros((taps, M), dtype=np.int32)
+        h[:, sample] = 100003
+        out = corr.pfb(torch.from_numpy(adc).cuda(), n_taps=taps, coeffs=torch.from_numpy(h.ravel()).cuda())
+        x = out.cpu().numpy()[0, 0].astype(np.float64)
+        k = np.arange(M // 2)
+        w = np.exp(-2j * np.pi * k / M) * (77 * 100003) / 8192
+        for got, want in ((x[:, 0], w.real), (x[:, 1], w.imag)):
+            # (at k = 0 and 2048 one component is zero: the table's is 6e-17, exact arithmetic on it gives as little)
+            assert np.all(np.abs(got - want) <= np.abs(want) * (2.0 ** -23 + 2.0 ** -40) + 1e-12 * 941)
