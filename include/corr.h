@@ -463,14 +463,15 @@ int corr_probe_mma_rate(int n_mma, int n_cols, double* tflops, double* cycles_pe
  * Groups of sub-arrays. The paper's architecture scales by giving each GPU its own slice of the
  * problem (Sec. 2.5, Sec. 6: 109 channels per GPU, the same code from 32 to 512 inputs); a group
  * correlates several independent sub-arrays of different input and channel counts (sharing the
- * block length T and n_pol) on one GPU, each array's kernels behind the other's on one stream, which a CUDA graph
- * can replay.
+ * block length T and n_pol) on one GPU. Arrays of more than 64 inputs share one operand build and one persistent
+ * tensor-core launch, so small ones do not each pay a partly empty wave (those on SM pairs with long items run by
+ * themselves, which is faster); the others follow on the same stream. A CUDA graph can replay it all.
  *
  * corr_group_create   n_arrays (1..8) sub-arrays; each is an ordinary corr_ctx (tensor path).
  * corr_group_member   the i-th sub-array's context, for corr_dump / corr_reset / counters; owned by
  *                     the group (do not destroy it).
  * corr_group_accumulate  one block per sub-array (d_samples[i] device uint8[T][C_i][N_i]); mode 0:
- *                     all operand work first, then all X-engines; sub-arrays of at most 64 inputs
+ *                     all operand work first, then the X-engines; sub-arrays of at most 64 inputs
  *                     without an operand in HBM, whatever their tile plan; mode 1: as corr_accumulate
  *                     on each context (for comparison). Results are identical.
  * corr_group_autotune times the two tile plans of each sub-array on the given blocks, keeps the

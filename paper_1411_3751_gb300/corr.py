@@ -593,7 +593,7 @@ class Correlator:
 
 
 class Group:
-    """A group of sub-arrays correlated with one persistent tensor-core launch (corr_group_*)."""
+    """A group of sub-arrays correlated by one call, the larger ones in shared launches (corr_group_*)."""
 
     def __init__(self, shapes, n_time_per_block: int, n_pol: int = 2):
         self.shapes = [(int(n), int(c)) for n, c in shapes]

@@ -276,7 +276,9 @@ void free_ctx(corr_ctx* c) {
 
 // The context's two-pass launch on its own work list; buf: operand buffer d_op (0) or d_op2 (1).
 XengArgs xeng_args(const corr_ctx* c, int buf, int T_run, int flush);
+// One array's, on items of tile plan `plan`.
 XengArgs xeng_args(const corr_ctx* c, int plan, int buf, int T_run, int flush, const WorkItem* items, long long n_items);
+XengArray xeng_array(const corr_ctx* c, int plan, int buf);
 
 // How a block takes the tensor path: arrays of at most 64 inputs without an operand in HBM (launch_xeng_small) from
 // their own rows or from rows repacked to whole 16-byte columns; others, and where a tile plan or a build
@@ -292,6 +294,8 @@ Route direct_route(const corr_ctx* c, const uint8_t* d_in) {
   if (c->d_op && xeng_small_supported(s, Np, c->d_op)) return ROUTE_REPACK;
   return ROUTE_TWO_PASS;
 }
+
+bool takes_two_passes(const corr_ctx* c) { return !xeng_small_supported(c->L.s, repacked_inputs(c), nullptr); }
 
 bool uses_operand_scratch(const corr_ctx* c, const uint8_t* d_in) { return direct_route(c, d_in) != ROUTE_DIRECT; }
 
@@ -347,47 +351,57 @@ int accumulate_direct(corr_ctx* c, const uint8_t* const* blocks, int n, int T_bl
   return CORR_OK;
 }
 
-// One block of every array: the operand work first (repacked rows, or the two-pass build), then the X-engines one
-// behind the other, at most 64 inputs without an operand in HBM, the others on the group's own lists. Counts
-// nothing: a captured launch is counted when it is replayed. Timed and its waits reported on the first array,
-// flushed by its period. (One merged launch of all members' items on the one-SM kernel: five arrays of 32 to 512 inputs x 4096
-// samples with their dumps 1563 us, so 1280.)
+// One block of every array: the operand work first (repacked rows, or the two-pass build), then the X-engines, all on
+// one stream: at most 64 inputs without an operand in HBM, the others on the group's lists, merged or each by itself
+// (corr_group.cu). Counts nothing: a captured launch is counted when it is replayed. Timed and its waits reported
+// on the first array, flushed by its period.
 int enqueue_group(corr_ctx* const* ctx, int n, const GroupWork& work, const uint8_t* const* in, cudaStream_t st) {
   corr_ctx* c0 = ctx[0];
-  const int flush = flush_for(c0, CORR_PATH_FP8TC);
+  const int flush = flush_for(c0, CORR_PATH_FP8TC), T = c0->L.s.T, T_pad = c0->L.T_pad;  // shared by the arrays
   bool tb = timer_begin(c0, CORR_KERNEL_UNPACK, st);
+  PrepJobDesc jobs[kMaxGroupArrays];
+  int n_jobs = 0;
   for (int i = 0; i < n; ++i) {
     corr_ctx* c = ctx[i];
     const Shape& s = c->L.s;
     const Route route = direct_route(c, in[i]);
     cudaError_t e = cudaSuccess;
     if (route == ROUTE_REPACK)
-      e = launch_repack(in[i], (long long)s.T * s.C, s.N, repacked_inputs(c), c->d_op, st);
+      e = launch_repack(in[i], (long long)T * s.C, s.N, repacked_inputs(c), c->d_op, st);
+    else if (route == ROUTE_TWO_PASS && work.in_merged[i])
+      jobs[n_jobs++] = PrepJobDesc{s, in[i], T_pad * c->L.K_batch, c->L.R_buf, c->d_op, c->d_soff, c->d_soff_auto};
     else if (route == ROUTE_TWO_PASS)
-      e = launch_f8_prep(s, in[i], s.T, c->L.T_pad, c->L.T_pad * c->L.K_batch, 0, c->L.R_buf, c->d_op, c->d_soff,
-                         c->d_soff_auto, st);
+      e = launch_f8_prep(s, in[i], T, T_pad, T_pad * c->L.K_batch, 0, c->L.R_buf, c->d_op, c->d_soff, c->d_soff_auto, st);
     if (e != cudaSuccess) return cuda_fail(e, "group operand build");
   }
+  if (const cudaError_t e = launch_f8_prep_group(jobs, n_jobs, T, T_pad, st); e != cudaSuccess)
+    return cuda_fail(e, "group operand build");
   timer_end(c0, CORR_KERNEL_UNPACK, st, tb);
   tb = timer_begin(c0, CORR_KERNEL_XENG, st);
   for (int i = 0; i < n; ++i) {
     corr_ctx* c = ctx[i];
     const Route route = direct_route(c, in[i]);
-    cudaError_t e;
+    cudaError_t e = cudaSuccess;
     if (route == ROUTE_TWO_PASS) {
-      const GroupWork::List& l = work.list[i];
-      XengArgs a = xeng_args(c, l.plan, 0, c->L.T_pad, flush, work.d_items + l.first, l.n);
+      const GroupWork::List& l = work.own[i];
+      XengArgs a = xeng_args(c, l.plan, 0, T_pad, flush, work.d_items + l.first, l.n);
       a.err = c0->d_err;
-      e = launch_f8_xeng(a, c->num_sms, st);
+      e = launch_f8_xeng(a, c->num_sms, st);  // nothing to do for a merged one
     } else {
       const uint8_t* block = route == ROUTE_REPACK ? c->d_op : in[i];
-      DirectJob j = direct_job(c, c->L.s.T, route);
+      DirectJob j = direct_job(c, T, route);
       j.blocks = &block;
       j.n = 1;
       j.flush_len = flush;
       j.err = c0->d_err;
       e = launch_xeng_small(j, c->num_sms, st);
     }
+    if (e != cudaSuccess) return cuda_fail(e, "group x-engine launch");
+  }
+  if (work.merged.n > 0) {
+    XengArgs a = xeng_args(c0, work.merged.plan, 0, T_pad, flush, work.d_items + work.merged.first, work.merged.n);
+    for (int i = 0; i < n; ++i) a.a[i] = xeng_array(ctx[i], work.merged.plan, 0);
+    const cudaError_t e = launch_f8_xeng(a, c0->num_sms, st);
     if (e != cudaSuccess) return cuda_fail(e, "group x-engine launch");
   }
   timer_end(c0, CORR_KERNEL_XENG, st, tb);
@@ -493,18 +507,24 @@ int default_tile_plan(int N) {
 
 int channel_group(const Layout& L) { return L.R_buf == 64 ? 2 : (L.R_buf == 32 ? 4 : 0); }
 
+XengArray xeng_array(const corr_ctx* c, int plan, int buf) {
+  XengArray a;
+  std::memset(&a, 0, sizeof(a));
+  a.cgroup = plan < 2 ? channel_group(c->L) : 0;
+  a.tmap = a.cgroup ? (buf ? c->tmap2_cp : c->tmap_cp) : (buf ? c->tmap2 : c->tmap);
+  a.C = c->L.s.C;
+  a.cross = c->d_cross;
+  a.autos = c->d_autos;
+  a.Bs = c->L.s.Bs;
+  a.N = c->L.s.N;
+  a.npol = c->L.s.npol;
+  return a;
+}
+
 XengArgs xeng_args(const corr_ctx* c, int plan, int buf, int T_run, int flush, const WorkItem* items, long long n_items) {
   XengArgs a;
   std::memset(&a, 0, sizeof(a));
-  const int cgroup = plan < 2 ? channel_group(c->L) : 0;
-  a.a[0].tmap = cgroup ? (buf ? c->tmap2_cp : c->tmap_cp) : (buf ? c->tmap2 : c->tmap);
-  a.a[0].C = c->L.s.C;
-  a.a[0].cgroup = cgroup;
-  a.a[0].cross = c->d_cross;
-  a.a[0].autos = c->d_autos;
-  a.a[0].Bs = c->L.s.Bs;
-  a.a[0].N = c->L.s.N;
-  a.a[0].npol = c->L.s.npol;
+  a.a[0] = xeng_array(c, plan, buf);
   a.items = items;
   a.n_items = n_items;
   a.T_run = T_run;

@@ -113,15 +113,20 @@ int max_batch_blocks(const corr_ctx* c);
 int accumulate_batch_chunks(corr_ctx* c, const uint8_t* const* blocks, int n, cudaStream_t st);
 // Channel-major work list of the two-pass path on a tile plan.
 std::vector<WorkItem> work_items(const Layout& L, int plan);
-// Work lists of a group's arrays, owned by the group: a captured launch keeps reading them, whatever becomes of the
-// arrays' own lists (corr_set_tile_plan and corr_autotune replace those).
+// Work lists of a group's two-pass arrays, owned by the group: a captured launch keeps reading them, whatever becomes
+// of the arrays' own lists (corr_set_tile_plan and corr_autotune replace those).
 struct GroupWork {
-  WorkItem* d_items;  // list i: d_items[first .. first + n - 1], of tile plan `plan`
+  WorkItem* d_items;
   struct List {
-    long long first, n;
+    long long first, n;  // d_items[first .. first + n - 1]
     int plan;
-  } list[kMaxGroupArrays];
+  };
+  List own[kMaxGroupArrays];      // arrays that launch by themselves (n == 0: not this one)
+  List merged;                    // several arrays' items in one launch
+  bool in_merged[kMaxGroupArrays];
 };
+// the array takes the two passes whatever its block's alignment
+bool takes_two_passes(const corr_ctx* c);
 // a grouped launch on the array's block d_in goes through the operand scratch
 bool uses_operand_scratch(const corr_ctx* c, const uint8_t* d_in);
 // one block in[i] of each of n arrays through the tensor path (no counting)

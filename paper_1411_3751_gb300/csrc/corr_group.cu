@@ -62,25 +62,55 @@ void tune_store(const std::tuple<int, int, int, int, int>& k, int plan) {
   std::fclose(fh);
 }
 
-// The arrays' work lists on their tile plans, one behind the other; replaces the group's lists, so a graph that
-// reads these has to be dropped first.
+// Arrays that take two passes share one build and one X-engine launch on the one-SM kernel, where one array's last wave
+// is filled by the next one's items (with their dumps, 4096 samples: eight arrays of 256 inputs x 4 channels 387 us
+// each by itself, 177 so; four of 256 x 40 387 and 302; 32 to 512 inputs x 2400 to 109 channels 1285 and 1216). On SM
+// pairs (plan 3) an array with long items is faster by itself: two of 512 x 109 911 us apart and 864 merged at 4096
+// samples, 978 and 945 at 5120, but 1052 and 1072 at 6144 and 1267 and 1323 at 8192; three of 512 x 40 (5 items a
+// pair) 817 and 770 there.
+constexpr int kPairAloneSamples = 5632, kPairAloneItems = 8;  // longer blocks, at least so many items an SM pair
+bool launches_alone(const corr_ctx* c) {
+  return c->tile_plan == 3 && c->L.T_pad > kPairAloneSamples &&
+         (long long)work_items(c->L, 3).size() >= (long long)kPairAloneItems * (c->num_sms / 2);
+}
+
+// The work lists of the arrays that take two passes: the merged ones', in order of decreasing N (short items last, where
+// they even out the tail; plan 0 for 2 and 3), and the others', each on its tile plan. Replaces the group's
+// lists, so a graph that reads these has to be dropped first.
 int group_build_work(corr_group* g) {
   GroupWork w{};
   std::vector<WorkItem> items;
+  std::vector<int> merged;
+  for (int i = 0; i < g->n; ++i)
+    if (takes_two_passes(g->ctx[i]) && !launches_alone(g->ctx[i])) merged.push_back(i);
+  if (merged.size() < 2) merged.clear();
+  std::stable_sort(merged.begin(), merged.end(), [&](int x, int y) { return g->ctx[x]->L.s.N > g->ctx[y]->L.s.N; });
+  for (int i : merged) {
+    const corr_ctx* c = g->ctx[i];
+    w.in_merged[i] = true;
+    for (WorkItem it : work_items(c->L, c->tile_plan >= 2 ? 0 : c->tile_plan)) {
+      it.array = i;
+      items.push_back(it);
+    }
+  }
+  w.merged = GroupWork::List{0, (long long)items.size(), 0};
   for (int i = 0; i < g->n; ++i) {
     const corr_ctx* c = g->ctx[i];
+    if (!takes_two_passes(c) || w.in_merged[i]) continue;
     const std::vector<WorkItem> own = work_items(c->L, c->tile_plan);
-    w.list[i] = GroupWork::List{(long long)items.size(), (long long)own.size(), c->tile_plan};
+    w.own[i] = GroupWork::List{(long long)items.size(), (long long)own.size(), c->tile_plan};
     items.insert(items.end(), own.begin(), own.end());
   }
-  if (cudaMalloc(&w.d_items, items.size() * sizeof(WorkItem)) != cudaSuccess) {
-    cudaGetLastError();
-    return fail(CORR_ERR_OOM, "group work list allocation failed");
-  }
-  const cudaError_t e = cudaMemcpy(w.d_items, items.data(), items.size() * sizeof(WorkItem), cudaMemcpyHostToDevice);
-  if (e != cudaSuccess) {
-    cudaFree(w.d_items);
-    return cuda_fail(e, "group work list upload");
+  if (!items.empty()) {
+    if (cudaMalloc(&w.d_items, items.size() * sizeof(WorkItem)) != cudaSuccess) {
+      cudaGetLastError();
+      return fail(CORR_ERR_OOM, "group work list allocation failed");
+    }
+    const cudaError_t e = cudaMemcpy(w.d_items, items.data(), items.size() * sizeof(WorkItem), cudaMemcpyHostToDevice);
+    if (e != cudaSuccess) {
+      cudaFree(w.d_items);
+      return cuda_fail(e, "group work list upload");
+    }
   }
   cudaFree(g->work.d_items);
   g->work = w;

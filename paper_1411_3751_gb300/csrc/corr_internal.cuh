@@ -51,13 +51,13 @@ struct F8Tile {
   int pad;
 };
 
-// One work item of the two-pass tensor-core X-engine: a tile of one channel (array: always 0).
+// One work item of the two-pass tensor-core X-engine: a tile of one channel of one of the launch's arrays.
 struct WorkItem {
   int array, f, c0, a0, nb, pad;
 };
 
 constexpr int kMaxGroupArrays = 8;
-// The array of a two-pass tensor-core X-engine launch.
+// An array of a two-pass tensor-core X-engine launch: one, or several of a group (one-SM tile plans only).
 struct XengArray {
   CUtensorMap tmap;  // operand op[C][T_span][R] (the channel-group box when cgroup is set)
   long long* cross;
@@ -69,7 +69,7 @@ struct XengArray {
                // channels f .. f + cgroup - 1 stacked in one 128-row tile (c0 = a0 = 0, nb = 128)
 };
 struct XengArgs {
-  XengArray a[1];
+  XengArray a[kMaxGroupArrays];
   const WorkItem* items;
   long long n_items;
   int T_run;      // samples multiplied per item (multiple of kF8Kt)
@@ -127,6 +127,17 @@ cudaError_t launch_f8_fused(const Shape& s, const uint8_t* d_in, int T_blk, int 
 // The block is written at sample offset t_base of each channel's operand rows.
 cudaError_t launch_f8_prep(const Shape& s, const uint8_t* d_in, int T_blk, int T_run, int T_stride, int t_base, int R,
                            uint8_t* d_op, long long* d_s1, long long* d_s2, cudaStream_t st);
+// The builds of several arrays (one block of T_blk samples each, T_run written) in one launch; each job as
+// launch_f8_prep would build it alone at sample offset 0.
+struct PrepJobDesc {
+  Shape s;
+  const uint8_t* in;
+  int T_stride, R;
+  uint8_t* op;
+  long long* s1;
+  long long* s2;
+};
+cudaError_t launch_f8_prep_group(const PrepJobDesc* jobs, int n, int T_blk, int T_run, cudaStream_t st);
 
 // The same operand bytes and offset sums built with TMA loads and stores by at most max_ctas persistent
 // CTAs (one per SM), for running beside the X-engine (prep_tma.cu); f8_prep_tma_supported says whether

@@ -2,6 +2,9 @@
 // the GPU): packed bytes in[T][C][N] -> op[C][T_pad][R] (offset e4m3 bytes, group row order, MN-major:
 // one contiguous row of R bytes per channel and sample) plus the per-input offset sums. Streams
 // through HBM. Operand encoding and row order: f8_common.cuh.
+#include <cstring>
+#include <type_traits>
+
 #include "corr_internal.cuh"
 #include "f8_common.cuh"
 
@@ -27,13 +30,14 @@ constexpr int PREP_ROWS_PER_THREAD_MAX = 2048;
 // words around them, shifted together (single bytes where those would leave the block), four samples in flight.
 // 131 inputs x 300 channels x 4096 samples: 229 us by single bytes, 130 so (175 with eight samples in flight);
 // 202 inputs 329 and 175. (Widths as an argument and not a template cost the 16- and 8-byte builds 4 and 6%.)
+// The build of one block (bx, bz) of a grid: bx picks 8 units, bz the time range; part is shared memory for the
+// sums, [warp][unit][16 inputs x (Re, Im)].
+typedef int PrepSums[8][8][32];
 template <int VEC>
-__global__ void __launch_bounds__(256) f8_prep_kernel(const uint8_t* __restrict__ in, int N, int C, int T, int T_run,
-                                                      int T_stride, int t_base, int R, int rows_per_split,
-                                                      uint8_t* __restrict__ op, long long* __restrict__ s1,
-                                                      long long* __restrict__ s2) {
-  const long long bx = blockIdx.x;  // 8 units
-  const int bz = blockIdx.z;        // time range
+__device__ __forceinline__ void prep_block(const uint8_t* __restrict__ in, int N, int C, int T, int T_run, int T_stride,
+                                           int t_base, int R, int rows_per_split, uint8_t* __restrict__ op,
+                                           long long* __restrict__ s1, long long* __restrict__ s2, long long bx, int bz,
+                                           PrepSums& part) {
   const int G = R / 32;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int tl = lane >> 3, us = lane & 7;
@@ -49,7 +53,7 @@ __global__ void __launch_bounds__(256) f8_prep_kernel(const uint8_t* __restrict_
   uint32_t sre[4][2] = {{0u, 0u}, {0u, 0u}, {0u, 0u}, {0u, 0u}};
   uint32_t sim[4][2] = {{0u, 0u}, {0u, 0u}, {0u, 0u}, {0u, 0u}};
   if (unit_ok) {
-    // 8 samples per thread per iteration (4 if ANY), all loads issued before any conversion
+    // 8 samples per thread per iteration (4 by five-word loads), all loads issued before any conversion
     constexpr int U = VEC == 1 ? 4 : 8;
     const uint8_t* end = in + (size_t)T * C * N;
     for (int t0 = t_begin + 4 * warp + tl; t0 < t_end; t0 += 32 * U) {
@@ -116,7 +120,6 @@ __global__ void __launch_bounds__(256) f8_prep_kernel(const uint8_t* __restrict_
   }
   if (!s1 && !s2) return;
   // unpack to per-input sums, input j = 4 k + byte: even bytes 0, 2 / odd bytes 1, 3
-  __shared__ int part[8][8][32];  // [warp][unit][16 inputs x (Re, Im)]
   int v[32];
 #pragma unroll
   for (int k = 0; k < 4; ++k) {
@@ -156,6 +159,47 @@ __global__ void __launch_bounds__(256) f8_prep_kernel(const uint8_t* __restrict_
   }
 }
 
+template <int VEC>
+__global__ void __launch_bounds__(256) f8_prep_kernel(const uint8_t* __restrict__ in, int N, int C, int T, int T_run,
+                                                      int T_stride, int t_base, int R, int rows_per_split,
+                                                      uint8_t* __restrict__ op, long long* __restrict__ s1,
+                                                      long long* __restrict__ s2) {
+  __shared__ PrepSums part;
+  prep_block<VEC>(in, N, C, T, T_run, T_stride, t_base, R, rows_per_split, op, s1, s2, blockIdx.x, blockIdx.z, part);
+}
+
+// Several arrays' builds in one launch (arrays of a group that leave the GPU partly idle alone): job i owns the linear
+// blocks [blk0_i, blk0_{i+1}), gx_i blocks of units by its time ranges, as its own launch would lay them out.
+struct PrepJob {
+  const uint8_t* in;
+  uint8_t* op;
+  long long* s1;
+  long long* s2;
+  long long blk0;
+  int N, C, R, T_stride, rows, gx, vec;
+};
+struct PrepGroupArgs {
+  PrepJob job[kMaxGroupArrays];
+  int n, T, T_run;
+};
+
+__global__ void __launch_bounds__(256) f8_prep_group_kernel(const __grid_constant__ PrepGroupArgs a) {
+  __shared__ PrepSums part;
+  int i = 0;
+  while (i + 1 < a.n && blockIdx.x >= a.job[i + 1].blk0) ++i;
+  const PrepJob& j = a.job[i];
+  const long long b = blockIdx.x - j.blk0, bx = b % j.gx;
+  const int bz = (int)(b / j.gx);
+  auto build = [&](auto vec) {
+    prep_block<decltype(vec)::value>(j.in, j.N, j.C, a.T, a.T_run, j.T_stride, 0, j.R, j.rows, j.op, j.s1, j.s2, bx, bz,
+                                     part);
+  };
+  if (j.vec == 16) build(std::integral_constant<int, 16>());
+  else if (j.vec == 8) build(std::integral_constant<int, 8>());
+  else if (j.vec == 4) build(std::integral_constant<int, 4>());
+  else build(std::integral_constant<int, 1>());
+}
+
 // Widest load (16, 8 or 4 bytes, else 1) that keeps every unit's 16 input bytes aligned: the rows of
 // in[T][C][N] start at multiples of N bytes.
 int load_width(int N, const void* in) {
@@ -184,6 +228,28 @@ void prep_geometry(const Shape& s, int T_run, int R, long long* gx, int* split_o
 }
 
 }  // namespace
+
+cudaError_t launch_f8_prep_group(const PrepJobDesc* jobs, int n, int T_blk, int T_run, cudaStream_t st) {
+  if (T_run == 0 || n <= 0) return cudaSuccess;
+  if (n > kMaxGroupArrays) return cudaErrorInvalidValue;
+  PrepGroupArgs a;
+  std::memset(&a, 0, sizeof(a));
+  a.n = n;
+  a.T = T_blk;
+  a.T_run = T_run;
+  long long blocks = 0;
+  for (int i = 0; i < n; ++i) {
+    const PrepJobDesc& d = jobs[i];
+    int split = 1, rows = 0;
+    long long gx = 0;
+    prep_geometry(d.s, T_run, d.R, &gx, &split, &rows);
+    a.job[i] = PrepJob{d.in, d.op, d.s1, d.s2, blocks, d.s.N, d.s.C, d.R, d.T_stride, rows, (int)gx, load_width(d.s.N, d.in)};
+    blocks += gx * split;
+  }
+  if (blocks > 0x7FFFFFFFLL) return cudaErrorInvalidConfiguration;
+  f8_prep_group_kernel<<<(unsigned)blocks, 256, 0, st>>>(a);
+  return cudaGetLastError();
+}
 
 cudaError_t launch_f8_prep(const Shape& s, const uint8_t* d_in, int T_blk, int T_run, int T_stride, int t_base, int R,
                            uint8_t* d_op, long long* d_s1, long long* d_s2, cudaStream_t st) {

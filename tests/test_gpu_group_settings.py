@@ -85,3 +85,36 @@ def test_captured_group_is_refused_once_its_scratch_is_gone(env, release):
         g.capture(blk, stream)
         g.launch(stream)
         _check(corr, g, [blk, blk], npol)
+
+
+@pytest.mark.parametrize("shapes,T", [([(256, 4)] * 8, 700), ([(66, 5), (68, 3), (131, 2), (72, 4), (512, 2), (128, 3), (65, 1), (67, 7)], 1001),
+                                      ([(130, 3), (20, 4), (130, 3)], 130), ([(512, 1), (64, 2)], 300)])
+def test_members_that_share_a_launch(env, shapes, T):
+    """Groups whose larger members share one build and one X-engine launch: equal and uneven members, rows of every load
+    width, members without a share in it between them, a single larger member; two blocks, then a replayed graph."""
+    corr, synth, torch = env
+    npol = 1 if any(n % 2 for n, _ in shapes) else 2
+    blk = [_blocks(synth, shapes, T, k) for k in range(3)]
+    stream = torch.cuda.Stream()
+    with torch.cuda.stream(stream), corr.Group(shapes, T, npol) as g:
+        g.accumulate(blk[0])
+        g.accumulate(blk[1])
+        g.capture(blk[2], stream)
+        g.launch(stream)
+        _check(corr, g, blk, npol)
+
+
+def test_members_on_sm_pairs_beside_a_shared_launch(env):
+    """Blocks of more than 5632 samples and enough items for the 512-input member to launch by itself on SM pairs,
+    beside two members that share a launch and one on the 64-input kernel: every cell against the int8 path."""
+    corr, synth, torch = env
+    shapes, T, npol = [(512, 64), (128, 9), (64, 5), (200, 6)], 5700, 2
+    blk = _blocks(synth, shapes, T, 0)
+    with corr.Group(shapes, T, npol) as g:
+        g.accumulate(blk)
+        for (n, c), m, b in zip(shapes, g.members, blk):
+            with corr.Correlator(n, c, T, npol, path="i8mma") as ref:
+                ref.accumulate(b)
+                for what in (corr.CORR_WHAT_CROSS, corr.CORR_WHAT_AUTO):
+                    assert torch.equal(m.dump(what), ref.dump(what)), (n, what)
+            m.sync()
