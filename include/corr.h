@@ -474,9 +474,11 @@ int corr_probe_mma_rate(int n_mma, int n_cols, double* tflops, double* cycles_pe
  *                     all operand work first, then the X-engines; sub-arrays of at most 64 inputs
  *                     without an operand in HBM, whatever their tile plan; mode 1: as corr_accumulate
  *                     on each context (for comparison). Results are identical.
- * corr_group_autotune times the two tile plans of each sub-array on the given blocks, keeps the
- *                     faster one (cached in-process by (N, C, T, n_pol, SM count), and in the file
- *                     named by CORR_AUTOTUNE_CACHE if set), then zeroes the accumulators it touched.
+ * corr_group_autotune times the tile plans that the group's launch can run each sub-array on (0 and 1, and
+ *                     3 where that is the sub-array's default and it launches by itself) on the given
+ *                     blocks, keeps the fastest (cached in-process by (N, C, T, n_pol, SM count), and in the
+ *                     file named by CORR_AUTOTUNE_CACHE if set), then zeroes the accumulators it touched.
+ *                     Sub-arrays of at most 64 inputs, which run without a tile plan, go back to the default.
  *                     Synchronizes the stream. plans_out (optional) receives the chosen plans.
  *                     A graph captured earlier is dropped (capture again afterwards).
  * corr_group_capture  records one grouped accumulate of the given buffers into a CUDA graph

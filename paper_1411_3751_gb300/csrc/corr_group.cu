@@ -30,10 +30,12 @@ struct corr_group {
 
 namespace {
 
-// autotuner cache: (N, C, T, n_pol, SMs) -> tile plan; optionally mirrored in the file named by the
-// CORR_AUTOTUNE_CACHE environment variable (lines "N C T n_pol SMs plan")
+// autotuner cache: (N, C, T, n_pol, SMs, launched by itself) -> tile plan; optionally mirrored in the file named by the
+// CORR_AUTOTUNE_CACHE environment variable (lines "group N C T n_pol SMs by_itself plan"; lines without the tag are
+// an earlier version's, whose plans were chosen among fewer and for launches that are no longer made)
+typedef std::tuple<int, int, int, int, int, int> TuneKey;
 std::mutex g_tune_mu;
-std::map<std::tuple<int, int, int, int, int>, int> g_tune;
+std::map<TuneKey, int> g_tune;
 bool g_tune_loaded = false;
 
 void tune_load() {
@@ -43,22 +45,21 @@ void tune_load() {
   if (!path) return;
   FILE* fh = std::fopen(path, "r");
   if (!fh) return;
-  // lines "N C T n_pol SMs plan" (other lines in the file belong to other tuners)
   char line[256];
-  int a, b, c, d, e, p;
-  while (std::fgets(line, sizeof line, fh))
-    if (std::sscanf(line, "%d %d %d %d %d %d", &a, &b, &c, &d, &e, &p) == 6) g_tune[std::make_tuple(a, b, c, d, e)] = p;
+  int a, b, c, d, e, f, p;
+  while (std::fgets(line, sizeof line, fh))  // other lines in the file belong to other tuners
+    if (std::sscanf(line, "group %d %d %d %d %d %d %d", &a, &b, &c, &d, &e, &f, &p) == 7) g_tune[TuneKey(a, b, c, d, e, f)] = p;
   std::fclose(fh);
 }
 
-void tune_store(const std::tuple<int, int, int, int, int>& k, int plan) {
+void tune_store(const TuneKey& k, int plan) {
   g_tune[k] = plan;
   const char* path = std::getenv("CORR_AUTOTUNE_CACHE");
   if (!path) return;
   FILE* fh = std::fopen(path, "a");
   if (!fh) return;
-  std::fprintf(fh, "%d %d %d %d %d %d\n", std::get<0>(k), std::get<1>(k), std::get<2>(k), std::get<3>(k),
-               std::get<4>(k), plan);
+  std::fprintf(fh, "group %d %d %d %d %d %d %d\n", std::get<0>(k), std::get<1>(k), std::get<2>(k), std::get<3>(k),
+               std::get<4>(k), std::get<5>(k), plan);
   std::fclose(fh);
 }
 
@@ -69,10 +70,11 @@ void tune_store(const std::tuple<int, int, int, int, int>& k, int plan) {
 // samples, 978 and 945 at 5120, but 1052 and 1072 at 6144 and 1267 and 1323 at 8192; three of 512 x 40 (5 items a
 // pair) 817 and 770 there.
 constexpr int kPairAloneSamples = 5632, kPairAloneItems = 8;  // longer blocks, at least so many items an SM pair
-bool launches_alone(const corr_ctx* c) {
-  return c->tile_plan == 3 && c->L.T_pad > kPairAloneSamples &&
+bool long_on_pairs(const corr_ctx* c) {
+  return c->L.T_pad > kPairAloneSamples &&
          (long long)work_items(c->L, 3).size() >= (long long)kPairAloneItems * (c->num_sms / 2);
 }
+bool launches_alone(const corr_ctx* c) { return c->tile_plan == 3 && long_on_pairs(c); }
 
 // The work lists of the arrays that take two passes: the merged ones', in order of decreasing N (short items last, where
 // they even out the tail; plan 0 for 2 and 3), and the others', each on its tile plan. Replaces the group's
@@ -206,17 +208,29 @@ int corr_group_autotune(corr_group* g, const void* const* d_samples, int* plans_
   cudaEvent_t e0, e1;
   if (cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess)
     return cuda_fail(cudaGetLastError(), "corr_group_autotune: events");
-  int rc = CORR_OK;
+  int rc = CORR_OK, n_two_pass = 0;
+  for (int i = 0; i < g->n; ++i) n_two_pass += takes_two_passes(g->ctx[i]);
   for (int i = 0; i < g->n && rc == CORR_OK; ++i) {
     corr_ctx* c = g->ctx[i];
-    const auto key = std::make_tuple(c->L.s.N, c->L.s.C, c->L.s.T, c->L.s.npol, c->num_sms);
+    if (!takes_two_passes(c)) {  // correlated without a tile plan in a group, and by itself on the default one
+      if (c->tile_plan != c->plan_default) rc = set_tile_plan(c, c->plan_default);
+      if (rc == CORR_OK) rc = corr_reset(c, CORR_WHAT_CROSS | CORR_WHAT_AUTO, stream);
+      if (plans_out) plans_out[i] = c->plan_default;
+      continue;
+    }
+    // the plans that the group's launch can run the array on: the one-SM ones, and SM pairs where that is the default
+    // and the array would not be merged on it
+    const bool by_itself = n_two_pass == 1 || long_on_pairs(c);
+    std::vector<int> plans = {0, 1};
+    if (by_itself && c->plan_default == 3) plans = {3, 0, 1};
+    const TuneKey key(c->L.s.N, c->L.s.C, c->L.s.T, c->L.s.npol, c->num_sms, by_itself);
     auto it = g_tune.find(key);
-    int best = 0;
-    if (it != g_tune.end()) {
+    int best = plans[0];
+    if (it != g_tune.end() && std::find(plans.begin(), plans.end(), it->second) != plans.end()) {
       best = it->second;
     } else {
       float best_ms = 1e30f;
-      for (int plan = 0; plan < 2 && rc == CORR_OK; ++plan) {
+      for (int plan : plans) {
         rc = set_tile_plan(c, plan);
         if (rc != CORR_OK) break;
         // one warm-up block, then three timed blocks through the tensor path of this array alone
@@ -226,6 +240,7 @@ int corr_group_autotune(corr_group* g, const void* const* d_samples, int* plans_
         }
         cudaEventRecord(e1, st);
         if (cudaEventSynchronize(e1) != cudaSuccess) rc = cuda_fail(cudaGetLastError(), "corr_group_autotune");
+        if (rc != CORR_OK) break;
         float ms = 0.f;
         cudaEventElapsedTime(&ms, e0, e1);
         if (ms < best_ms) {

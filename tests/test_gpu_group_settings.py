@@ -118,3 +118,56 @@ def test_members_on_sm_pairs_beside_a_shared_launch(env):
                 for what in (corr.CORR_WHAT_CROSS, corr.CORR_WHAT_AUTO):
                     assert torch.equal(m.dump(what), ref.dump(what)), (n, what)
             m.sync()
+
+
+# run in a process of its own: the tuner reads the file named by CORR_AUTOTUNE_CACHE once
+TUNE = """
+import sys, torch
+sys.path.insert(0, %r)
+from paper_1411_3751_gb300 import corr, synth
+shapes, T = %r, %d
+blk = [synth.generate_device(synth.Spec(kind="gauss_tone", seed=i), T, c, n) for i, (n, c) in enumerate(shapes)]
+with corr.Group(shapes, T, 2) as g:
+    g.members[0].set_tile_plan(1)
+    plans = g.autotune(blk)
+    assert plans == [m.tile_plan for m in g.members]
+    g.accumulate(blk)
+    for m, (n, c), b in zip(g.members, shapes, blk):
+        with corr.Correlator(n, c, T, 2, path="i8mma") as ref:
+            ref.accumulate(b)
+            assert torch.equal(m.dump(corr.CORR_WHAT_CROSS), ref.dump(corr.CORR_WHAT_CROSS))
+    g.members[0].sync()
+print("plans", plans)
+"""
+
+
+def test_group_autotuner_chooses_among_what_the_group_runs(env, tmp_path):
+    """Members without a tile plan keep the default; the 512-input member that launches by itself on SM pairs can stay
+    there. Plans that an earlier version saved for members of the same shapes are not applied; the new ones are."""
+    import os
+    import re
+    import subprocess
+    import sys
+
+    corr, _, torch = env
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    shapes, T = [(64, 4), (32, 5), (512, 64), (200, 3)], 5700
+    cache = tmp_path / "tuned"
+
+    def tune(lines):
+        cache.write_text("".join(line + "\n" for line in lines))
+        r = subprocess.run([sys.executable, "-c", TUNE % (root, shapes, T)], capture_output=True, text=True, timeout=300,
+                           env=dict(os.environ, CORR_AUTOTUNE_CACHE=str(cache)))
+        assert r.returncode == 0, r.stderr[-2000:]
+        saved = cache.read_text().splitlines()[len(lines):]
+        return [int(p) for p in re.search(r"plans \[(.*)\]", r.stdout).group(1).split(",")], saved
+
+    old = ["%d %d %d 2 %d 1" % (n, c, T, sms) for n, c in shapes]
+    plans, saved = tune(old)
+    assert plans[:2] == [0, 0] and plans[2] in (0, 1, 3) and plans[3] in (0, 1)
+    # timed and saved anew: the two members that have a choice, nothing for the others
+    assert [line.split()[:3] for line in saved] == [["group", "512", "64"], ["group", "200", "3"]]
+    for want in (3, 1):  # a saved choice among the plans that the launch can run is applied without timing
+        plans, again = tune(["group 512 64 %d 2 %d 1 %d" % (T, sms, want), "group 200 3 %d 2 %d 0 1" % (T, sms)])
+        assert plans == [0, 0, want, 1] and not again
