@@ -203,8 +203,8 @@ typedef struct corr_tuning {
  * and `reps` (1 .. 100) times timed with CUDA events on cuda_stream; the default schedule (the
  * shape's default plan) is timed first and another replaces the best only when at least 1% faster.
  * The results are cached in-process by (N, C, T, n_pol, SMs, n_blocks), and in the file named by
- * CORR_AUTOTUNE_CACHE if set; a cached
- * choice is applied without timing. Afterwards the accumulators and sample counts are zero (the trials
+ * CORR_AUTOTUNE_CACHE if set; a cached choice is applied without timing (what earlier versions saved for
+ * at most 64 inputs is not used: those arrays run without the two passes by default now). Afterwards the accumulators and sample counts are zero (the trials
  * added into them). Synchronizes the device. out (optional) receives the choice. No counterpart in the
  * paper. CORR_ERR_STATE unless the context runs the two-pass tensor path.
  */

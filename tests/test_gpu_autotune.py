@@ -81,3 +81,44 @@ def test_autotune_needs_the_tensor_path(env):
     with corr.Correlator(64, 1, 256, 2, path="fp32") as xc:
         with pytest.raises(corr.CorrError):
             xc.autotune(blocks)
+
+
+# run in a process of its own: the tuner reads the file named by CORR_AUTOTUNE_CACHE once
+TUNE = """
+import sys, torch
+sys.path.insert(0, %r)
+from paper_1411_3751_gb300 import corr
+for n in (64, 256):
+    blocks = [torch.zeros((128, 2, n), dtype=torch.uint8, device="cuda") for _ in range(3)]
+    with corr.Correlator(n, 2, 128, 2) as xc:
+        c = xc.autotune(blocks, reps=1)
+        print("tuned", n, c["n_tried"] > 0, c["tile_plan"], c["batch_blocks"], c["prep_sms"])
+"""
+
+
+def test_saved_schedules_of_small_arrays_from_earlier_versions_are_timed_anew(env, tmp_path):
+    """A "batch" line holds for more than 64 inputs; at most 64 have a tag of their own, since what was saved for them
+    before would keep them in the two passes."""
+    import os
+    import subprocess
+    import sys
+
+    _, _, torch = env
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    cache = tmp_path / "tuned"
+    line = "%%s %%d 2 128 2 %d 3 1 2 0 0.001000" % sms
+
+    def tune():
+        r = subprocess.run([sys.executable, "-c", TUNE % root], capture_output=True, text=True, timeout=300,
+                           env=dict(os.environ, CORR_AUTOTUNE_CACHE=str(cache)))
+        assert r.returncode == 0, r.stderr[-2000:]
+        return [t.split()[1:] for t in r.stdout.splitlines() if t.startswith("tuned")]
+
+    cache.write_text(line % ("batch", 64) + "\n" + line % ("batch", 256) + "\n")
+    small, large = tune()
+    assert small[:2] == ["64", "True"] and large == ["256", "False", "1", "2", "0"]
+    assert [t.split()[:2] for t in cache.read_text().splitlines()[2:]] == [["batch64", "64"]]
+    cache.write_text(line % ("batch64", 64) + "\n" + line % ("batch64", 256) + "\n")
+    small, large = tune()
+    assert small == ["64", "False", "1", "2", "0"] and large[:2] == ["256", "True"]
