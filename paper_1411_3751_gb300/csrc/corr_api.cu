@@ -983,7 +983,12 @@ int corr_autotune(corr_ctx* c, const void* const* d_blocks, int n_blocks, int re
   double best_ms = 0.0;
   int rc = CORR_OK;
   const auto hit = g_ctx_tune.find(key);
-  if (hit != g_ctx_tune.end()) {
+  // a line of the file is taken only if it could have been saved for this context
+  const auto usable = [c](const std::tuple<int, int, int, double>& v) {
+    const int plan = std::get<0>(v), K = std::get<1>(v), prep = std::get<2>(v);
+    return plan >= 0 && plan <= 3 && K >= 1 && (K <= max_batch_blocks(c) || K == c->K_default) && prep >= 0 && prep <= c->num_sms;
+  };
+  if (hit != g_ctx_tune.end() && usable(hit->second)) {
     std::tie(best_plan, best_K, best_prep, best_ms) = hit->second;
   } else {
     cudaEvent_t e0 = nullptr, e1 = nullptr;

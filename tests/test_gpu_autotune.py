@@ -122,3 +122,22 @@ def test_saved_schedules_of_small_arrays_from_earlier_versions_are_timed_anew(en
     cache.write_text(line % ("batch64", 64) + "\n" + line % ("batch64", 256) + "\n")
     small, large = tune()
     assert small == ["64", "False", "1", "2", "0"] and large[:2] == ["256", "True"]
+
+
+@pytest.mark.parametrize("plan,blocks,prep", [(9, 2, 0), (-1, 2, 0), (1, 0, 0), (1, 20000000, 0), (1, 2, 100000), (1, 2, -5)])
+def test_impossible_saved_schedules_are_not_applied(env, tmp_path, plan, blocks, prep):
+    """A damaged line (no such tile plan, no or more blocks a launch than the operand buffer may hold, no such number of
+    SMs) is timed anew: 20 million blocks a launch of this shape would overflow the sample offsets."""
+    import os
+    import subprocess
+    import sys
+
+    _, _, torch = env
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    cache = tmp_path / "tuned"
+    cache.write_text("batch 256 2 128 2 %d 3 %d %d %d 0.001000\n" % (sms, plan, blocks, prep))
+    r = subprocess.run([sys.executable, "-c", TUNE % root], capture_output=True, text=True, timeout=300,
+                       env=dict(os.environ, CORR_AUTOTUNE_CACHE=str(cache)))
+    assert r.returncode == 0, r.stderr[-2000:]
+    assert any(t.split()[1:3] == ["256", "True"] for t in r.stdout.splitlines() if t.startswith("tuned"))
