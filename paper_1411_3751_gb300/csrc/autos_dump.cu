@@ -14,8 +14,8 @@ namespace {
 //
 // A square of a 4-bit component x = m - 8 s (s the sign bit, m the low three) is m^2 or (8 - m)^2: a byte
 // permute with the nibbles as selectors looks four of them up at once, the selectors' top bit making
-// the other sign's entries zero (the permute then repeats the entry's top bit, clear in every entry). Three
-// rows' squares (at most 64) fit a byte lane; then the halves of a sample are added into 16-bit lanes.
+// the other sign's entries zero (the permute then repeats the entry's top bit, clear in every entry). Two
+// rows' squares (at most 64 each) fit a byte lane; then the halves of a sample are added into 16-bit lanes.
 // (A dp4a a sample for the sums runs at a quarter of the other instructions' rate: 85 us at 512 inputs x 2400
 // channels x 240 aligned samples, 77 so, 358 with one byte a load.)
 constexpr int AU_NT = 256, AU_W = AU_NT / 32, AU_U = 4;
@@ -28,16 +28,10 @@ __device__ __forceinline__ uint32_t squares4(uint32_t w, uint32_t wx) {
   return p | q;
 }
 
-// acc[0], acc[1] (16-bit lanes, samples 0, 1 and 2, 3 of the words) += |x|^2 over the same word of R <= 3 rows.
-template <int R>
-__device__ __forceinline__ void add_power4(uint32_t (&acc)[2], const uint32_t (&w)[R]) {
-  uint32_t lo = 0u, hi = 0u;
-#pragma unroll
-  for (int r = 0; r < R; ++r) {
-    const uint32_t wx = w[r] ^ 0x88888888u;
-    lo += squares4(w[r], wx);
-    hi += squares4(w[r] >> 16, wx >> 16);
-  }
+// acc[0], acc[1] (16-bit lanes, samples 0, 1 and 2, 3 of the words) += |x|^2 over the same word of two rows.
+__device__ __forceinline__ void add_power4(uint32_t (&acc)[2], uint32_t w0, uint32_t w1) {
+  const uint32_t x0 = w0 ^ 0x88888888u, x1 = w1 ^ 0x88888888u;
+  const uint32_t lo = squares4(w0, x0) + squares4(w1, x1), hi = squares4(w0 >> 16, x0 >> 16) + squares4(w1 >> 16, x1 >> 16);
   acc[0] += (lo & 0x00FF00FFu) + ((lo >> 8) & 0x00FF00FFu);
   acc[1] += (hi & 0x00FF00FFu) + ((hi >> 8) & 0x00FF00FFu);
 }
@@ -87,10 +81,10 @@ __global__ void __launch_bounds__(AU_NT) autos_kernel(const uint8_t* __restrict_
       load(nx, t0);
 #pragma unroll
       for (int u = 0; u < AU_U; u += 2) {
-        add_power4<2>(acc[0], {w[u].x, w[u + 1].x});
-        add_power4<2>(acc[1], {w[u].y, w[u + 1].y});
-        add_power4<2>(acc[2], {w[u].z, w[u + 1].z});
-        add_power4<2>(acc[3], {w[u].w, w[u + 1].w});
+        add_power4(acc[0], w[u].x, w[u + 1].x);
+        add_power4(acc[1], w[u].y, w[u + 1].y);
+        add_power4(acc[2], w[u].z, w[u + 1].z);
+        add_power4(acc[3], w[u].w, w[u + 1].w);
       }
 #pragma unroll
       for (int u = 0; u < AU_U; ++u) w[u] = nx[u];

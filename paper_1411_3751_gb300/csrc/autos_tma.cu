@@ -135,7 +135,7 @@ cudaError_t launch_autos_tma(const Shape& s, const uint8_t* d_in, int T_blk, lon
   std::memset(&a, 0, sizeof(a));
   a.M = (long long)s.C * s.N;
   std::string err;
-  if (encode_raw_tensor_map(&a.map, d_in, a.M, T_blk, 128, &err) != 0) {
+  if (encode_raw_tensor_map(&a.map, d_in, a.M, T_blk, &err) != 0) {
     set_last_error(err);
     return cudaErrorInvalidValue;
   }

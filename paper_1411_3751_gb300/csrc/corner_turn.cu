@@ -32,11 +32,11 @@ __device__ __forceinline__ int find_part(const Bounds& bd, long long x) {
 }
 
 // HBM-bound (1000 samples x 2398 channels x 32 inputs, then 16 sources of 32 inputs x 109 channels: one
-// warp per 32-byte row, two of its lanes busy and a 64-bit division and a search a row, took 367 + 181 us).
+// warp per 32-byte row, two of its lanes busy and a 64-bit division and a search a row, took 367 + 182 us).
 //
 // Pack: the channels of destination d are neighbours in every input row t, and stay neighbours in its
 // block, so (t, d) is one contiguous run of C_d n_local bytes on both sides. A warp copies pieces of
-// at most PIECE bytes of such a run, four loads in flight a lane: 367 -> 47 us.
+// at most PIECE bytes of such a run, four loads in flight a lane: 367 -> 25 us.
 constexpr int CT_PIECE = 4096;
 constexpr int CT_NT = 256;
 
@@ -74,7 +74,7 @@ __global__ void __launch_bounds__(CT_NT) ct_pack_kernel(const uint8_t* __restric
 // Unpack: a thread keeps one granule column of the output rows, so it looks its source up once, and
 // walks down the rows, eight loads in flight; neighbouring threads write neighbouring granules.
 // `cols` columns a block (threadIdx.x % cols; blockIdx.x counts blocks of columns), CT_NT / cols rows a
-// step: 181 -> 22 us.
+// step: 182 -> 23 us.
 template <typename V>
 __global__ void __launch_bounds__(CT_NT) ct_unpack_kernel(const uint8_t* __restrict__ in, long long rows, int N, int cols,
                                                           const __grid_constant__ Bounds inputs,

@@ -203,10 +203,8 @@ int encode_op_tensor_map(CUtensorMap* map, void* d_op, int R, int T_pad, int C, 
 // Raw input in[T][C][N] as a 3-D map, boxes of 64 inputs x 1 channel x 128 samples, no swizzle.
 int encode_input_tensor_map(CUtensorMap* map, const void* d_in, int N, int C, int T, std::string* err);
 
-// A block in[T][C][N] as a 2-D map of T rows of C N bytes, boxes of box_bytes (64 or 128, swizzled as
-// wide) x 128 samples.
-int encode_raw_tensor_map(CUtensorMap* map, const void* d_in, long long row_bytes, int T, int box_bytes,
-                          std::string* err);
+// A block in[T][C][N] as a 2-D map of T rows of C N bytes, boxes of 128 bytes (128-byte swizzle) x 128 samples.
+int encode_raw_tensor_map(CUtensorMap* map, const void* d_in, long long row_bytes, int T, std::string* err);
 
 // X-engine that builds its operand on the chip (xeng_small.cu), at most 64 inputs: n blocks of one array, products
 // into cross and autos, offset sums into s1 and s2. xeng_small_supported: the shapes, row lengths ld (inputs a

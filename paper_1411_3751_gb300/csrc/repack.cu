@@ -2,7 +2,7 @@
 // TMA (xeng_small.cu): in[rows][N] -> out[rows][Np], Np = N rounded up to 16, zeros behind the last input. Taken where
 // a sample of all channels is not a multiple of 16 bytes (TMA's stride) or the block starts between 16-byte
 // boundaries. Reads one byte a sample and writes little more (the two-pass path writes two and reads them back):
-// 20 inputs x 1200 channels x 4096 samples with the X-engine behind it 91 us (two passes 157).
+// with the X-engine behind it 20 inputs x 1201 channels x 4096 samples 91 us (two passes 163), 63 x 601 118 (172).
 //
 // HBM-bound. A thread keeps one 16-byte column of the output rows and walks down them, several rows in flight. The
 // input rows start at any byte: where rows and buffer are not multiples of 8 or 4 bytes a column is the five
@@ -14,7 +14,7 @@ namespace corr {
 namespace {
 
 constexpr int RP_NT = 256;
-// rows in flight: 8, or 4 of the five-word columns (134 inputs x 300 channels x 4096: 8 rows took 21 us more)
+// rows in flight: 8, or 4 of the five-word columns (63 inputs x 601 channels x 4096: 64 us, with 8 rows 80)
 constexpr int RP_WIDE = 8, RP_NARROW = 4;
 
 // The 16 bytes at p, nv of them inputs, zeros behind. ALIGN 8 or 4: rows and buffer are multiples of it, whole pieces.
@@ -55,18 +55,18 @@ __device__ __forceinline__ uint4 load_column(const uint8_t* p, int nv, const uin
   return make_uint4(x[0], x[1], x[2], x[3]);
 }
 
-// blockIdx.x: blocks of `cols` columns; blockIdx.y: rows.
+// A block step takes RP_NT / cols rows of cols = Np / 16 columns (at most four, so a few threads idle at three).
 template <int ALIGN>
-__global__ void __launch_bounds__(RP_NT) repack_kernel(const uint8_t* __restrict__ in, long long rows, int N, int Np, int cols,
+__global__ void __launch_bounds__(RP_NT) repack_kernel(const uint8_t* __restrict__ in, long long rows, int N, int Np,
                                                        uint8_t* __restrict__ out) {
   constexpr int RP_U = ALIGN > 1 ? RP_WIDE : RP_NARROW;
-  const int rpb = RP_NT / cols, sub = (int)threadIdx.x / cols;
-  const int n0 = 16 * ((int)blockIdx.x * cols + (int)threadIdx.x - sub * cols);
-  if (sub >= rpb || n0 >= Np) return;
+  const int cols = Np / 16, rpb = RP_NT / cols, sub = (int)threadIdx.x / cols;
+  const int n0 = 16 * ((int)threadIdx.x - sub * cols);
+  if (sub >= rpb) return;
   const int nv = min(16, N - n0);
   const uint8_t* end = in + rows * N;
-  const long long step = (long long)gridDim.y * rpb;
-  for (long long r = (long long)blockIdx.y * rpb + sub; r < rows; r += RP_U * step) {
+  const long long step = (long long)gridDim.x * rpb;
+  for (long long r = (long long)blockIdx.x * rpb + sub; r < rows; r += RP_U * step) {
     uint4 v[RP_U];
 #pragma unroll
     for (int u = 0; u < RP_U; ++u)
@@ -81,21 +81,18 @@ __global__ void __launch_bounds__(RP_NT) repack_kernel(const uint8_t* __restrict
 
 cudaError_t launch_repack(const uint8_t* d_in, long long rows, int N, int Np, uint8_t* d_out, cudaStream_t st) {
   if (rows == 0) return cudaSuccess;
-  const int all = Np / 16, cols = all < RP_NT ? all : RP_NT;
-  const unsigned gx = (unsigned)((all + cols - 1) / cols);
-  const int rpb = RP_NT / cols;
+  if (Np > 64) return cudaErrorInvalidValue;
+  const int rpb = RP_NT / (Np / 16);
   const uintptr_t x = reinterpret_cast<uintptr_t>(d_in) | (uintptr_t)N;
   const int rows_step = rpb * (x % 4 == 0 ? RP_WIDE : RP_NARROW);
-  long long gy = (rows + rows_step - 1) / rows_step;
-  const long long cap = ((long long)sm_count() * 16 + gx - 1) / gx;
-  if (gy > cap) gy = cap;
-  const dim3 grid(gx, (unsigned)gy);
+  const long long want = (rows + rows_step - 1) / rows_step, cap = (long long)sm_count() * 16;
+  const unsigned grid = (unsigned)(want < cap ? want : cap);
   if (x % 8 == 0)
-    repack_kernel<8><<<grid, RP_NT, 0, st>>>(d_in, rows, N, Np, cols, d_out);
+    repack_kernel<8><<<grid, RP_NT, 0, st>>>(d_in, rows, N, Np, d_out);
   else if (x % 4 == 0)
-    repack_kernel<4><<<grid, RP_NT, 0, st>>>(d_in, rows, N, Np, cols, d_out);
+    repack_kernel<4><<<grid, RP_NT, 0, st>>>(d_in, rows, N, Np, d_out);
   else
-    repack_kernel<1><<<grid, RP_NT, 0, st>>>(d_in, rows, N, Np, cols, d_out);
+    repack_kernel<1><<<grid, RP_NT, 0, st>>>(d_in, rows, N, Np, d_out);
   return cudaGetLastError();
 }
 

@@ -394,16 +394,15 @@ int encode_input_tensor_map(CUtensorMap* map, const void* d_in, int N, int C, in
   return 0;
 }
 
-int encode_raw_tensor_map(CUtensorMap* map, const void* d_in, long long row_bytes, int T, int box_bytes,
-                          std::string* err) {
+int encode_raw_tensor_map(CUtensorMap* map, const void* d_in, long long row_bytes, int T, std::string* err) {
   encode_fn_t fn = encode_fn(err);
   if (!fn) return -1;
   const cuuint64_t dims[2] = {(cuuint64_t)row_bytes, (cuuint64_t)T};
   const cuuint64_t strides[1] = {(cuuint64_t)row_bytes};
-  const cuuint32_t box[2] = {(cuuint32_t)box_bytes, (cuuint32_t)KT};
+  const cuuint32_t box[2] = {128, (cuuint32_t)KT};
   const cuuint32_t estr[2] = {1, 1};
   const CUresult r = fn(map, CU_TENSOR_MAP_DATA_TYPE_UINT8, 2, const_cast<void*>(d_in), dims, strides, box, estr,
-                        CU_TENSOR_MAP_INTERLEAVE_NONE, box_bytes == 64 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B,
+                        CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
                         CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   if (r != CUDA_SUCCESS) {
     if (err) *err = "cuTensorMapEncodeTiled (samples) failed: " + std::to_string((int)r);

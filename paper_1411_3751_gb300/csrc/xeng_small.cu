@@ -381,12 +381,12 @@ int direct_splits(long long items, int slots, int n_k, int overhead) {
   return best;
 }
 
-cudaError_t direct_args(const DirectJob& j, int box_bytes, xd::Args* a) {
+cudaError_t direct_args(const DirectJob& j, xd::Args* a) {
   std::memset(a, 0, sizeof(*a));
   if (j.n > xd::MAX_BLOCKS) return cudaErrorInvalidValue;
   for (int b = 0; b < j.n; ++b) {
     std::string err;
-    if (encode_raw_tensor_map(&a->map[b], j.blocks[b], (long long)j.s.C * j.ld, j.T_blk, box_bytes, &err) != 0) {
+    if (encode_raw_tensor_map(&a->map[b], j.blocks[b], (long long)j.s.C * j.ld, j.T_blk, &err) != 0) {
       set_last_error(err);
       return cudaErrorInvalidValue;
     }
@@ -418,7 +418,7 @@ bool xeng_small_supported(const Shape& s, int ld, const void* d_in) {
 cudaError_t launch_xeng_small(const DirectJob& j, int num_sms, cudaStream_t st) {
   if (j.n == 0 || j.T_blk == 0) return cudaSuccess;
   xd::Args a;
-  cudaError_t e = direct_args(j, 128, &a);
+  cudaError_t e = direct_args(j, &a);
   if (e != cudaSuccess) return e;
   a.g = small_group(j.ld);
   a.ub = a.g * j.ld;
