@@ -168,8 +168,8 @@ __global__ void __launch_bounds__(256) f8_prep_kernel(const uint8_t* __restrict_
   prep_block<VEC>(in, N, C, T, T_run, T_stride, t_base, R, rows_per_split, op, s1, s2, blockIdx.x, blockIdx.z, part);
 }
 
-// Several arrays' builds in one launch (arrays of a group that leave the GPU partly idle alone): job i owns the linear
-// blocks [blk0_i, blk0_{i+1}), gx_i blocks of units by its time ranges, as its own launch would lay them out.
+// Several arrays' builds in one launch (a group's merged arrays): job i owns the linear blocks [blk0_i, blk0_{i+1}), gx_i
+// blocks of units by its time ranges, as its own launch would lay them out.
 struct PrepJob {
   const uint8_t* in;
   uint8_t* op;
