@@ -89,8 +89,8 @@ constexpr int PFB_ZLEN = PFB_H + PFB_H / 16;  // padded complex buffer per spect
 
 // Rows q < 8 of the split step's factors W^(u + 256 q), u <= 128, beside the buffers (the others are -i times these).
 // From the table, each rounded once: as products W^u W^(256 q) their error is 2.4 times as large (the spectrum's 1.44e-7
-// instead of 1.39e-7, relative, 4 taps). They come with cp.async while the FIR runs: at the size above 573 us, as products 588, loaded
-// where they are used 628, all 16 rows so 716.
+// instead of 1.39e-7, relative, 4 taps). They come with cp.async while the FIR runs: at the size above 573 us, as
+// products 588, loaded where they are used 628, all 16 rows so 716.
 constexpr int PFB_WLD = 130;  // row stride
 constexpr int PFB_SMEM = (PFB_SPB * PFB_ZLEN + 8 * PFB_WLD) * (int)sizeof(float2);
 
@@ -177,7 +177,8 @@ __global__ void __launch_bounds__(PFB_NT, 2) pfb_kernel(const int8_t* __restrict
   } else {
     // any tap count: four points at a time, four taps of each in flight. (A tap of all 16 points at a time was slower:
     // 512 inputs x 8 spectra, 16 taps 180 us, 155 so, and with few spectra, where each step's latency shows, slower than
-    // the shared-memory FIR that it replaced: 64 inputs x 1 spectrum, 16 taps 16.4 us, 14.5 that one, 14.4 so.)
+    // the shared-memory FIR that it replaced: 64 inputs x 1 spectrum, 16 taps 16.4 us, 14.5 that one, 14.4 so. Between
+    // one and three waves of blocks it was the faster one: 128 x 8, 9 taps 31 and 35 us, the shared-memory FIR 47.)
 #pragma unroll
     for (int r0 = 0; r0 < 16; r0 += 4) {
       int y[4][PFB_SPB][2] = {};
